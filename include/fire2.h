@@ -74,14 +74,15 @@ typedef enum {
 } fire_pot_kind;
 
 /* How the RGL pair functions phi(r), g(r) and their derivatives are
- * evaluated.  FIRE_PAIR_TABLE: piecewise quintic Hermite polynomials in
- * u = r^2 - r0^2 (knots every ~0.04 A^2, on rs and rc, matching value, first
- * and second derivative at every knot; interpolation error ~1e-13 relative
- * for values, ~1e-11 for derivatives), no square root or exponential per
- * pair; pairs closer than r0/2 use the analytic functions.  In the FP64
- * precision the table terms are computed from exact fixed-point separations
- * (2^-44 A) in double-float arithmetic (float pairs, ~2^-44 relative), with
- * FP64 sums, reductions and integration.
+ * evaluated.  FIRE_PAIR_TABLE: piecewise polynomials in r^2, no square root
+ * or exponential per pair; pairs closer than r0/2 use the analytic functions.
+ * In the FP64 precision: quartics on intervals of r0^2/326 or less (a power of
+ * two; the taper's third-derivative jumps at rs and rc on row boundaries;
+ * interpolation error ~1e-13 relative for values, ~1e-12 for derivatives,
+ * largest near r0/2), computed from exact fixed-point separations (2^-44 A)
+ * in double-float arithmetic (float pairs, ~2^-44 relative), with FP64 sums,
+ * reductions and integration.  In the FP32-pair precision: quintic Hermite
+ * polynomials with knots every ~0.12 A^2, on rs and rc.
  * FIRE_PAIR_ANALYTIC: the exponentials and the taper per pair, IEEE FP64 in
  * the FP64 precision. */
 typedef enum {

@@ -994,7 +994,6 @@ static bool fill_potc(fire_handle* h) {
     }
     c.rc2 = pot->rc * pot->rc;
     c.r0sq = pot->r0 * pot->r0;
-    c.r0sq_f = (float)c.r0sq;
     c.rc2_f = (float)c.rc2;
     c.A = pot->A;
     c.xi2 = pot->xi * pot->xi;
@@ -1038,26 +1037,29 @@ static bool fill_potc(fire_handle* h) {
 // to the device (allocating on the first call).
 static fire_status upload_tables(fire_handle* h) {
     const fire_potential_t& p = h->pot;
-    const RglTables T = build_rgl_tables(p.A, p.xi, p.p, p.q, p.r0, p.rs, p.rc, 0.04);
-    const RglTables T32 = build_rgl_tables(p.A, p.xi, p.p, p.q, p.r0, p.rs, p.rc, 0.12);
-    h->potc.tab = T.meta;
+    // the FP32 tables only where the FP32-pair passes read them
+    const bool t32 = p.precision == FIRE_PREC_FP32_PAIR && p.pair_eval == FIRE_PAIR_TABLE;
+    const RglTables T32 = t32 ? build_rgl_tables(p.A, p.xi, p.p, p.q, p.r0, p.rs, p.rc) : RglTables{};
     h->potc.tab32 = T32.meta;
     std::vector<float> ffd, fff;
-    build_ff_tables(T, p.r0, ffd, fff);
+    h->potc.ff = build_ff_tables(p.A, p.xi, p.p, p.q, p.r0, p.rs, p.rc, ffd, fff);
     const size_t nff = ffd.size();
     const size_t nd32 = T32.dens32.size(), nf32 = T32.force32.size();
     if (!h->tab_ffd) {
         CK(h, cudaMalloc(&h->tab_ffd, nff * sizeof(float)));
         CK(h, cudaMalloc(&h->tab_fff, nff * sizeof(float)));
-        CK(h, cudaMalloc(&h->tab_d32, nd32 * sizeof(float)));
-        CK(h, cudaMalloc(&h->tab_f32, nf32 * sizeof(float)));
+        if (t32) {
+            CK(h, cudaMalloc(&h->tab_d32, nd32 * sizeof(float)));
+            CK(h, cudaMalloc(&h->tab_f32, nf32 * sizeof(float)));
+        }
     }
     CK(h, cudaMemcpy(h->tab_ffd, ffd.data(), nff * sizeof(float), cudaMemcpyHostToDevice));
     CK(h, cudaMemcpy(h->tab_fff, fff.data(), nff * sizeof(float), cudaMemcpyHostToDevice));
-    CK(h, cudaMemcpy(h->tab_d32, T32.dens32.data(), nd32 * sizeof(float), cudaMemcpyHostToDevice));
-    CK(h, cudaMemcpy(h->tab_f32, T32.force32.data(), nf32 * sizeof(float), cudaMemcpyHostToDevice));
     h->b.tab_ffd = h->tab_ffd;
     h->b.tab_fff = h->tab_fff;
+    if (!t32) return FIRE_OK;
+    CK(h, cudaMemcpy(h->tab_d32, T32.dens32.data(), nd32 * sizeof(float), cudaMemcpyHostToDevice));
+    CK(h, cudaMemcpy(h->tab_f32, T32.force32.data(), nf32 * sizeof(float), cudaMemcpyHostToDevice));
     h->b.tab_d32 = h->tab_d32;
     h->b.tab_f32 = h->tab_f32;
     // FP32-pair tables sit in shared memory (one per kernel, grid-stride
@@ -1953,23 +1955,20 @@ fire_status fire_diag_rgl_table(const fire_potential_t* pot, int64_t n, const do
     if (!pot || n < 0 || (n > 0 && (!r || !out)) || pot->kind != FIRE_POT_RGL ||
         !(pot->rc > pot->rs && pot->rs > 0.0 && pot->r0 > 0.0 && pot->xi > 0.0))
         return FIRE_ERR_ARG;
-    const RglTables T = build_rgl_tables(pot->A, pot->xi, pot->p, pot->q, pot->r0, pot->rs,
-                                         pot->rc, 0.04);
     std::vector<float> ffd, fff;
-    build_ff_tables(T, pot->r0, ffd, fff);
-    const float r0sq_f = (float)(pot->r0 * pot->r0), rc2_f = (float)(pot->rc * pot->rc);
+    const FFTab T = build_ff_tables(pot->A, pot->xi, pot->p, pot->q, pot->r0, pot->rs, pot->rc, ffd,
+                                    fff);
+    const float rc2_f = (float)(pot->rc * pot->rc);
     for (int64_t i = 0; i < n; ++i) {
         double* o = out + 4 * i;
         // the FP64 kernels' arithmetic from r^2 on (r^2 as a float pair)
         const ffloat r2 = f64_to_ff(r[i] * r[i]);
-        const float* rd = ff_row(T.meta, ffd, r2.hi - r0sq_f);
-        const float* rf = ff_row(T.meta, fff, r2.hi - r0sq_f);
         if (!(r2.hi < rc2_f)) {
             o[0] = o[1] = o[2] = o[3] = 0.0;
-        } else if (rd) {
+        } else if (r2.hi >= T.r2_lo) {
             ffloat d[2], f[2];
-            ff_row_eval(rd, r2, d);
-            ff_row_eval(rf, r2, f);
+            ff_eval(ffd, T, r2, d);
+            ff_eval(fff, T, r2, f);
             o[0] = ff_to_f64(d[0]);                 // phi
             o[1] = ff_to_f64(d[1]);                 // g
             o[2] = 0.5 * r[i] * ff_to_f64(f[0]);    // phi' = r (2 phi'/r) / 2

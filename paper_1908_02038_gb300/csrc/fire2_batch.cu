@@ -218,9 +218,9 @@ __device__ __forceinline__ int b_build(const BArgs& a, const BInst& I, int lo, i
 }
 
 // Separation x_j - x_i - shift of list entry e in the FP64 table form: exact
-// in 2^-44 A fixed point, split into float pairs; returns r^2.
-__device__ __forceinline__ ffloat b_sep_ff(const BArgs& a, const BInst& I, const lvec4& qi,
-                                           uint32_t e, ffloat& dx, ffloat& dy, ffloat& dz) {
+// in 2^-44 A fixed point, split into float pairs.
+__device__ __forceinline__ ffvec b_sep_ff(const BArgs& a, const BInst& I, const lvec4& qi,
+                                          uint32_t e) {
     const int j = (int)(e & kIdxMask), code = (int)(e >> kIdxBits);
     const lvec4 qj = a.xq64[I.off + j];
     long long ix = qj.x - qi.x, iy = qj.y - qi.y, iz = qj.z - qi.z;
@@ -229,10 +229,7 @@ __device__ __forceinline__ ffloat b_sep_ff(const BArgs& a, const BInst& I, const
         iy -= (long long)((code / 5) % 5 - 2) * I.Lq64[1];
         iz -= (long long)(code / 25 - 2) * I.Lq64[2];
     }
-    dx = fixed_to_ff(ix);
-    dy = fixed_to_ff(iy);
-    dz = fixed_to_ff(iz);
-    return ff_norm2(dx, dy, dz);
+    return {fixed_to_ff2(ix, iy), fixed_to_ff(iz)};
 }
 
 // Energy and forces of atoms [lo, hi) of one system (full list, no
@@ -275,33 +272,28 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
             e_sum += erep.value() - (double)sq;
         } else if (a.ff) {   // FP64 table form: double-float pair terms, FP64 embedding
             const lvec4 qi = a.xq64[gi];
-            ffloat rho = {0.f, 0.f}, erep = {0.f, 0.f};
+            ffloat2 acc = {{0.f, 0.f}, {0.f, 0.f}};   // repulsive energy, density
             for (int k = 0; k < m; ++k) {
-                ffloat dx, dy, dz;
                 const ffloat r2 =
-                    b_sep_ff(a, I, qi, a.nbr[I.list_off + (long long)k * I.n + i], dx, dy, dz);
+                    ff_norm2(b_sep_ff(a, I, qi, a.nbr[I.list_off + (long long)k * I.n + i]));
                 if (!(r2.hi < P.rc2_f)) continue;
-                const float uf = r2.hi - P.r0sq_f;
-                if (uf >= P.tab.u_lo_f) {
-                    float row[kFFRow];
-                    load_row(a.tab_ffd, ff_index(P.tab, uf), row);
-                    ffloat v[2];
-                    ff_row_eval(row, r2, v);
-                    erep = ff_acc(erep, v[0]);
-                    rho = ff_acc(rho, v[1]);
+                ffloat2 w;
+                if (r2.hi >= P.ff.r2_lo) {
+                    w = ff_eval2(a.tab_ffd, P.ff, r2);
                 } else {   // compressed below the table: FP64 exponentials
                     double rinv, phi, dphi, g, dg;
                     rgl_pair64(P, ff_to_f64(r2), etab, rinv, phi, dphi, g, dg);
-                    erep = ff_acc(erep, f64_to_ff(phi));
-                    rho = ff_acc(rho, f64_to_ff(g));
+                    const ffloat p = f64_to_ff(phi), q = f64_to_ff(g);
+                    w = {make_float2(p.hi, q.hi), make_float2(p.lo, q.lo)};
                 }
+                acc = ff_acc2(acc, w);
             }
             double sq, fp;
             ffloat fpf;
-            rgl_embed_dd(ff_to_f64(rho), sq, fp, fpf);
+            rgl_embed_dd(ff_to_f64(ff_second(acc)), sq, fp, fpf);
             a.fp64[gi] = fp;
             a.fpff[gi] = make_float2(fpf.hi, fpf.lo);
-            e_sum += ff_to_f64(erep) - sq;
+            e_sum += ff_to_f64(ff_first(acc)) - sq;
         } else {
             const dvec4 xi = a.x[gi];
             double rho = 0.0, erep = 0.0;
@@ -362,31 +354,32 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
             const lvec4 qi = a.xq64[gi];
             const float2 fpi2 = a.fpff[gi];
             const ffloat fpi = {fpi2.x, fpi2.y};
-            ffloat fx = {0.f, 0.f}, fy = {0.f, 0.f}, fz = {0.f, 0.f};
+            ffloat2 fxy = {{0.f, 0.f}, {0.f, 0.f}};
+            ffloat fz = {0.f, 0.f};
             for (int k = 0; k < m; ++k) {
                 const uint32_t e = a.nbr[I.list_off + (long long)k * I.n + i];
-                ffloat dx, dy, dz;
-                const ffloat r2 = b_sep_ff(a, I, qi, e, dx, dy, dz);
+                const ffvec d = b_sep_ff(a, I, qi, e);
+                const ffloat r2 = ff_norm2(d);
                 if (!(r2.hi < P.rc2_f)) continue;
-                const float uf = r2.hi - P.r0sq_f;
-                ffloat c[2];
-                if (uf >= P.tab.u_lo_f) {
-                    float row[kFFRow];
-                    load_row(a.tab_fff, ff_index(P.tab, uf), row);
-                    ff_row_eval(row, r2, c);
+                ffloat c0, c1;
+                if (r2.hi >= P.ff.r2_lo) {
+                    const ffloat2 c = ff_eval2(a.tab_fff, P.ff, r2);
+                    c0 = ff_first(c);
+                    c1 = ff_second(c);
                 } else {
                     double rinv, phi, dphi, g, dg;
                     rgl_pair64(P, ff_to_f64(r2), etab, rinv, phi, dphi, g, dg);
-                    c[0] = f64_to_ff(2.0 * dphi * rinv);
-                    c[1] = f64_to_ff(dg * rinv);
+                    c0 = f64_to_ff(2.0 * dphi * rinv);
+                    c1 = f64_to_ff(dg * rinv);
                 }
                 const float2 fpj2 = a.fpff[I.off + (int)(e & kIdxMask)];
-                const ffloat fs = ff_madd(ff_add(fpi, {fpj2.x, fpj2.y}), c[1], c[0]);
-                fx = ff_acc(fx, ff_mul_nn(fs, dx));
-                fy = ff_acc(fy, ff_mul_nn(fs, dy));
-                fz = ff_acc(fz, ff_mul_nn(fs, dz));
+                const ffloat fs = ff_madd(ff_add(fpi, {fpj2.x, fpj2.y}), c1, c0);
+                const ffloat2 t = ff_mul2_neg(fs, d.xy);
+                fxy = ff_acc2_neg(fxy, t.hi, t.lo);
+                fz = ff_acc(fz, ff_mul_nn(fs, d.z));
             }
-            a.f[gi] = make_dvec4(ff_to_f64(fx), ff_to_f64(fy), ff_to_f64(fz), 0.0);
+            a.f[gi] = make_dvec4(ff_to_f64(ff_first(fxy)), ff_to_f64(ff_second(fxy)), ff_to_f64(fz),
+                                 0.0);
         } else {
             const dvec4 xi = a.x[gi];
             const double fpi = a.fp64[gi];

@@ -37,7 +37,7 @@ enum { STOP_FTOL = 0, STOP_MAXITER = 1, STOP_MAXVDOTF = 2 };
 enum { POT_LJ = 0, POT_RGL = 1 };
 enum { CTL_INITIAL = 0, CTL_LOOP = 1, CTL_EVAL = 2 };
 
-// Knots of the tabulated RGL pair functions (built in fire2_table.cuh):
+// Knots of the FP32 tables of the RGL pair functions (built in fire2_table.cuh):
 // region A covers [u_lo, u_rs] with spacing 1/hA_inv and a knot at u = 0,
 // region B covers [u_rs, rc^2 - r0^2] with spacing 1/hB_inv.
 struct TabMeta {
@@ -47,6 +47,13 @@ struct TabMeta {
     int pad;
     double hA_inv, hB_inv, u_lo, u_rs;
     float hA_inv_f, hB_inv_f, u_lo_f, u_rs_f;
+};
+
+// Intervals of the FP64 form's pair tables (fire2_table.cuh): width h in r^2,
+// from row 0 = [j_lo h, (j_lo + 1) h); rs2 = rs^2, r2_lo = j_lo h.
+struct FFTab {
+    float h, hinv, r2_lo, rs2;
+    int j_lo, last;
 };
 
 // Potential constants, passed by value.
@@ -68,8 +75,8 @@ struct PotC {
     float qinv, qinv2;        // 1 / qscale, 1 / qscale^2
     double xi_inv;            // 1 / xi (theta-derivatives)
     double r0sq;              // r0^2 (table variable u = r^2 - r0^2)
-    float r0sq_f, rc2_f;      // FP32 copies (table index and cut-off test of the FP64 pass)
-    TabMeta tab;              // knots of the tabulated pair functions (FP64)
+    float rc2_f;              // FP32 copy (cut-off test of the FP64 pass)
+    FFTab ff;                 // intervals of the FP64 form's tables
     TabMeta tab32;            // knots of the FP32 tables
 };
 

@@ -1014,11 +1014,9 @@ __device__ __forceinline__ void fill_qshift64_table(long long* qt, const GeoC& g
 }
 
 // Separation x_j - x_i - shift of list slot e (atom j at fixed-point position
-// qj) as float pairs (exact), and r^2.
-__device__ __forceinline__ ffloat pair_sep_ff_q(const long long* qt, const lvec4& qi,
-                                                const lvec4& qj, uint32_t e, ffloat& dx,
-                                                ffloat& dy, ffloat& dz, int& j) {
-    j = (int)(e & kIdxMask);
+// qj) as float pairs (exact).
+__device__ __forceinline__ ffvec pair_sep_ff(const long long* qt, const lvec4& qi,
+                                             const lvec4& qj, uint32_t e) {
     const int code = (int)(e >> kIdxBits);
     long long ix = qj.x - qi.x, iy = qj.y - qi.y, iz = qj.z - qi.z;
     if (code != kCodeZero) {
@@ -1026,17 +1024,7 @@ __device__ __forceinline__ ffloat pair_sep_ff_q(const long long* qt, const lvec4
         iy -= qt[3 * code + 1];
         iz -= qt[3 * code + 2];
     }
-    dx = fixed_to_ff(ix);
-    dy = fixed_to_ff(iy);
-    dz = fixed_to_ff(iz);
-    return ff_norm2(dx, dy, dz);
-}
-
-// The same, loading atom j's position.
-__device__ __forceinline__ ffloat pair_sep_ff(const Bufs& b, const long long* qt, const lvec4& qi,
-                                              uint32_t e, ffloat& dx, ffloat& dy, ffloat& dz,
-                                              int& j) {
-    return pair_sep_ff_q(qt, qi, b.xq64[e & kIdxMask], e, dx, dy, dz, j);
+    return {fixed_to_ff2(ix, iy), fixed_to_ff(iz)};
 }
 
 // Pass 1.  Full list (HALF = false): rho_i, F'(rho_i) (FP64 per atom) and the
@@ -1062,31 +1050,27 @@ __device__ __forceinline__ void density_ff_body(const Bufs& b, const PotC& P, co
     if (i < b.n) {
         const lvec4 qi = b.xq64[i];
         const int m = b.nnbr[i];
-        ffloat rho = {0.f, 0.f}, erep = {0.f, 0.f};
+        ffloat2 acc = {{0.f, 0.f}, {0.f, 0.f}};   // repulsive energy, density
         for (int k = lane; k < m; k += TPA) {
-            ffloat dx, dy, dz;
-            int j;
-            const ffloat r2 = pair_sep_ff(b, qt, qi, b.nbr[(size_t)k * b.n + i], dx, dy, dz, j);
+            const uint32_t e = b.nbr[(size_t)k * b.n + i];
+            const int j = (int)(e & kIdxMask);
+            const ffloat r2 = ff_norm2(pair_sep_ff(qt, qi, b.xq64[j], e));
             if (!(r2.hi < P.rc2_f)) continue;
-            const float uf = r2.hi - P.r0sq_f;
-            if (uf >= P.tab.u_lo_f) {
-                float row[kFFRow];
-                load_row(b.tab_ffd, ff_index(P.tab, uf), row);
-                ffloat v[2];
-                ff_row_eval(row, r2, v);
-                erep = ff_acc(erep, v[0]);   // doubled at the end on the half list
-                rho = ff_acc(rho, v[1]);
-                if (HALF) atomicAdd(&b.rho[j], ff_to_f64(v[1]));
+            ffloat2 v;   // phi (doubled at the end on the half list), g
+            if (r2.hi >= P.ff.r2_lo) {
+                v = ff_eval2(b.tab_ffd, P.ff, r2);
+                if (HALF) atomicAdd(&b.rho[j], ff_to_f64(ff_second(v)));
             } else {
                 double rinv, phi, dphi, gg, dg;
                 rgl_pair64(P, ff_to_f64(r2), etab, rinv, phi, dphi, gg, dg);
-                erep = ff_acc(erep, f64_to_ff(phi));
-                rho = ff_acc(rho, f64_to_ff(gg));
+                const ffloat p = f64_to_ff(phi), q = f64_to_ff(gg);
+                v = {make_float2(p.hi, q.hi), make_float2(p.lo, q.lo)};
                 if (HALF) atomicAdd(&b.rho[j], gg);
             }
+            acc = ff_acc2(acc, v);
         }
-        const double rho_d = group_sum<TPA>(ff_to_f64(rho));
-        const double erep_d = group_sum<TPA>(ff_to_f64(erep));
+        const double rho_d = group_sum<TPA>(ff_to_f64(ff_second(acc)));
+        const double erep_d = group_sum<TPA>(ff_to_f64(ff_first(acc)));
         if (lane == 0 && HALF) {
             atomicAdd(&b.rho[i], rho_d);
             e_atom = 2.0 * erep_d;   // each pair's 2 phi credited to i
@@ -1137,7 +1121,8 @@ __global__ void __launch_bounds__(BLK) k_force_ff(Bufs b, PotC P, GeoC g) {
     const lvec4 qi = b.xq64[i];
     const ffloat fpi = fp_load(qi);
     const int m = b.nnbr[i];
-    ffloat fx = {0.f, 0.f}, fy = {0.f, 0.f}, fz = {0.f, 0.f};
+    ffloat2 fxy = {{0.f, 0.f}, {0.f, 0.f}};
+    ffloat fz = {0.f, 0.f};
     // software pipeline: the next list entry and its atom's record (position
     // and F') load while this pair is evaluated
     uint32_t e_nx = lane < m ? b.nbr[(size_t)lane * b.n + i] : 0u;
@@ -1149,34 +1134,33 @@ __global__ void __launch_bounds__(BLK) k_force_ff(Bufs b, PotC P, GeoC g) {
             e_nx = b.nbr[(size_t)(k + TPA) * b.n + i];
             q_nx = b.xq64[e_nx & kIdxMask];
         }
-        ffloat dx, dy, dz;
-        int j;
-        const ffloat r2 = pair_sep_ff_q(qt, qi, qj, e, dx, dy, dz, j);
+        const ffvec d = pair_sep_ff(qt, qi, qj, e);
+        const ffloat r2 = ff_norm2(d);
         if (!(r2.hi < P.rc2_f)) continue;
-        const float uf = r2.hi - P.r0sq_f;
-        ffloat c[2];
-        if (uf >= P.tab.u_lo_f) {
-            float row[kFFRow];
-            load_row(b.tab_fff, ff_index(P.tab, uf), row);
-            ff_row_eval(row, r2, c);
+        ffloat c0, c1;
+        if (r2.hi >= P.ff.r2_lo) {
+            const ffloat2 c = ff_eval2(b.tab_fff, P.ff, r2);
+            c0 = ff_first(c);
+            c1 = ff_second(c);
         } else {
             double rinv, phi, dphi, gg, dg;
             rgl_pair64(P, ff_to_f64(r2), etab, rinv, phi, dphi, gg, dg);
-            c[0] = f64_to_ff(2.0 * dphi * rinv);
-            c[1] = f64_to_ff(dg * rinv);
+            c0 = f64_to_ff(2.0 * dphi * rinv);
+            c1 = f64_to_ff(dg * rinv);
         }
-        const ffloat fs = ff_madd(ff_add(fpi, fp_load(qj)), c[1], c[0]);
-        // unnormalised products: ff_acc and ff_to_f64 take any pair
-        const ffloat tx = ff_mul_nn(fs, dx), ty = ff_mul_nn(fs, dy), tz = ff_mul_nn(fs, dz);
-        fx = ff_acc(fx, tx);
-        fy = ff_acc(fy, ty);
+        const ffloat fs = ff_madd(ff_add(fpi, fp_load(qj)), c1, c0);
+        // unnormalised products (x and y with the high part negated): the
+        // sums and ff_to_f64 take any pair
+        const ffloat2 t = ff_mul2_neg(fs, d.xy);
+        const ffloat tz = ff_mul_nn(fs, d.z);
+        fxy = ff_acc2_neg(fxy, t.hi, t.lo);
         fz = ff_acc(fz, tz);
-        if (HALF) {
-            f_add(b, j, -ff_to_f64(tx), -ff_to_f64(ty), -ff_to_f64(tz));
-        }
+        if (HALF)
+            f_add(b, (int)(e & kIdxMask), f32_to_f64(t.hi.x) - f32_to_f64(t.lo.x),
+                  f32_to_f64(t.hi.y) - f32_to_f64(t.lo.y), -ff_to_f64(tz));
     }
-    const double sx = group_sum<TPA>(ff_to_f64(fx));
-    const double sy = group_sum<TPA>(ff_to_f64(fy));
+    const double sx = group_sum<TPA>(ff_to_f64(ff_first(fxy)));
+    const double sy = group_sum<TPA>(ff_to_f64(ff_second(fxy)));
     const double sz = group_sum<TPA>(ff_to_f64(fz));
     if (lane != 0) return;
     if (HALF) {   // k_reduce_ctl applies the frozen-DOF mask

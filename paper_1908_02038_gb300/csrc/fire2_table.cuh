@@ -1,29 +1,28 @@
 // Tabulated RGL pair functions.
 //
 // The two exponentials, the square root and the taper of every pair are
-// replaced by piecewise quintic Hermite polynomials in u = r^2 - r0^2:
-//   density table: phi(u), g(u)               (6 coefficients each)
-//   force table:   phi_u(u), g_u(u) = d/du    (6 coefficients each)
+// replaced by piecewise polynomials in r^2:
+//   density table: phi, g            force table: phi_u, g_u = d/d(r^2)
 // with phi = A e^{-p(r/r0-1)} S(r) and g = xi^2 e^{-2q(r/r0-1)} S(r).  Since
 // (dE/dr)/r = 2 dE/du, the force pass needs neither r nor 1/r.
 //
-// Knots: region A covers [u_lo, u_rs] with spacing hA, and u = 0 and
-// u_rs = rs^2 - r0^2 are knots; region B covers the taper [u_rs, u_rc] with
-// spacing hB (u_rc = rc^2 - r0^2 a knot), so the jumps of S''' at rs and rc
-// fall on knots.  u_lo = -0.75 r0^2 (r = r0/2); closer pairs fall back to the
+// FP32 tables (the FP32-pair form, in shared memory): quintic Hermite
+// polynomials in u = r^2 - r0^2, 0.12 A^2 apart.  Region A covers [u_lo, u_rs],
+// and u = 0 and u_rs = rs^2 - r0^2 are knots; region B covers the taper
+// [u_rs, u_rc] (u_rc = rc^2 - r0^2 a knot), so the jumps of S''' at rs and rc
+// fall on knots.  Index arithmetic: region A uses x = u / hA (so pairs near
+// r0, where the forces are stiffest, keep the full precision of u even in
+// FP32), region B x = (u - u_rs) / hB.
+//
+// FP64 form (build_ff_tables below): intervals of a power of two, about
+// r0^2 / 420, in r^2 itself.
+//
+// In both u_lo = -0.75 r0^2 (r = r0/2); closer pairs fall back to the
 // analytic functions.  Each interval's quintic matches the function and its
 // first two u-derivatives at both ends: for the density table f, f_u, f_uu
 // and for the force table f_u, f_uu, f_uuu, with (primes = d/dr)
 //   f_u = f'/(2r),  f_uu = (f'' - f'/r)/(4 r^2),
 //   f_uuu = (f''' - 3 f''/r + 3 f'/r^2)/(8 r^3).
-// With spacings near 0.04 A^2 (FP64 tables) the interpolation error is
-// ~1e-11 relative or better on the Cu parameters (largest for pairs
-// compressed towards r0/2, ~1e-12 above 0.8 r0); the FP32 tables use
-// 0.12 A^2, still far below float rounding.
-//
-// Index arithmetic: region A uses x = u / hA (so pairs near r0, where the
-// forces are stiffest, keep the full precision of u even in FP32), region B
-// x = (u - u_rs) / hB.
 #pragma once
 
 #include <cmath>
@@ -39,25 +38,25 @@ constexpr int kTabForce = 12;   // coefficients per interval, force table
 
 struct RglTables {
     TabMeta meta;
-    std::vector<double> dens64, force64;
     std::vector<float> dens32, force32;
 };
 
 // Analytic phi, g and their first three r-derivatives (host):
 // out = (phi, phi', phi'', phi''', g, g', g'', g''').  taper < 0: decide from
 // r; taper = 0: S = 1 (inside region A); taper = 1: the taper polynomial
-// with t clamped to [0, 1] (inside region B) -- the table builder passes the
-// region so that the one-sided limits at rs and rc are used (S''' jumps there).
+// with t clamped to [0, 1] (inside region B); taper = 3: the polynomial as it
+// is, also outside [rs, rc] -- the table builders pass the region so that the
+// one-sided limits at rs and rc are used (S''' jumps there).
 inline void rgl_analytic(double A, double xi, double p, double q, double r0, double rs,
                          double rc, double r, double out[8], int taper = -1) {
     double S = 1.0, dS = 0.0, d2S = 0.0, d3S = 0.0;
     if (taper < 0) taper = (r >= rc) ? 2 : (r > rs ? 1 : 0);
     if (taper == 2) {
         S = 0.0;
-    } else if (taper == 1) {
+    } else if (taper == 1 || taper == 3) {
         const double w = rc - rs;
         double t = (r - rs) / w;
-        t = t < 0.0 ? 0.0 : (t > 1.0 ? 1.0 : t);
+        if (taper == 1) t = t < 0.0 ? 0.0 : (t > 1.0 ? 1.0 : t);
         S = 1.0 - 10.0 * t * t * t + 15.0 * t * t * t * t - 6.0 * t * t * t * t * t;
         dS = (-30.0 * t * t + 60.0 * t * t * t - 30.0 * t * t * t * t) / w;
         d2S = (-60.0 * t + 180.0 * t * t - 120.0 * t * t * t) / (w * w);
@@ -88,9 +87,23 @@ inline void quintic_hermite(double F0, double D0, double S0, double F1, double D
     c[5] = 6.0 * dF - 3.0 * D0 - 3.0 * D1 - 0.5 * S0 + 0.5 * S1;
 }
 
-// target: knot spacing in A^2 (0.04 for the FP64 tables, 0.12 for FP32).
+// f, f_u, f_uu, f_uuu (u = r^2 - r0^2) at r for phi (k = 0) and g (k = 1)
+inline void rgl_derivs_u(double A, double xi, double p, double q, double r0, double rs, double rc,
+                         double r, int taper, double f[2][4]) {
+    double a[8];
+    rgl_analytic(A, xi, p, q, r0, rs, rc, r, a, taper);
+    for (int k = 0; k < 2; ++k) {
+        const double f0 = a[4 * k], f1 = a[4 * k + 1], f2 = a[4 * k + 2], f3 = a[4 * k + 3];
+        f[k][0] = f0;
+        f[k][1] = f1 / (2.0 * r);
+        f[k][2] = (f2 - f1 / r) / (4.0 * r * r);
+        f[k][3] = (f3 - 3.0 * f2 / r + 3.0 * f1 / (r * r)) / (8.0 * r * r * r);
+    }
+}
+
+// The FP32 tables; target: knot spacing in A^2.
 inline RglTables build_rgl_tables(double A, double xi, double p, double q, double r0, double rs,
-                                  double rc, double target = 0.04) {
+                                  double rc, double target = 0.12) {
     RglTables T;
     const double r02 = r0 * r0;
     const double u_rs = rs * rs - r02, u_rc = rc * rc - r02, u_min = -0.75 * r02;
@@ -112,21 +125,8 @@ inline RglTables build_rgl_tables(double A, double xi, double p, double q, doubl
     m.u_lo_f = (float)m.u_lo;
     m.u_rs_f = (float)u_rs;
     const int nint = m.nA + m.nB;
-    T.dens64.resize((size_t)nint * kTabDens);
-    T.force64.resize((size_t)nint * kTabForce);
-    // f, f_u, f_uu, f_uuu in u for phi (k = 0) and g (k = 1)
-    auto derivs_u = [&](double u, int taper, double f[2][4]) {
-        const double r = std::sqrt(r02 + u);
-        double a[8];
-        rgl_analytic(A, xi, p, q, r0, rs, rc, r, a, taper);
-        for (int k = 0; k < 2; ++k) {
-            const double f0 = a[4 * k], f1 = a[4 * k + 1], f2 = a[4 * k + 2], f3 = a[4 * k + 3];
-            f[k][0] = f0;
-            f[k][1] = f1 / (2.0 * r);
-            f[k][2] = (f2 - f1 / r) / (4.0 * r * r);
-            f[k][3] = (f3 - 3.0 * f2 / r + 3.0 * f1 / (r * r)) / (8.0 * r * r * r);
-        }
-    };
+    T.dens32.resize((size_t)nint * kTabDens);
+    T.force32.resize((size_t)nint * kTabForce);
     for (int i = 0; i < nint; ++i) {
         double ua, h;
         if (i < m.nA) {
@@ -139,55 +139,23 @@ inline RglTables build_rgl_tables(double A, double xi, double p, double q, doubl
         const double ub = (i == m.nA - 1) ? u_rs : ((i == nint - 1) ? u_rc : ua + h);
         double fa[2][4], fb[2][4];
         const int taper = i < m.nA ? 0 : 1;
-        derivs_u(ua, taper, fa);
-        derivs_u(ub, taper, fb);
+        rgl_derivs_u(A, xi, p, q, r0, rs, rc, std::sqrt(r02 + ua), taper, fa);
+        rgl_derivs_u(A, xi, p, q, r0, rs, rc, std::sqrt(r02 + ub), taper, fb);
         for (int k = 0; k < 2; ++k) {
             double c[6];
             quintic_hermite(fa[k][0], h * fa[k][1], h * h * fa[k][2], fb[k][0], h * fb[k][1],
                             h * h * fb[k][2], c);
-            for (int j = 0; j < 6; ++j) T.dens64[(size_t)i * kTabDens + 6 * k + j] = c[j];
+            for (int j = 0; j < 6; ++j) T.dens32[(size_t)i * kTabDens + 6 * k + j] = (float)c[j];
             quintic_hermite(fa[k][1], h * fa[k][2], h * h * fa[k][3], fb[k][1], h * fb[k][2],
                             h * h * fb[k][3], c);
-            for (int j = 0; j < 6; ++j) T.force64[(size_t)i * kTabForce + 6 * k + j] = c[j];
+            for (int j = 0; j < 6; ++j) T.force32[(size_t)i * kTabForce + 6 * k + j] = (float)c[j];
         }
     }
-    T.dens32.assign(T.dens64.begin(), T.dens64.end());
-    T.force32.assign(T.force64.begin(), T.force64.end());
     return T;
 }
 
 // Interval index and local coordinate t in [0, 1]; false outside the table
 // (u < u_lo; u >= u_rc never reaches here because of the cut-off test).
-__host__ __device__ __forceinline__ bool tab_locate(const TabMeta& m, double u, int& k, double& t) {
-    if (u < m.u_lo) return false;
-    double x;
-    if (u < m.u_rs) {
-        x = u * m.hA_inv;
-        const double fl = floor(x);
-        k = (int)fl + m.nA0;
-        t = x - fl;
-        if (k >= m.nA) {   // rounding at u_rs
-            k = m.nA - 1;
-            t = 1.0;
-        }
-    } else {
-        x = (u - m.u_rs) * m.hB_inv;
-        const double fl = floor(x);
-        k = (int)fl;
-        t = x - fl;
-        if (k >= m.nB) {
-            k = m.nB - 1;
-            t = 1.0;
-        }
-        k += m.nA;
-    }
-    if (k < 0) {
-        k = 0;
-        t = 0.0;
-    }
-    return true;
-}
-
 __device__ __forceinline__ bool tab_locate_f(const TabMeta& m, float u, int& k, float& t) {
     if (u < m.u_lo_f) return false;
     if (u < m.u_rs_f) {
@@ -221,11 +189,6 @@ template <typename T>
 __host__ __device__ __forceinline__ T poly5(const T* c, T t) {
     return ((((c[5] * t + c[4]) * t + c[3]) * t + c[2]) * t + c[1]) * t + c[0];
 }
-template <typename T>
-__host__ __device__ __forceinline__ T poly4(const T* c, T t) {
-    return (((c[4] * t + c[3]) * t + c[2]) * t + c[1]) * t + c[0];
-}
-
 }  // namespace fire2
 
 namespace fire2 {
@@ -241,25 +204,40 @@ namespace fire2 {
 //   * everything else is double-float arithmetic: each value is an
 //     unevaluated sum hi + lo of two floats (Dekker 1971; Knuth's TwoSum),
 //     good to ~2^-44 relative, in FP32 instructions only:
-//       r^2 = dx^2 + dy^2 + dz^2,  s = r^2 - (u_k + r0^2),
-//       f = c0 + s (c1 + s (c2 + s q)),   q = c3 + s (c4 + s c5)
-//     with c0..c2 and s as float pairs and q in plain FP32: on these tables
-//     |s c_{j+1} / c_j| < ~0.07, so s^3 q is < ~1e-4 of f and its FP32
-//     rounding enters at ~1e-11 relative or less;
+//       r^2 = dx^2 + dy^2 + dz^2,  s = r^2 - (middle of its interval),
+//       f = c0 + s (c1 + s (c2 + s q)),   q = c3 + s c4
+//     with c0..c2 and s as float pairs, q in plain FP32 and the product s q
+//     added to c2's low part: an interval spans ~r0^2 / 420, so that
+//     |s c_{j+1} / c_j| is below ~0.01 / (j + 1) on the Cu parameters, s q is
+//     below 2^-8 of c2 and its rounding 2^-32 of c2, ~2^-48 of f;
 //   * the cut-off test and the interval index use the FP32 high part of r^2:
 //     the taper makes phi, g and their first two derivatives vanish at rc,
 //     so a pair within FP32 rounding of rc contributes nothing either way,
-//     and an index one off at an interval edge only moves s by ~1e-6 of the
-//     interval outside [0, h], where the quintic is still accurate.
+//     and at rs the two rows of an interval agree to the second derivative.
 // Float/double crossings (per atom only) are integer operations on the
 // IEEE-754 fields.
 //
-// Rows (kFFRow floats = 80 bytes, 16-byte aligned): [0], [1] u_k + r0^2 as
-// hi, lo; then two polynomials of 9 floats each: c0 hi, c0 lo, c1 hi, c1 lo,
-// c2 hi, c2 lo, c3, c4, c5 (coefficients in s, i.e. divided by h^j).
-// Density rows: phi, g.  Force rows: 4 phi_u = 2 phi'/r, 2 g_u = g'/r.
+// Intervals: [j h, (j + 1) h) in r^2 with h a power of two, so that the index
+// is one FMA rounded down and the interval's middle is exact in FP32 (nothing
+// of it is stored).  The interval that contains rs^2 has two rows, one for
+// either side, each built from its side's function continued over the whole
+// interval.  Rows (kFFRow floats): the eight numbers c0 hi, c0 lo, c1 hi,
+// c1 lo, c2 hi, c2 lo, c3, c4 (coefficients in s) of two polynomials, side by
+// side: number j of polynomial p is float 2 j + p, so that a 16-byte load
+// brings register pairs for the packed FP32 instructions (ff_eval2).  The
+// four 16-byte pieces of the rows lie in four arrays (piece q of row k at
+// float4 q * rows + k).  Density rows: phi, g.  Force rows: 4 phi_u =
+// 2 phi'/r, 2 g_u = g'/r.
+//
+// The passes gather a row per pair through L1, whose eight 16-byte banks
+// decide the time: 1M-atom box, density / force pass 349 / 452 us with whole
+// 64-byte rows (two banks serve the first piece of every row), 277 / 376 us
+// with the rows 80 bytes apart, 270 / 369 us with the pieces in arrays of
+// their own (any eight neighbouring rows in eight banks, and fewer lines).
+// Rows of 20 floats (degree 5, intervals of 0.04 A^2, the knot stored) took
+// 288 / 385 us and were 10 times less accurate.
 
-constexpr int kFFRow = 20;
+constexpr int kFFRow = 16;
 constexpr int kFixedBits64 = 44;   // fixed-point positions of the FP64 form: 2^44 per A
 
 
@@ -457,50 +435,112 @@ __device__ __forceinline__ void rgl_embed_dd(double rho, double& sq, double& fp,
     }
 }
 
-// One quintic of a row: c = 9 floats (see the layout above), s as a float pair.
-// Horner steps c_k + s r as fused double-float multiply-adds.
+// One polynomial of a row: c = its 8 numbers at stride 2 (see the layout
+// above), s as a float pair.
 __host__ __device__ __forceinline__ ffloat ff_poly(const float* c, ffloat s) {
-    const float q = fmaf(fmaf(c[8], s.hi, c[7]), s.hi, c[6]);
-    ffloat r = ff_madd_f(s, q, {c[4], c[5]});
-    r = ff_madd(s, r, {c[2], c[3]});
-    return ff_madd(s, r, {c[0], c[1]});
+    const float q = fmaf(c[14], s.hi, c[12]);
+    ffloat r = {c[8], fmaf(s.hi, q, c[10])};
+    r = ff_madd(s, r, {c[4], c[6]});
+    return ff_madd(s, r, {c[0], c[2]});
 }
 
-__host__ __device__ __forceinline__ ffloat ff_neg(ffloat a) { return {-a.hi, -a.lo}; }
-
-// Interval of u (from its FP32 copy uf), clamped to the table.
-__host__ __device__ __forceinline__ int ff_index(const TabMeta& m, float uf) {
-    int k = uf < m.u_rs_f ? m.nA0 + (int)floorf(uf * m.hA_inv_f)
-                          : m.nA + (int)floorf((uf - m.u_rs_f) * m.hB_inv_f);
-    const int last = m.nA + m.nB - 1;
-    return k < 0 ? 0 : (k > last ? last : k);
+// Row of r^2 (its FP32 high part, at least t.r2_lo) and the middle of its
+// interval.  r2 >= rs2 implies j >= floor(rs^2 / h), whose multiple of h is an
+// FP32 number that rs^2 cannot round below; the last row is a bound only.
+__host__ __device__ __forceinline__ int ff_row_of(const FFTab& t, float r2, float& mid) {
+#ifdef __CUDA_ARCH__
+    const float x = __fmaf_rd(r2, t.hinv, 0x1p23f);   // floor(r2 / h) + 2^23
+    const int j = __float_as_int(x) - 0x4B000000;
+    mid = fmaf(x - 0x1p23f, t.h, 0.5f * t.h);
+#else
+    const int j = (int)floorf(r2 * t.hinv);
+    mid = (j + 0.5f) * t.h;
+#endif
+    const int k = j - t.j_lo + (r2 >= t.rs2 ? 1 : 0);
+    return k > t.last ? t.last : k;
 }
 
-// Row k of a table in global memory (80 bytes, 16-byte aligned), through L1.
-__device__ __forceinline__ void load_row(const float* tab, int k, float row[kFFRow]) {
-    const float4* src = reinterpret_cast<const float4*>(tab + (size_t)k * kFFRow);
+#ifdef __CUDACC__
+// ---------------------------------------------------------------------------
+// Two double-floats side by side on the packed FP32 instructions (f32x2: one
+// instruction, two independent FP32 operations, each rounded like its scalar
+// form).  The pair passes are bound by instruction issue (71-73 % issue slots
+// busy with the FP32 pipe at 42-47 %), and most of what they issue comes in
+// independent pairs: the two polynomials of a table row, the x and y
+// components of a separation, of a pair force and of its sum.  The results
+// are those of the scalar functions bit for bit.  1M-atom box, with the rows of
+// 20 floats: force pass 406 -> 385 us, density pass 281 -> 288 us (its
+// gathers, see above, were the bound).
+struct ffloat2 {
+    float2 hi, lo;
+};
+__device__ __forceinline__ float2 f2_both(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 f2_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 f2_sub(float2 a, float2 b) {   // a - b, rounded once
+    return __ffma2_rn(b, f2_both(-1.f), a);
+}
+__device__ __forceinline__ float2 f2_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+__device__ __forceinline__ ffloat2 fast_two_sum2(float2 a, float2 b) {
+    const float2 s = f2_add(a, b);
+    return {s, f2_sub(b, f2_sub(s, a))};
+}
+__device__ __forceinline__ ffloat2 two_sum2(float2 a, float2 b) {
+    const float2 s = f2_add(a, b), bb = f2_sub(s, a);
+    return {s, f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb))};
+}
+// two_sum of a and -nb (products arrive negated, which their error terms
+// fma(x, y, -xy) need)
+__device__ __forceinline__ ffloat2 two_diff2(float2 a, float2 nb) {
+    const float2 s = f2_sub(a, nb), bb = f2_sub(s, a);
+    return {s, f2_sub(f2_sub(a, f2_sub(s, bb)), f2_add(nb, bb))};
+}
+// ff_acc on two running sums; the second form takes the term's high part negated
+__device__ __forceinline__ ffloat2 ff_acc2(ffloat2 acc, ffloat2 t) {
+    const ffloat2 s = two_sum2(acc.hi, t.hi);
+    return {s.hi, f2_add(acc.lo, f2_add(s.lo, t.lo))};
+}
+__device__ __forceinline__ ffloat2 ff_acc2_neg(ffloat2 acc, float2 nhi, float2 lo) {
+    const ffloat2 s = two_diff2(acc.hi, nhi);
+    return {s.hi, f2_add(acc.lo, f2_add(s.lo, lo))};
+}
+// A double-float times the two of b, unnormalised (ff_mul_nn); the high part
+// is returned negated.
+__device__ __forceinline__ ffloat2 ff_mul2_neg(ffloat a, ffloat2 b) {
+    const float2 h = f2_both(a.hi), np = f2_mul(f2_both(-a.hi), b.hi);
+    return {np, f2_fma(h, b.lo, f2_fma(f2_both(a.lo), b.hi, f2_fma(h, b.hi, np)))};
+}
+
+// The two polynomials of a table (in global memory, rows through L1) at r^2.
+__device__ __forceinline__ ffloat2 ff_eval2(const float* tab, const FFTab& t, ffloat r2) {
+    float mid;
+    const float4* src = reinterpret_cast<const float4*>(tab) + ff_row_of(t, r2.hi, mid);
+    float2 c[kFFRow / 2];   // number j of both
 #pragma unroll
     for (int q = 0; q < kFFRow / 4; ++q) {
-        const float4 v = __ldg(src + q);
-        row[4 * q] = v.x;
-        row[4 * q + 1] = v.y;
-        row[4 * q + 2] = v.z;
-        row[4 * q + 3] = v.w;
+        const float4 v = __ldg(src + q * (t.last + 1));
+        c[2 * q] = make_float2(v.x, v.y);
+        c[2 * q + 1] = make_float2(v.z, v.w);
     }
+    // r2.hi - mid is exact (they lie within a factor 2); where the low part
+    // exceeds it, both are below 2^-20 A^2 and the pair is off by far less
+    // than 2^-40 A^2
+    const ffloat s = fast_two_sum(add_rn(r2.hi, -mid), r2.lo);
+    const float2 sh = f2_both(s.hi), nh = f2_both(-s.hi), sl = f2_both(s.lo);
+    ffloat2 v = {c[4], f2_fma(sh, f2_fma(c[7], sh, c[6]), c[5])};
+#pragma unroll
+    for (int k = 2; k >= 0; k -= 2) {   // v = c1 + s v, then c0 + s v (ff_madd)
+        const float2 np = f2_mul(nh, v.hi);
+        const float2 e = f2_fma(sh, v.lo, f2_fma(sl, v.hi, f2_fma(sh, v.hi, np)));
+        const ffloat2 w = two_diff2(c[k], np);
+        v = fast_two_sum2(w.hi, f2_add(w.lo, f2_add(c[k + 1], e)));
+    }
+    return v;
 }
-
-// The two polynomials of `row` at r^2 (float pair): out[0], out[1].
-__host__ __device__ __forceinline__ void ff_row_eval(const float* row, ffloat r2, ffloat out[2]) {
-    // s = r^2 - (u_k + r0^2): r2.hi and the knot's high part row[0] lie
-    // within a factor 2 of each other (r^2 falls in the knot's interval,
-    // ~0.04 A^2 wide, above 0.25 r0^2), so their difference is exact
-    // (Sterbenz); the low parts' difference joins it in one Fast2Sum (where
-    // that difference exceeds the first, both are below 2^-20 A^2 and the
-    // pair is off by far less than 2^-40 A^2)
-    const ffloat s = fast_two_sum(add_rn(r2.hi, -row[0]), add_rn(r2.lo, -row[1]));
-    out[0] = ff_poly(row + 2, s);
-    out[1] = ff_poly(row + 11, s);
-}
+__device__ __forceinline__ ffloat ff_first(ffloat2 v) { return {v.hi.x, v.lo.x}; }
+__device__ __forceinline__ ffloat ff_second(ffloat2 v) { return {v.hi.y, v.lo.y}; }
+#endif  // __CUDACC__
 
 // Exact split of a 64-bit integer |n| < 2^47 times 2^-kFixedBits64 into a
 // float pair (both parts exact: 24 + 23 bits).
@@ -528,49 +568,108 @@ __host__ __device__ __forceinline__ ffloat ff_norm2(ffloat x, ffloat y, ffloat z
     return fast_two_sum(s2.hi, add_rn(add_rn(s1.lo, s2.lo), add_rn(add_rn(ex, ey), ez)));
 }
 
-// Host evaluation with the kernels' arithmetic (diagnostic): row of the
-// table of u = r^2 - r0^2, or NULL below the table (u < u_lo, where the
-// kernels use the exponentials).
-inline const float* ff_row(const TabMeta& m, const std::vector<float>& tab, float uf) {
-    if (uf < m.u_lo_f) return nullptr;
-    return tab.data() + (size_t)ff_index(m, uf) * kFFRow;
+#ifdef __CUDACC__
+// fixed_to_ff of two separations.
+__device__ __forceinline__ ffloat2 fixed_to_ff2(long long m, long long n) {
+    const float2 hi = f2_mul(make_float2((float)(int)(m >> 23), (float)(int)(n >> 23)),
+                             f2_both(0x1p-21f));
+    const float2 lo = f2_add(make_float2(flt_from_bits((106u << 23) | ((unsigned)m & 0x7fffffu)),
+                                         flt_from_bits((106u << 23) | ((unsigned)n & 0x7fffffu))),
+                             f2_both(-0x1p-21f));
+    return fast_two_sum2(hi, lo);
+}
+// A separation: x and y side by side, z.
+struct ffvec {
+    ffloat2 xy;
+    ffloat z;
+};
+// ff_norm2 of a separation.
+__device__ __forceinline__ ffloat ff_norm2(const ffvec& d) {
+    const float2 h = d.xy.hi, np = f2_mul(f2_mul(h, f2_both(-1.f)), h);
+    const float2 e = f2_fma(f2_add(h, h), d.xy.lo, f2_fma(h, h, np));
+    const float pz = mul_rn(d.z.hi, d.z.hi);
+    const float ez = fmaf(2.f * d.z.hi, d.z.lo, fmaf(d.z.hi, d.z.hi, -pz));
+    const ffloat s1 = two_sum(-np.x, -np.y);
+    const ffloat s2 = two_sum(s1.hi, pz);
+    return fast_two_sum(s2.hi, add_rn(add_rn(s1.lo, s2.lo), add_rn(add_rn(e.x, e.y), ez)));
+}
+#endif  // __CUDACC__
+
+// Host evaluation of a table at r^2 with the kernels' arithmetic (diagnostic).
+inline void ff_eval(const std::vector<float>& tab, const FFTab& t, ffloat r2, ffloat out[2]) {
+    float mid;
+    const int k = ff_row_of(t, r2.hi, mid);
+    float row[kFFRow];
+    for (int e = 0; e < kFFRow; ++e) row[e] = tab[((size_t)(e / 4) * (t.last + 1) + k) * 4 + e % 4];
+    const ffloat s = fast_two_sum(add_rn(r2.hi, -mid), r2.lo);
+    out[0] = ff_poly(row, s);
+    out[1] = ff_poly(row + 1, s);
 }
 
-// Density rows (phi, g) and force rows (2 phi'/r, g'/r) from the Hermite
-// coefficients of build_rgl_tables (in t = s / h).
-inline void build_ff_tables(const RglTables& T, double r0, std::vector<float>& dens,
-                            std::vector<float>& force) {
-    const TabMeta& m = T.meta;
-    const int nint = m.nA + m.nB;
-    dens.assign((size_t)nint * kFFRow, 0.f);
-    force.assign((size_t)nint * kFFRow, 0.f);
-    const double hA = 1.0 / m.hA_inv, hB = 1.0 / m.hB_inv;
-    const double scale[4] = {1.0, 1.0, 4.0, 2.0};
-    auto split = [](double v, float* o) {
-        const float hi = (float)v;
-        o[0] = hi;
-        o[1] = (float)(v - (double)hi);
-    };
-    for (int i = 0; i < nint; ++i) {
-        const double h = i < m.nA ? hA : hB;
-        const double uk = i < m.nA ? (i - m.nA0) * hA : m.u_rs + (i - m.nA) * hB;
-        float* rows[2] = {dens.data() + (size_t)i * kFFRow, force.data() + (size_t)i * kFFRow};
-        split(uk + r0 * r0, rows[0]);
-        split(uk + r0 * r0, rows[1]);
-        for (int p = 0; p < 4; ++p) {
-            const double* src = (p < 2 ? T.dens64.data() + (size_t)i * kTabDens + 6 * p
-                                       : T.force64.data() + (size_t)i * kTabForce + 6 * (p - 2));
-            double hp = 1.0;
-            double cs[6];
-            for (int j = 0; j < 6; ++j) {
-                cs[j] = scale[p] * src[j] / hp;
-                hp *= h;
+// Density rows (phi, g) and force rows (2 phi'/r, g'/r).  Each polynomial is
+// the quintic Hermite interpolant of its interval, moved to the interval's
+// middle, with its fifth-degree term replaced by the Chebyshev-economised
+// lower ones (x^5 -> (20 x^3 - 5 x) / 16 on [-1, 1]): relative error
+// (a h / 2)^5 / 1920 for a function of logarithmic slope a in r^2, 6e-15 for
+// the Cu phi near r0.
+inline FFTab build_ff_tables(double A, double xi, double p, double q, double r0, double rs,
+                             double rc, std::vector<float>& dens, std::vector<float>& force) {
+    const double h = std::exp2(std::floor(std::log2(r0 * r0 / 326.0)));
+    FFTab t;
+    t.h = (float)h;
+    t.hinv = (float)(1.0 / h);
+    t.j_lo = std::max(1, (int)std::floor(0.25 * r0 * r0 / h));
+    t.r2_lo = (float)(t.j_lo * h);
+    t.rs2 = (float)(rs * rs);
+    const int j_rs = (int)std::floor(rs * rs / h), j_rc = (int)std::floor(rc * rc / h);
+    const int rows = std::max(j_rc - t.j_lo, 0) + 2;
+    t.last = rows - 1;
+    dens.assign((size_t)rows * kFFRow, 0.f);
+    force.assign((size_t)rows * kFFRow, 0.f);
+    auto fill = [&](int row, const double fa[2][4], const double fb[2][4]) {
+        for (int d = 0; d < 2; ++d)        // d = 0: f; d = 1: f_u, scaled for the force rows
+            for (int k = 0; k < 2; ++k) {
+                const double scale = d == 0 ? 1.0 : (k == 0 ? 4.0 : 2.0);
+                const double* a = fa[k] + d;
+                const double* b = fb[k] + d;
+                double x[6];
+                quintic_hermite(a[0], h * a[1], h * h * a[2], b[0], h * b[1], h * h * b[2], x);
+                // t = (1 + x) / 2: to the middle (Horner's shift), then x^n / 2^n
+                for (int m = 0; m < 5; ++m)
+                    for (int n = 4; n >= m; --n) x[n] += 0.5 * x[n + 1];
+                x[3] += 1.25 * 0.25 * x[5];          // 20/16 x^3 and -5/16 x of x^5
+                x[1] -= 0.3125 * 0.0625 * x[5];
+                const double s1 = 1.0 / h;           // powers of two: exact
+                double sm = scale;
+                auto put = [&](int j, float v) {   // number j of polynomial k
+                    const int e = 2 * j + k;
+                    (d == 0 ? dens : force)[((size_t)(e / 4) * rows + row) * 4 + e % 4] = v;
+                };
+                for (int m = 0; m < 5; ++m) {
+                    const double v = sm * x[m];
+                    sm *= s1;
+                    const float hi = (float)v;
+                    if (m < 3) {
+                        put(2 * m, hi);
+                        put(2 * m + 1, (float)(v - (double)hi));
+                    } else {
+                        put(m + 3, hi);
+                    }
+                }
             }
-            float* o = rows[p / 2] + 2 + 9 * (p % 2);
-            for (int j = 0; j < 3; ++j) split(cs[j], o + 2 * j);
-            for (int j = 0; j < 3; ++j) o[6 + j] = (float)cs[3 + j];
+    };
+    auto region = [&](int j0, int j1, int taper, int row) {
+        double f[2][2][4];   // at both ends of an interval
+        for (int j = j0; j <= j1; ++j) {
+            if (j == j0) rgl_derivs_u(A, xi, p, q, r0, rs, rc, std::sqrt(j * h), taper, f[j & 1]);
+            rgl_derivs_u(A, xi, p, q, r0, rs, rc, std::sqrt((j + 1) * h), taper, f[(j + 1) & 1]);
+            fill(row + j - j0, f[j & 1], f[(j + 1) & 1]);
         }
-    }
+    };
+    const int jb = std::max(t.j_lo, j_rs);
+    region(t.j_lo, std::min(j_rs, j_rc), 0, 0);
+    region(jb, j_rc, 3, jb - t.j_lo + 1);
+    return t;
 }
 
 }  // namespace fire2

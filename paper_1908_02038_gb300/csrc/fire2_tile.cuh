@@ -340,12 +340,11 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_density_tile(B
                 ffloat dx, dy, dz;
                 const ffloat r2 = tile_sep(qjx - qix, qjy - qiy, qjz - qiz, dx, dy, dz);
                 if (!(r2.hi < P.rc2_f)) continue;
-                const float uf = r2.hi - P.r0sq_f;
                 ffloat v[2];
-                if (uf >= P.tab.u_lo_f) {
-                    float row[kFFRow];
-                    load_row(b.tab_ffd, ff_index(P.tab, uf), row);
-                    ff_row_eval(row, r2, v);
+                if (r2.hi >= P.ff.r2_lo) {
+                    const ffloat2 w = ff_eval2(b.tab_ffd, P.ff, r2);
+                    v[0] = ff_first(w);
+                    v[1] = ff_second(w);
                 } else {
                     double rinv, phi, dphi, gg, dg;
                     rgl_pair64(P, ff_to_f64(r2), b.exp_table, rinv, phi, dphi, gg, dg);
@@ -462,12 +461,11 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_force_tile(Buf
                 ffloat dx, dy, dz;
                 const ffloat r2 = tile_sep(qjx - qix, qjy - qiy, qjz - qiz, dx, dy, dz);
                 if (!(r2.hi < P.rc2_f)) continue;
-                const float uf = r2.hi - P.r0sq_f;
                 ffloat c[2];
-                if (uf >= P.tab.u_lo_f) {
-                    float row[kFFRow];
-                    load_row(b.tab_fff, ff_index(P.tab, uf), row);
-                    ff_row_eval(row, r2, c);
+                if (r2.hi >= P.ff.r2_lo) {
+                    const ffloat2 w = ff_eval2(b.tab_fff, P.ff, r2);
+                    c[0] = ff_first(w);
+                    c[1] = ff_second(w);
                 } else {
                     double rinv, phi, dphi, gg, dg;
                     rgl_pair64(P, ff_to_f64(r2), b.exp_table, rinv, phi, dphi, gg, dg);
