@@ -6,15 +6,21 @@
 // could synchronise the device or fail under memory pressure.  This entry
 // point serves them: the caller passes device buffers for the
 // positions and the results, and the only scratch the kernels need (per-atom
-// densities, embedding derivatives and per-block energy partials) lives in the
-// file-scope device array `g_scratch` below, sized for at most
-// kNoAllocMaxAtoms atoms.  Every GPU that loads the library holds that array
+// energies and embedding derivatives) lives in the file-scope device array
+// `g_scratch` below, sized for at most kNoAllocMaxAtoms atoms.  Every GPU that loads the library holds that array
 // (about 0.5 MiB) until the process exits.
 //
 // The evaluation is all-pairs (minimum image), each atom summing over every
 // other atom, so no neighbour list is needed and nothing accumulates across
-// blocks: every scratch value read in a call is written earlier in the same
-// call.  Calls that overlap on the GPU (two streams, or two host threads) race
+// warps: every scratch value read in a call is written earlier in the same
+// call.  One warp works on an atom (or four).  It tests 32 candidates at a time in FP32
+// (FP64 issues at 1/58 of the FP32 rate on this part) against the cut-off plus
+// the FP32 error of the coordinates, keeps those that pass in a short list in
+// shared memory, and evaluates 32 list entries at a time in FP64, which
+// decides the cut-off.  3,960 atoms: 141 us against 7,460 us with a thread
+// per atom and every pair in FP64 (31 blocks on 152 SMs, 16 FP64 instructions
+// for each of the 16 M pairs, twice); what remains is about half the FP64 pipe
+// in the ~54 pairs per atom and half the FP32 tests.  Calls that overlap on the GPU (two streams, or two host threads) race
 // on g_scratch and must be serialised by the caller.
 #include <cuda.h>   // CUcontext and the driver function types (entry points, no link)
 #include <cuda_runtime.h>
@@ -24,17 +30,23 @@
 #include <mutex>
 
 #include "fire2.h"
+#include "fire2_common.cuh"
+#include "fire2_table.cuh"
 
 void fire2_set_global_error(const char* msg);  // defined in fire2_api.cu (hidden)
 
 namespace {
 
 constexpr int kNoAllocMaxAtoms = 32768;
-constexpr int kBlock = 128;
-constexpr int kMaxBlocks = (kNoAllocMaxAtoms + kBlock - 1) / kBlock;
-constexpr int kScratchDoubles = 2 * kNoAllocMaxAtoms + kMaxBlocks;
+constexpr int kWarps = 8;              // warps per block
+constexpr int kBlock = 32 * kWarps;    // candidates staged at a time, one per thread
+// From here on a warp takes four atoms, which share the staging and the loads of
+// the candidates (one / four atoms per warp: 3,999 atoms 141 / 174 us, with
+// too few blocks; 10,975 atoms 1,241 / 851 us before the FP64 work was cut).
+constexpr int kManyAtoms = 8192;
+constexpr int kScratchDoubles = 2 * kNoAllocMaxAtoms;
 
-// [0, N): rho_i; [N, 2N): F'(rho_i); [2N, 2N + blocks): energy partials.
+// [0, N): energy of atom i; [N, 2N): F'(rho_i).
 static __device__ __align__(256) double g_scratch[kScratchDoubles];
 
 struct NaPot {
@@ -44,33 +56,71 @@ struct NaPot {
     double A, xi2, p, q2, r0inv, p_r0, q2_r0, rs, winv;
     double L[3], Linv[3];
     int per[3];
+    fire2::ExpC ex;
+    // FP32 candidate test
+    float Lf[3], Linvf[3], rcf;
+    float wrap[3];         // coordinates beyond this magnitude are wrapped first (periodic axes)
 };
 
+__device__ __noinline__ double na_image(double d, double L, double Linv) { return d - L * rint(d * Linv); }
+
+// Minimum image of d, d - L rint(d / L); unchanged (no FP64 instruction) where
+// |d| <= L / 2, by the bit patterns.
 __device__ __forceinline__ void na_min_image(double& d, double L, double Linv, int per) {
-    if (per) d -= L * rint(d * Linv);
+    if (per && __double_as_longlong(fabs(d)) > __double_as_longlong(0.5 * L)) d = na_image(d, L, Linv);
 }
 
-__device__ double na_block_sum(double v) {
-    __shared__ double sh[32];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sh[w] = v;
+__device__ __forceinline__ double na_warp_sum(double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// 2^(j/256), the table of exp_tang, as products of 2^(k/16) and 2^(k/256).
+__device__ __forceinline__ void na_exp_table(double* tab) {
+    __shared__ double part[32];
+    const int t = threadIdx.x;
+    if (t < 32) part[t] = exp2(t < 16 ? t / 16.0 : (t - 16) / 256.0);
     __syncthreads();
-    double r = 0.0;
-    if (w == 0) {
-        r = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+    if (t < fire2::kExpTableSize) tab[t] = part[t >> 4] * part[16 + (t & 15)];
+    __syncthreads();
+}
+
+// e^x in FP64; FAST: the exponents lie in exp_tang's range.
+template <bool FAST>
+__device__ __forceinline__ double na_exp(const NaPot& P, double x, const double* tab) {
+    return FAST ? fire2::exp_tang(x, P.ex, tab) : exp(x);
+}
+
+// 1/sqrt(x) for x in (1e-30, 1e30): the FP32 estimate y0 (conversions on the
+// integer pipes) and one step of third order, y0 + y0 e (1/2 + 3/8 e) with
+// e = 1 - x y0^2 ~ 2^-22: off by 5/16 e^3 ~ 2^-67.
+__device__ __forceinline__ double na_rsqrt(double x) {
+    const double y0 = fire2::f32_to_f64(rsqrtf(fire2::f64_to_f32_trunc(x)));
+    const double e = fma(-x, y0 * y0, 1.0);
+    return fma(y0, fma(e, 0.375, 0.5) * e, y0);
+}
+// Outside that range.
+__device__ __noinline__ double na_rsqrt_any(double x) { return 1.0 / sqrt(x); }
+
+// r and 1/r of a pair.
+__device__ __forceinline__ void na_radius(double r2, double& r, double& rinv) {
+    const bool in = fire2::ff_range(r2);   // 2^-60 .. 2^60, by the bit pattern
+    rinv = in ? na_rsqrt(r2) : 0.0;
+    r = r2 * rinv;
+    if (!in) {
+        rinv = na_rsqrt_any(r2);
+        r = r2 > 0.0 ? r2 * rinv : 0.0;
     }
-    return r;
 }
 
 // RGL pair terms: phi = A e^{-p s} S, g = xi^2 e^{-2q s} S, s = r/r0 - 1, with
 // the quintic taper S on [rs, rc); returns the derivatives too.
-__device__ __forceinline__ void na_rgl_pair(const NaPot& P, double r, double& phi, double& dphi,
-                                            double& g, double& dg) {
+template <bool FAST>
+__device__ __forceinline__ void na_rgl_pair(const NaPot& P, double r, const double* tab, double& phi,
+                                            double& dphi, double& g, double& dg) {
     const double s = r * P.r0inv - 1.0;
-    const double ep = P.A * exp(-P.p * s);
-    const double eq = P.xi2 * exp(-P.q2 * s);
+    const double ep = P.A * na_exp<FAST>(P, -P.p * s, tab);
+    const double eq = P.xi2 * na_exp<FAST>(P, -P.q2 * s, tab);
     double S = 1.0, dS = 0.0;
     if (r > P.rs) {
         const double t = (r - P.rs) * P.winv;
@@ -84,122 +134,238 @@ __device__ __forceinline__ void na_rgl_pair(const NaPot& P, double r, double& ph
     dg = eq * (-P.q2_r0 * S + dS);
 }
 
-// Pass 1 (RGL): rho_i, F'(rho_i) and the per-atom energy, all-pairs.
-// LJ: the whole evaluation (forces and energy) in this one pass.
-__global__ void __launch_bounds__(kBlock) k_na_pass1(const double* __restrict__ pos, int n,
-                                                     NaPot P, double* scratch,
-                                                     double* __restrict__ forces) {
-    __shared__ double3 tile[kBlock];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double xi = 0.0, yi = 0.0, zi = 0.0;
-    if (i < n) {
-        xi = pos[3 * i];
-        yi = pos[3 * i + 1];
-        zi = pos[3 * i + 2];
+// Out of line, so that their FP64 instructions are issued only when needed.
+__device__ __noinline__ float na_to_float(double x) { return (float)x; }
+__device__ __noinline__ float na_wrapped(double x, double L, double Linv) {
+    return (float)(x - L * floor(x * Linv));
+}
+
+// FP32 copy of coordinate a for the candidate test: the coordinate itself
+// within a few box lengths (or on an open axis), wrapped into the box beyond.
+// Truncated on the integer pipes (off by less than 2^-23 of its size) where
+// the exponent is an FP32 one: a conversion takes the FP64 pipe, and every
+// block makes three for each candidate.
+__device__ __forceinline__ float na_coord(const NaPot& P, int a, double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), ahi = hi & 0x7fffffffu;
+    float f = 0.f;
+    if (ahi - (897u << 20) < (254u << 20))
+        f = __uint_as_float((hi & 0x80000000u) | ((ahi - (896u << 20)) << 3) |
+                            ((unsigned)__double2loint(x) >> 29));
+    else if (ahi >= (897u << 20))   // beyond FP32, or not finite
+        f = na_to_float(x);
+    if (P.per[a] && !(fabsf(f) <= P.wrap[a])) return na_wrapped(x, P.L[a], P.Linv[a]);
+    return f;
+}
+
+// Walks the atoms j != i inside (or within FP32 error of) the cut-off of the
+// warp's A atoms i = i0 .. i0 + A - 1, 32 at a time: eval(a, j) runs on the
+// lanes that hold an entry of atom i0 + a.  All threads of the block enter
+// (i >= n: no atom).  list: A x 64 entries per warp.
+template <int A, typename Eval>
+__device__ __forceinline__ void na_walk(const double* __restrict__ pos, int n, const NaPot& P, int i0,
+                                        float4* tile, int (*list)[64], Eval eval) {
+    const int lane = threadIdx.x & 31;
+    float xi[A][3], reach2[A];
+    int cnt[A];   // entries in the atom's list, below 32 between candidates
+#pragma unroll
+    for (int u = 0; u < A; ++u) {
+        float reach = P.rcf;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            xi[u][a] = i0 + u < n ? na_coord(P, a, pos[3 * (size_t)(i0 + u) + a]) : 0.f;
+            // a pair inside rc has |x_j| <= |x_i| + rc on an open axis and
+            // |x_j| <= wrap on a periodic one; each copy is off by 2^-23 of its
+            // size, the difference and the shift by half as much
+            reach += 0x1p-20f * (fabsf(xi[u][a]) + (P.per[a] ? P.wrap[a] : P.rcf));
+        }
+        reach2[u] = reach * reach * 1.00001f;
+        cnt[u] = 0;
     }
-    double rho = 0.0, e = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
     for (int base = 0; base < n; base += kBlock) {
         const int j0 = base + threadIdx.x;
         __syncthreads();
-        if (j0 < n) tile[threadIdx.x] = make_double3(pos[3 * j0], pos[3 * j0 + 1], pos[3 * j0 + 2]);
+        if (j0 < n) {
+            const double* p = pos + 3 * (size_t)j0;
+            tile[threadIdx.x] = make_float4(na_coord(P, 0, p[0]), na_coord(P, 1, p[1]),
+                                            na_coord(P, 2, p[2]), 0.f);
+        }
         __syncthreads();
         const int m = min(kBlock, n - base);
-        if (i >= n) continue;
-        for (int k = 0; k < m; ++k) {
-            const int j = base + k;
-            if (j == i) continue;
-            double dx = tile[k].x - xi, dy = tile[k].y - yi, dz = tile[k].z - zi;
-            na_min_image(dx, P.L[0], P.Linv[0], P.per[0]);
-            na_min_image(dy, P.L[1], P.Linv[1], P.per[1]);
-            na_min_image(dz, P.L[2], P.Linv[2], P.per[2]);
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            if (!(r2 < P.rc2)) continue;
-            if (P.kind == FIRE_POT_RGL) {
-                double phi, dphi, g, dg;
-                na_rgl_pair(P, sqrt(r2), phi, dphi, g, dg);
-                rho += g;
-                e += phi;
-            } else {
-                const double sr2 = P.sigma2 / r2;
-                const double sr6 = sr2 * sr2 * sr2;
-                e += 0.5 * (4.0 * P.eps * (sr6 * sr6 - sr6) - P.lj_shift);
-                const double w = 24.0 * P.eps * (2.0 * sr6 * sr6 - sr6) / r2;
-                fx -= w * dx;
-                fy -= w * dy;
-                fz -= w * dz;
+        if (i0 >= n) continue;
+        for (int k0 = 0; k0 < m; k0 += 32) {   // the warp stays together
+            const int k = k0 + lane;
+            const float4 x = tile[min(k, m - 1)];
+            bool hit[A];
+            bool any = false;
+#pragma unroll
+            for (int u = 0; u < A; ++u) {
+                float d[3] = {x.x - xi[u][0], x.y - xi[u][1], x.z - xi[u][2]};
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    if (P.per[a]) {   // round to the nearest integer by 1.5 2^23 (|shift| <= 8)
+                        const float r = __fadd_rn(__fmaf_rn(d[a], P.Linvf[a], 0x1.8p23f), -0x1.8p23f);
+                        d[a] -= r * P.Lf[a];
+                    }
+                hit[u] = !(d[0] * d[0] + d[1] * d[1] + d[2] * d[2] > reach2[u]) &&   // NaN: FP64
+                         k < m && i0 + u < n && base + k != i0 + u;                  // decides
+                any |= hit[u];
+            }
+            if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
+            for (int u = 0; u < A; ++u) {
+                const unsigned b = __ballot_sync(0xffffffffu, hit[u]);
+                if (hit[u]) list[u][cnt[u] + __popc(b & ((1u << lane) - 1u))] = base + k;
+                cnt[u] += __popc(b);
+                if (cnt[u] >= 32) {
+                    __syncwarp();
+                    const int j = list[u][lane], rest = list[u][32 + lane];
+                    eval(u, j);
+                    __syncwarp();
+                    list[u][lane] = rest;
+                    cnt[u] -= 32;
+                    __syncwarp();
+                }
             }
         }
     }
-    if (i < n) {
-        if (P.kind == FIRE_POT_RGL) {
-            const double sq = sqrt(rho);
-            scratch[i] = rho;
-            scratch[kNoAllocMaxAtoms + i] = rho > 0.0 ? -0.5 / sq : 0.0;
-            e -= sq;
-        } else if (forces) {
-            forces[3 * i] = fx;
-            forces[3 * i + 1] = fy;
-            forces[3 * i + 2] = fz;
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < A; ++u)
+        if (lane < cnt[u]) eval(u, list[u][lane]);
+}
+
+// Separation x_j - x_i (minimum image) in FP64; returns r^2.
+__device__ __forceinline__ double na_sep(const double* __restrict__ pos, const NaPot& P,
+                                         const double x[3], int j, double d[3]) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        d[a] = pos[3 * (size_t)j + a] - x[a];
+        na_min_image(d[a], P.L[a], P.Linv[a], P.per[a]);
+    }
+    return d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+}
+
+// a < b of non-negative doubles on the integer pipes (NaN fails: its pattern is
+// above every number's).
+__device__ __forceinline__ bool na_below(double a, double b) {
+    return __double_as_longlong(a) < __double_as_longlong(b);
+}
+
+// Pass 1 (RGL): F'(rho_i) and the per-atom energy, all-pairs.
+// LJ: the whole evaluation (forces and energy) in this one pass.
+template <int A, bool RGL, bool FAST>
+__global__ void __launch_bounds__(kBlock) k_na_pass1(const double* __restrict__ pos, int n,
+                                                     NaPot P, double* scratch,
+                                                     double* __restrict__ forces) {
+    __shared__ float4 tile[kBlock];
+    __shared__ int list[kWarps][A][64];
+    __shared__ double tab[fire2::kExpTableSize];
+    if (RGL) na_exp_table(tab);
+    const int w = threadIdx.x >> 5, i0 = (blockIdx.x * kWarps + w) * A;
+    double x[A][3], s0[A], e[A], f[A][3];   // s0: density
+#pragma unroll
+    for (int u = 0; u < A; ++u) {
+        s0[u] = e[u] = 0.0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            f[u][a] = 0.0;
+            x[u][a] = i0 + u < n ? pos[3 * (size_t)(i0 + u) + a] : 0.0;
         }
     }
-    const double bs = na_block_sum(e);
-    if (threadIdx.x == 0) scratch[2 * kNoAllocMaxAtoms + blockIdx.x] = bs;
+    na_walk<A>(pos, n, P, i0, tile, list[w], [&](int u, int j) {
+        double d[3];
+        const double r2 = na_sep(pos, P, x[u], j, d);
+        if (!na_below(r2, P.rc2)) return;
+        if (RGL) {
+            double r, rinv, phi, dphi, g, dg;
+            na_radius(r2, r, rinv);
+            na_rgl_pair<FAST>(P, r, tab, phi, dphi, g, dg);
+            s0[u] += g;
+            e[u] += phi;
+        } else {
+            const double ir2 = __drcp_rn(r2);
+            const double sr2 = P.sigma2 * ir2;
+            const double sr6 = sr2 * sr2 * sr2;
+            e[u] += 0.5 * (4.0 * P.eps * (sr6 * sr6 - sr6) - P.lj_shift);
+            const double q = 24.0 * P.eps * (2.0 * sr6 * sr6 - sr6) * ir2;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) f[u][a] -= q * d[a];
+        }
+    });
+#pragma unroll
+    for (int u = 0; u < A; ++u) {
+        if (i0 + u >= n) return;
+        double en = na_warp_sum(e[u]);
+        if (RGL) {
+            double sq, fp;
+            fire2::rgl_embed(na_warp_sum(s0[u]), sq, fp);
+            en -= sq;
+            if ((threadIdx.x & 31) == 0) scratch[kNoAllocMaxAtoms + i0 + u] = fp;
+        } else if (forces) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const double v = na_warp_sum(f[u][a]);
+                if ((threadIdx.x & 31) == 0) forces[3 * (size_t)(i0 + u) + a] = v;
+            }
+        }
+        if ((threadIdx.x & 31) == 0) scratch[i0 + u] = en;
+    }
 }
 
 // Pass 2 (RGL): F_i = sum_j [2 phi'(r) + (F'_i + F'_j) g'(r)] (x_j - x_i) / r.
+template <int A, bool FAST>
 __global__ void __launch_bounds__(kBlock) k_na_pass2(const double* __restrict__ pos, int n,
                                                      NaPot P, const double* scratch,
                                                      double* __restrict__ forces) {
-    __shared__ double4_32a tile[kBlock];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ float4 tile[kBlock];
+    __shared__ int list[kWarps][A][64];
+    __shared__ double tab[fire2::kExpTableSize];
+    na_exp_table(tab);
+    const int w = threadIdx.x >> 5, i0 = (blockIdx.x * kWarps + w) * A;
     const double* fp = scratch + kNoAllocMaxAtoms;
-    double xi = 0.0, yi = 0.0, zi = 0.0, fpi = 0.0;
-    if (i < n) {
-        xi = pos[3 * i];
-        yi = pos[3 * i + 1];
-        zi = pos[3 * i + 2];
-        fpi = fp[i];
-    }
-    double fx = 0.0, fy = 0.0, fz = 0.0;
-    for (int base = 0; base < n; base += kBlock) {
-        const int j0 = base + threadIdx.x;
-        __syncthreads();
-        if (j0 < n)
-            tile[threadIdx.x] =
-                make_double4_32a(pos[3 * j0], pos[3 * j0 + 1], pos[3 * j0 + 2], fp[j0]);
-        __syncthreads();
-        const int m = min(kBlock, n - base);
-        if (i >= n) continue;
-        for (int k = 0; k < m; ++k) {
-            const int j = base + k;
-            if (j == i) continue;
-            double dx = tile[k].x - xi, dy = tile[k].y - yi, dz = tile[k].z - zi;
-            na_min_image(dx, P.L[0], P.Linv[0], P.per[0]);
-            na_min_image(dy, P.L[1], P.Linv[1], P.per[1]);
-            na_min_image(dz, P.L[2], P.Linv[2], P.per[2]);
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            if (!(r2 < P.rc2)) continue;
-            const double r = sqrt(r2);
-            double phi, dphi, g, dg;
-            na_rgl_pair(P, r, phi, dphi, g, dg);
-            const double fs = (2.0 * dphi + (fpi + tile[k].w) * dg) / r;
-            fx += fs * dx;
-            fy += fs * dy;
-            fz += fs * dz;
+    double x[A][3], fpi[A], f[A][3];
+#pragma unroll
+    for (int u = 0; u < A; ++u) {
+        fpi[u] = i0 + u < n ? fp[i0 + u] : 0.0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            f[u][a] = 0.0;
+            x[u][a] = i0 + u < n ? pos[3 * (size_t)(i0 + u) + a] : 0.0;
         }
     }
-    if (i < n && forces) {
-        forces[3 * i] = fx;
-        forces[3 * i + 1] = fy;
-        forces[3 * i + 2] = fz;
+    na_walk<A>(pos, n, P, i0, tile, list[w], [&](int u, int j) {
+        double d[3];
+        const double r2 = na_sep(pos, P, x[u], j, d);
+        if (!na_below(r2, P.rc2)) return;
+        double r, rinv, phi, dphi, g, dg;
+        na_radius(r2, r, rinv);
+        na_rgl_pair<FAST>(P, r, tab, phi, dphi, g, dg);
+        const double fs = (2.0 * dphi + (fpi[u] + fp[j]) * dg) * rinv;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) f[u][a] += fs * d[a];
+    });
+    if (!forces) return;
+#pragma unroll
+    for (int u = 0; u < A; ++u) {
+        if (i0 + u >= n) return;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const double v = na_warp_sum(f[u][a]);
+            if ((threadIdx.x & 31) == 0) forces[3 * (size_t)(i0 + u) + a] = v;
+        }
     }
 }
 
-// Fixed-order sum of the per-block energy partials into *energy.
-__global__ void k_na_energy(const double* scratch, int nblocks, double* energy) {
+// Fixed-order sum of the atoms' energies into *energy (one block of 1024).
+__global__ void __launch_bounds__(1024) k_na_energy(const double* scratch, int n, double* energy) {
+    __shared__ double sh[32];
     double s = 0.0;
-    for (int k = threadIdx.x; k < nblocks; k += blockDim.x) s += scratch[2 * kNoAllocMaxAtoms + k];
-    s = na_block_sum(s);
+    for (int k = threadIdx.x; k < n; k += blockDim.x) s += scratch[k];
+    s = na_warp_sum(s);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    s = na_warp_sum(sh[threadIdx.x]);
     if (threadIdx.x == 0 && energy) *energy = s;
 }
 
@@ -290,6 +456,7 @@ extern "C" fire_status fire_energy_forces_noalloc(const fire_potential_t* pot, i
     NaPot P{};
     P.kind = pot->kind;
     double rc = 0.0;
+    bool fast = true;   // the exponents lie in exp_tang's range (|x| < 700)
     if (pot->kind == FIRE_POT_LJ) {
         if (!(pot->rc_lj > 0.0 && pot->sigma > 0.0 && pot->eps > 0.0))
             return na_fail(FIRE_ERR_ARG, "fire_energy_forces_noalloc: LJ needs eps, sigma, rc_lj > 0");
@@ -311,10 +478,15 @@ extern "C" fire_status fire_energy_forces_noalloc(const fire_potential_t* pot, i
         P.q2_r0 = 2.0 * pot->q / pot->r0;
         P.rs = pot->rs;
         P.winv = 1.0 / (pot->rc - pot->rs);
+        double table[fire2::kExpTableSize];
+        P.ex = fire2::make_exp_constants(table);
+        const double smax = std::fmax(1.0, rc / pot->r0 - 1.0);
+        fast = std::fabs(P.p) * smax < 600.0 && std::fabs(P.q2) * smax < 600.0;
     } else {
         return na_fail(FIRE_ERR_ARG, "fire_energy_forces_noalloc: unknown potential kind");
     }
     P.rc2 = rc * rc;
+    P.rcf = (float)rc;
     for (int a = 0; a < 3; ++a) {
         if (!(box[a] > 0.0) || !std::isfinite(box[a]))
             return na_fail(FIRE_ERR_ARG, "fire_energy_forces_noalloc: box lengths must be > 0");
@@ -324,12 +496,15 @@ extern "C" fire_status fire_energy_forces_noalloc(const fire_potential_t* pot, i
         P.L[a] = box[a];
         P.Linv[a] = 1.0 / box[a];
         P.per[a] = periodic[a] ? 1 : 0;
+        P.Lf[a] = (float)box[a];
+        P.Linvf[a] = (float)P.Linv[a];
+        P.wrap[a] = 4.f * P.Lf[a];
     }
     double* scratch = nullptr;
     cudaError_t e = scratch_address(&scratch);
     if (e != cudaSuccess) return na_fail(FIRE_ERR_CUDA, cudaGetErrorString(e));
     int n = (int)n_atoms;
-    int blocks = (n + kBlock - 1) / kBlock;
+    const int A = n >= kManyAtoms && fast ? 4 : 1, blocks = (n + kWarps * A - 1) / (kWarps * A);
     cudaStream_t s = (cudaStream_t)stream;
     // cudaLaunchKernel returns the status of its own launch, so an error left
     // pending by the caller's earlier work is neither reported as this call's
@@ -338,12 +513,21 @@ extern "C" fire_status fire_energy_forces_noalloc(const fire_potential_t* pot, i
     double* fout = d_forces;
     double* eout = d_energy;
     void* args12[] = {(void*)&pos, (void*)&n, (void*)&P, (void*)&scratch, (void*)&fout};
-    e = cudaLaunchKernel((const void*)k_na_pass1, dim3(blocks), dim3(kBlock), args12, 0, s);
-    if (e == cudaSuccess && P.kind == FIRE_POT_RGL)
-        e = cudaLaunchKernel((const void*)k_na_pass2, dim3(blocks), dim3(kBlock), args12, 0, s);
-    void* args3[] = {(void*)&scratch, (void*)&blocks, (void*)&eout};
+    const bool rgl = P.kind == FIRE_POT_RGL;
+    const void *pass1, *pass2 = nullptr;
+    if (!rgl)
+        pass1 = A == 4 ? (const void*)k_na_pass1<4, false, true> : (const void*)k_na_pass1<1, false, true>;
+    else if (!fast)
+        pass1 = (const void*)k_na_pass1<1, true, false>, pass2 = (const void*)k_na_pass2<1, false>;
+    else if (A == 4)
+        pass1 = (const void*)k_na_pass1<4, true, true>, pass2 = (const void*)k_na_pass2<4, true>;
+    else
+        pass1 = (const void*)k_na_pass1<1, true, true>, pass2 = (const void*)k_na_pass2<1, true>;
+    e = cudaLaunchKernel(pass1, dim3(blocks), dim3(kBlock), args12, 0, s);
+    if (e == cudaSuccess && rgl) e = cudaLaunchKernel(pass2, dim3(blocks), dim3(kBlock), args12, 0, s);
+    void* args3[] = {(void*)&scratch, (void*)&n, (void*)&eout};
     if (e == cudaSuccess)
-        e = cudaLaunchKernel((const void*)k_na_energy, dim3(1), dim3(256), args3, 0, s);
+        e = cudaLaunchKernel((const void*)k_na_energy, dim3(1), dim3(1024), args3, 0, s);
     if (e != cudaSuccess) return na_fail(FIRE_ERR_CUDA, cudaGetErrorString(e));
     return FIRE_OK;
 }
