@@ -127,6 +127,8 @@ struct Bufs {
     int* tile_ns;
     double *crep, *cden;
     int *cell_of, *cell_count, *cell_start, *cell_atoms;
+    float4* xs;            // cell mode: FP32 positions in the order of cell_atoms, index in w
+    float2* cell_box;      // smallest and largest FP32 x, y, z of each cell's atoms [3 c + axis]
     double *epart, *rpart;
     DevState* st;
     double* pos_io;        // N x 3 row-major, in/out of a relaxation
@@ -266,32 +268,58 @@ __global__ void k_cell_count(Bufs b, GeoC g, int force) {
     atomicAdd(&b.cell_count[c], 1);
 }
 
-// Exclusive scan of the cell counts (one block); cell_start[ncell] = N.
+// Exclusive scan of the cell counts (one block of 1024); cell_start[ncell] = N.
 // cell_count is turned into a fill cursor (= cell_start) for k_cell_fill.
-__global__ void k_cell_scan(Bufs b, GeoC g, int force) {
+// Tiles of 4 counts per thread, read and written as 16-byte words: 9,700 cells
+// 15 -> 7 us (each thread a stretch of its own before, uncoalesced).
+__global__ void __launch_bounds__(1024) k_cell_scan(Bufs b, GeoC g, int force) {
     if (!need_rebuild(b.st, g, force)) return;
-    __shared__ int sh[1024];
-    const int T = blockDim.x, t = threadIdx.x;
-    const int per = (b.ncell + T - 1) / T;
-    const int lo = min(t * per, b.ncell), hi = min(lo + per, b.ncell);
-    int s = 0;
-    for (int c = lo; c < hi; ++c) s += b.cell_count[c];
-    sh[t] = s;
-    __syncthreads();
-    for (int o = 1; o < T; o <<= 1) {
-        int add = t >= o ? sh[t - o] : 0;
+    __shared__ int sh[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int carry = 0;   // cells before this tile, the same in every thread
+    for (int base = 0; base < b.ncell; base += 4096) {
+        const int c = base + 4 * (int)threadIdx.x;
+        int v[4], s = 0;
+        if (c + 4 <= b.ncell) {
+            const int4 q = *reinterpret_cast<const int4*>(b.cell_count + c);
+            v[0] = q.x;
+            v[1] = q.y;
+            v[2] = q.z;
+            v[3] = q.w;
+        } else {
+            for (int u = 0; u < 4; ++u) v[u] = c + u < b.ncell ? b.cell_count[c + u] : 0;
+        }
+        s = v[0] + v[1] + v[2] + v[3];
+        int t = s;   // inclusive scan over the warp
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += x;
+        }
+        __syncthreads();   // sh may hold the tile before
+        if (lane == 31) sh[w] = t;
         __syncthreads();
-        sh[t] += add;
-        __syncthreads();
+        int ws = sh[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, ws, o);
+            if (lane >= o) ws += x;
+        }
+        const int before = w ? __shfl_sync(0xffffffffu, ws, w - 1) : 0;
+        int run = carry + before + t - s;
+        carry += __shfl_sync(0xffffffffu, ws, 31);
+        int q[4];
+        for (int u = 0; u < 4; ++u) {
+            q[u] = run;
+            run += v[u];
+        }
+        if (c + 4 <= b.ncell) {
+            const int4 r = make_int4(q[0], q[1], q[2], q[3]);
+            *reinterpret_cast<int4*>(b.cell_start + c) = r;
+            *reinterpret_cast<int4*>(b.cell_count + c) = r;
+        } else {
+            for (int u = 0; u < 4 && c + u < b.ncell; ++u) b.cell_start[c + u] = b.cell_count[c + u] = q[u];
+        }
     }
-    int run = sh[t] - s;
-    for (int c = lo; c < hi; ++c) {
-        const int k = b.cell_count[c];
-        b.cell_start[c] = run;
-        b.cell_count[c] = run;
-        run += k;
-    }
-    if (t == T - 1) b.cell_start[b.ncell] = sh[t];
+    if (threadIdx.x == 0) b.cell_start[b.ncell] = carry;
 }
 
 __global__ void k_cell_fill(Bufs b, GeoC g, int force) {
@@ -304,28 +332,51 @@ __global__ void k_cell_fill(Bufs b, GeoC g, int force) {
 
 // The fill above places a cell's atoms in atomic order; sorting each cell by
 // atom index makes the neighbour lists, and with them every sum over a list,
-// the same from run to run (one thread per cell, ~13 atoms per cell).
-__global__ void k_cell_sort(Bufs b, GeoC g, int force) {
+// the same from run to run.  One warp per cell: an atom's place is the number
+// of smaller indices (~13 atoms per cell; a cell of more than 32 takes them 32
+// at a time).  The FP32 positions follow into cell order (xs), where the list
+// build reads its candidates from consecutive addresses.
+__global__ void __launch_bounds__(kElemBlock) k_cell_sort(Bufs b, GeoC g, int force) {
     if (!need_rebuild(b.st, g, force)) return;
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (c >= b.ncell) return;
-    int* a = b.cell_atoms + b.cell_start[c];
-    const int m = b.cell_start[c + 1] - b.cell_start[c];
-    for (int k = 1; k < m; ++k) {
-        const int v = a[k];
-        int j = k - 1;
-        while (j >= 0 && a[j] > v) {
-            a[j + 1] = a[j];
-            --j;
+    const int k0 = b.cell_start[c], m = b.cell_start[c + 1] - k0;
+    int* a = b.cell_atoms + k0;
+    float lo[3] = {INFINITY, INFINITY, INFINITY};   // NaN coordinates are in no pair
+    float hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    for (int base = 0; base < m; base += 32) {
+        const int v = base + lane < m ? a[base + lane] : 0;
+        int rank = 0;
+        for (int from = 0; from < m; from += 32) {
+            const int u = from + lane < m ? a[from + lane] : 0x7fffffff;
+            const int cnt = min(32, m - from);
+            for (int q = 0; q < cnt; ++q) rank += __shfl_sync(0xffffffffu, u, q) < v ? 1 : 0;
         }
-        a[j + 1] = v;
+        if (base + lane < m) {
+            float4 x = b.xf[v];
+            x.w = __int_as_float(v);
+            b.xs[k0 + rank] = x;
+            const float p[3] = {x.x, x.y, x.z};
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                lo[q] = fminf(lo[q], p[q]);
+                hi[q] = fmaxf(hi[q], p[q]);
+            }
+        }
     }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        for (int o = 16; o > 0; o >>= 1) {
+            lo[q] = fminf(lo[q], __shfl_xor_sync(0xffffffffu, lo[q], o));
+            hi[q] = fmaxf(hi[q], __shfl_xor_sync(0xffffffffu, hi[q], o));
+        }
+        if (lane == 0) b.cell_box[3 * (size_t)c + q] = make_float2(lo[q], hi[q]);
+    }
+    __syncwarp();   // every index is read (and the warp's xs are visible to it)
+    for (int k = lane; k < m; k += 32) a[k] = __float_as_int(b.xs[k0 + k].w);
 }
 
-// Candidate test in FP32 (the FP64 unit is ~58x slower on this part): the
-// list radius carries a margin larger than the FP32 rounding of the
-// positions, so every pair closer than rc + skin is kept; the force kernels
-// test r < rc again in FP64.
+// FP32 position of atom j from its FP64 one (the all-pairs build).
 __device__ __forceinline__ float4 xf_of(const Bufs& b, int j) {
     const dvec4 x = b.x[j];
     return make_float4((float)x.x, (float)x.y, (float)x.z, 0.f);
@@ -336,111 +387,309 @@ __device__ __forceinline__ float4 xf_of(const Bufs& b, int j) {
 // the lanes of a warp evaluate their in-range pairs together and skip their
 // skin pairs together; a warp otherwise issues the whole pair evaluation
 // whenever any of its lanes has an in-range pair at that list position.
-// Skin pairs wait in a small per-thread buffer and are appended at the end
-// (beyond kSkinBuf of them the rest are written in the order found).
+// Skin pairs wait in a small buffer and are appended at the end (beyond
+// kSkinBuf of them the rest are written in the order found).
+//
+// One warp builds the list of an atom: its lanes test 32 candidates, staged in
+// shared memory by the block, and ballots give the entries their places in
+// candidate order.  With a thread per atom (each lane walking cells of its own)
+// the lanes diverged at every cell and small systems had a few dozen warps;
+// the whole build, thread / warp per atom: 255 LJ atoms (all pairs) 111 / 9 us,
+// 497 atoms 177 / 37, 3,960 atoms 203 / 40, 31,680 atoms 228 / 74, 119,023
+// atoms 248 / 138, 997,450 atoms 1422 / 924 (half list) and 1467 / 1114 us
+// (full list).  Bound by the issue of the FP32 tests (67 % of the slots).
 constexpr int kSkinBuf = 24;
-struct SkinBuf {
-    uint32_t e[kSkinBuf];
-    int n;
+constexpr int kBuildWarps = 4;       // warps per block, and on small systems (few
+constexpr int kBuildWarpsSmall = 16; // blocks): an atom per warp
+constexpr int kBuildCand = 1024;     // staged candidates, padded to whole warps with NaN
+
+struct ListState {   // of one atom, the same in all lanes
+    int cnt = 0;     // entries written (in range, and skin beyond the buffer)
+    int skin = 0;    // entries in the skin buffer
 };
 
-// FP32 positions come from xf (refreshed by k_cell_count) in cell mode and
-// are converted from x in the all-pairs mode (small systems); the caller
-// passes candidate j's position xj.
-__device__ __forceinline__ void try_add_pair(const Bufs& b, const GeoC& g, int i, float4 xi,
-                                             int j, float4 xj, int& cnt, SkinBuf& sk) {
-    float d[3] = {xj.x - xi.x, xj.y - xi.y, xj.z - xi.z};
-    int s[3] = {0, 0, 0};
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        if (g.per[a]) {
-            s[a] = __float2int_rn(d[a] * g.Linvf[a]);
-            d[a] -= (float)s[a] * g.Lf[a];
-        }
-    }
-    const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-    if (!(r2 < g.rlist2f)) return;  // NaN fails too
-    if (!g.full && !upper_half(d[0], d[1], d[2])) return;
-    // image codes cover shifts of -2..2 box lengths; atoms further apart than
-    // that in raw coordinates are a caller error (positions far outside the box)
-    if (s[0] < -2 || s[0] > 2 || s[1] < -2 || s[1] > 2 || s[2] < -2 || s[2] > 2) {
-        set_status(b.st, ST_RANGE);
-        return;
-    }
-    const uint32_t code = (uint32_t)((s[0] + 2) + 5 * (s[1] + 2) + 25 * (s[2] + 2));
-    const uint32_t e = (code << kIdxBits) | (uint32_t)j;
-    if (!(r2 < g.rc2f) && sk.n < kSkinBuf) {
-        sk.e[sk.n++] = e;
-        return;
-    }
-    if (cnt < b.cap) b.nbr[(size_t)cnt * b.n + i] = e;
-    ++cnt;
+// Minimum image of the FP32 separation d on an axis of length L (Linv = 1 / L,
+// or 0 on an open axis); s receives the number of box lengths taken off.
+// The result is the same in every mode:
+//   IMG_NONE  no pair of the block is across a face (build_cell): s = 0
+//   IMG_NEAR  rounding to the nearest integer (half to even) by adding and
+//             subtracting 1.5 2^23, right for |d / L| < 2^21, on the FP32 pipe
+//             (the conversions issue at an eighth of its rate)
+//   IMG_FAR   by conversion
+enum { IMG_NONE = 0, IMG_NEAR = 1, IMG_FAR = 2 };
+template <int MODE>
+__device__ __forceinline__ float build_image(float d, float L, float Linv, float& s) {
+    s = 0.f;
+    if (MODE == IMG_NONE) return d;
+    const float x = __fmul_rn(d, Linv);
+    s = MODE == IMG_FAR ? (float)__float2int_rn(x) : __fadd_rn(__fadd_rn(x, 0x1.8p23f), -0x1.8p23f);
+    return __fmaf_rn(-s, L, d);
+}
+__device__ __forceinline__ float build_linv(const GeoC& g, int a) { return g.per[a] ? g.Linvf[a] : 0.f; }
+// Whether an atom lies 2^19 box lengths or more from the origin on a periodic
+// axis (or nowhere).
+__device__ __forceinline__ bool build_far(const GeoC& g, float4 x) {
+    return !(fabsf(x.x) * build_linv(g, 0) < 0x1p19f) || !(fabsf(x.y) * build_linv(g, 1) < 0x1p19f) ||
+           !(fabsf(x.z) * build_linv(g, 2) < 0x1p19f);
 }
 
-__global__ void k_nbr_build(Bufs b, GeoC g, int force) {
+// Candidate test in FP32 (the FP64 unit is ~58x slower on this part): the
+// list radius carries a margin larger than the FP32 rounding of the
+// positions, so every pair closer than rc + skin is kept; the force kernels
+// test r < rc again.  The warp's lanes test candidates [0, m) (position, index
+// in w; NaN up to the next multiple of 32) against atom i at xi.
+template <int MODE>
+__device__ __forceinline__ void build_scan(const Bufs& b, const GeoC& g, int i, float4 xi,
+                                           const float4* cand, int m, uint32_t* skin,
+                                           ListState& L) {
+    const int lane = threadIdx.x & 31, full = g.full;
+    const unsigned below = (1u << lane) - 1u;
+    const float lx = build_linv(g, 0), ly = build_linv(g, 1), lz = build_linv(g, 2);
+    const float Lx = g.Lf[0], Ly = g.Lf[1], Lz = g.Lf[2], rl2 = g.rlist2f, rc2 = g.rc2f;
+    uint32_t* out = b.nbr + i;
+    for (int k = lane; k < m + lane; k += 32) {   // the warp stays together
+        const float4 xj = cand[k];
+        const int j = __float_as_int(xj.w);
+        float sx, sy, sz;
+        const float dx = build_image<MODE>(xj.x - xi.x, Lx, lx, sx);
+        const float dy = build_image<MODE>(xj.y - xi.y, Ly, ly, sy);
+        const float dz = build_image<MODE>(xj.z - xi.z, Lz, lz, sz);
+        const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+        bool ok = r2 < rl2 && j != i && (full || upper_half(dx, dy, dz));   // NaN fails
+        const unsigned any = __ballot_sync(0xffffffffu, ok);
+        if (any == 0u) continue;
+        // image codes cover shifts of -2..2 box lengths; atoms further apart than
+        // that in raw coordinates are a caller error (positions far outside the box)
+        if (MODE != IMG_NONE) {
+            const bool range = ok && !(fmaxf(fabsf(sx), fmaxf(fabsf(sy), fabsf(sz))) <= 2.f);
+            if (__any_sync(0xffffffffu, range)) {
+                if (range) set_status(b.st, ST_RANGE);
+                ok = ok && !range;
+            }
+        }
+        const bool in = ok && r2 < rc2;
+        const unsigned bi = __ballot_sync(0xffffffffu, in);
+        const unsigned bs = __ballot_sync(0xffffffffu, ok) & ~bi;
+        // exact in FP32; the integer is in the sum's low bits
+        const uint32_t code = (uint32_t)__float_as_int(sx + 5.f * sy + 25.f * sz + (62.f + 0x1p23f)) & 0x7fu;
+        const uint32_t e = (code << kIdxBits) | (uint32_t)j;
+        if (L.skin + __popc(bs) <= kSkinBuf) {
+            const int at = (in ? L.cnt : L.skin) + __popc((in ? bi : bs) & below);
+            if (in) {
+                if (at < b.cap) out[(size_t)at * b.n] = e;
+            } else if (ok) {
+                skin[at] = e;
+            }
+            L.cnt += __popc(bi);
+            L.skin += __popc(bs);
+        } else {   // the buffer is full: the rest among the in-range ones
+            const int rank = L.skin + __popc(bs & below);
+            const bool now = in || (ok && rank >= kSkinBuf);
+            const unsigned bn = __ballot_sync(0xffffffffu, now);
+            const int at = L.cnt + __popc(bn & below);
+            if (ok && !now) skin[rank] = e;
+            if (now && at < b.cap) out[(size_t)at * b.n] = e;
+            L.cnt += __popc(bn);
+            L.skin = kSkinBuf;
+        }
+    }
+}
+
+// The rare form, out of line.
+__device__ __noinline__ ListState build_scan_far(const Bufs& b, const GeoC& g, int i, float4 xi,
+                                                 const float4* cand, int m, uint32_t* skin,
+                                                 ListState L) {
+    build_scan<IMG_FAR>(b, g, i, xi, cand, m, skin, L);
+    return L;
+}
+
+// The skin pairs after the in-range ones; the list's length.
+__device__ __forceinline__ void build_finish(const Bufs& b, int i, const uint32_t* skin,
+                                             const ListState& L) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    if (lane < L.skin && L.cnt + lane < b.cap) b.nbr[(size_t)(L.cnt + lane) * b.n + i] = skin[lane];
+    if (lane == 0) {
+        const int cnt = L.cnt + L.skin;
+        if (cnt > b.cap) set_status(b.st, ST_NBR_OVERFLOW);
+        b.nnbr[i] = min(cnt, b.cap);
+    }
+    __syncwarp();   // the buffer is free for the warp's next atom
+}
+
+template <int W>
+struct BuildShared {
+    float4 cand[kBuildCand];
+    uint32_t skin[W][kSkinBuf];
+    int beg[27], off[28], wrap;   // wrap: a pair of the stencil may be across a face
+};
+// NaN candidates after m up to the next multiple of 32 (kBuildCand is one).
+__device__ __forceinline__ void build_pad(float4* cand, int m) {
+    if ((int)threadIdx.x < 32 && m + (int)threadIdx.x < ((m + 31) & ~31))
+        cand[m + threadIdx.x] = make_float4(NAN, NAN, NAN, 0.f);
+}
+
+// All pairs of an image (boxes under three cells per axis): one atom per warp.
+__global__ void __launch_bounds__(32 * kBuildWarps) k_nbr_build_all(Bufs b, GeoC g, int force) {
+    __shared__ BuildShared<kBuildWarps> sh;
     if (!need_rebuild(b.st, g, force)) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) b.st->nbr_builds += 1;
-    if (i >= b.n) return;
-    const dvec4 xi = b.x[i];
-    const float4 xif = g.brute ? xf_of(b, i) : b.xf[i];
-    int cnt = 0;
-    SkinBuf sk;
-    sk.n = 0;
-    const int img = i / g.img_n;
-    if (g.brute) {
-        for (int j = img * g.img_n; j < (img + 1) * g.img_n; ++j)
-            if (j != i) try_add_pair(b, g, i, xif, j, xf_of(b, j), cnt, sk);
-    } else {
-        const int cx = cell_coord(xi.x, g.Linv[0], g.nc[0], g.per[0]);
-        const int cy = cell_coord(xi.y, g.Linv[1], g.nc[1], g.per[1]);
-        const int cz = cell_coord(xi.z, g.Linv[2], g.nc[2], g.per[2]);
-        for (int ox = -1; ox <= 1; ++ox) {
-            const int ax = cell_step(cx, ox, g.nc[0], g.per[0]);
-            if (ax < 0) continue;
-            for (int oy = -1; oy <= 1; ++oy) {
-                const int ay = cell_step(cy, oy, g.nc[1], g.per[1]);
-                if (ay < 0) continue;
-                for (int oz = -1; oz <= 1; ++oz) {
-                    const int az = cell_step(cz, oz, g.nc[2], g.per[2]);
-                    if (az < 0) continue;
-                    const int c = cell_index(g, img, ax, ay, az);
-                    const int k1 = b.cell_start[c + 1];
-                    int k = b.cell_start[c];
-                    // four candidates' indices and positions loaded before
-                    // any is tested, so that their loads are in flight
-                    // together (the same candidates in the same order)
-                    for (; k + 4 <= k1; k += 4) {
-                        int jj[4];
-                        float4 xx[4];
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.st->nbr_builds += 1;
+    const int w = threadIdx.x >> 5;
+    // blocks of one image only, so that they share its candidates
+    const int per_img = (g.img_n + kBuildWarps - 1) / kBuildWarps;
+    const int img = blockIdx.x / per_img, a = (blockIdx.x % per_img) * kBuildWarps + w;
+    const int lo = img * g.img_n, i = lo + a;
+    const bool on = a < g.img_n;
+    const float4 xi = on ? xf_of(b, i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    ListState L;
+    for (int base = 0; base < g.img_n; base += kBuildCand) {
+        const int m = min(kBuildCand, g.img_n - base);
+        __syncthreads();
+        bool far = build_far(g, xi);
+        for (int k = threadIdx.x; k < m; k += blockDim.x) {
+            float4 x = xf_of(b, lo + base + k);
+            x.w = __int_as_float(lo + base + k);
+            sh.cand[k] = x;
+            far = far || build_far(g, x);
+        }
+        build_pad(sh.cand, m);
+        far = __syncthreads_or(far);
+        if (!on) continue;
+        if (far)
+            L = build_scan_far(b, g, i, xi, sh.cand, m, sh.skin[w], L);
+        else
+            build_scan<IMG_NEAR>(b, g, i, xi, sh.cand, m, sh.skin[w], L);
+    }
+    if (!on) return;
+    build_finish(b, i, sh.skin[w], L);
+    // the FP32 copy of x at this build, for the displacement test of k_update
+    if ((threadIdx.x & 31) == 0) b.xf[i] = xi;
+}
+
+// Cell lists: a block takes a cell, whose atoms go to its W warps in turn; the
+// candidates of the cell's stencil (27 cells, ~350 atoms) are staged once.
+template <int W>
+__device__ __forceinline__ void build_cell(const Bufs& b, const GeoC& g, int c, BuildShared<W>& sh) {
+    float4* cand = sh.cand;
+    int *beg = sh.beg, *off = sh.off;
+    const int p0 = b.cell_start[c], na = b.cell_start[c + 1] - p0;
+    if (na == 0) return;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t* skin = sh.skin[w];
+    if (w == 0) {
+        // this cell's coordinates (the inverse of cell_index), its stencil's
+        // runs in the order (x, y, z) of the offsets
+        const int img = c / g.ncell_img, r = c - img * g.ncell_img;
+        const int bvol = g.bk[0] * g.bk[1] * g.bk[2], br = r / bvol, l = r - br * bvol;
+        const int cx = (br / (g.nbk[1] * g.nbk[2])) * g.bk[0] + l / (g.bk[1] * g.bk[2]);
+        const int cy = (br / g.nbk[2]) % g.nbk[1] * g.bk[1] + l / g.bk[2] % g.bk[1];
+        const int cz = br % g.nbk[2] * g.bk[2] + l % g.bk[2];
+        int len = 0;
+        bool wrap = false;
+        if (lane < 27) {
+            const int ax = cell_step(cx, lane / 9 - 1, g.nc[0], g.per[0]);
+            const int ay = cell_step(cy, lane / 3 % 3 - 1, g.nc[1], g.per[1]);
+            const int az = cell_step(cz, lane % 3 - 1, g.nc[2], g.per[2]);
+            if (ax >= 0 && ay >= 0 && az >= 0) {
+                const int nb = cell_index(g, img, ax, ay, az);
+                beg[lane] = b.cell_start[nb];
+                len = b.cell_start[nb + 1] - beg[lane];
+                // FP32 subtraction, multiplication and rounding are monotonic:
+                // every pair's separation and image lie between those of the
+                // two cells' extremes.
+                if (len > 0) {
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) jj[u] = b.cell_atoms[k + u];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) xx[u] = b.xf[jj[u]];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (jj[u] != i) try_add_pair(b, g, i, xif, jj[u], xx[u], cnt, sk);
-                    }
-                    for (; k < k1; ++k) {
-                        const int j = b.cell_atoms[k];
-                        if (j != i) try_add_pair(b, g, i, xif, j, b.xf[j], cnt, sk);
+                    for (int a = 0; a < 3; ++a) {
+                        const float2 xi = b.cell_box[3 * (size_t)c + a];
+                        const float2 xj = b.cell_box[3 * (size_t)nb + a];
+                        const float li = build_linv(g, a);
+                        float s0, s1;
+                        const float d0 = build_image<IMG_FAR>(xj.x - xi.y, g.Lf[a], li, s0);
+                        const float d1 = build_image<IMG_FAR>(xj.y - xi.x, g.Lf[a], li, s1);
+                        wrap = wrap || s0 != 0.f || s1 != 0.f;
+                        // half list: a run whose atoms all lie below this
+                        // cell's (the layer under it, as a rule) has no pair in
+                        // the upper half space
+                        if (a == 2 && !g.full && s0 == s1 && d0 <= d1 && d1 < 0.f) len = 0;
                     }
                 }
             }
         }
+        wrap = __any_sync(0xffffffffu, wrap);
+        if (lane == 0) sh.wrap = wrap;
+        int s = len;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += x;
+        }
+        if (lane < 27) off[lane + 1] = s;
+        if (lane == 0) off[0] = 0;
     }
-    for (int q = 0; q < sk.n; ++q) {   // the skin pairs after the in-range ones
-        if (cnt < b.cap) b.nbr[(size_t)cnt * b.n + i] = sk.e[q];
-        ++cnt;
+    __syncthreads();
+    const int total = off[27];
+    // candidates [from, from + kBuildCand) of the stencil; whether any is far
+    auto stage = [&](int from) {
+        bool far = false;
+        for (int r = w; r < 27; r += W) {
+            const int lo = max(off[r], from), hi = min(off[r + 1], from + kBuildCand);
+            for (int k = lo + lane; k < hi; k += 32) {
+                const float4 x = b.xs[beg[r] + k - off[r]];
+                cand[k - from] = x;
+                far = far || build_far(g, x);
+            }
+        }
+        build_pad(cand, min(kBuildCand, total - from));
+        return __syncthreads_or(far) != 0;
+    };
+    const bool once = total <= kBuildCand, wrap = sh.wrap != 0;
+    bool far = once ? stage(0) : false;
+    for (int a0 = 0; a0 < na; a0 += W) {
+        const bool on = a0 + w < na;
+        const float4 xi = b.xs[p0 + min(a0 + w, na - 1)];
+        const int i = __float_as_int(xi.w);
+        ListState L;
+        for (int from = 0; from < total; from += kBuildCand) {
+            if (!once) {   // a crowded stencil: piece by piece for each set of atoms
+                __syncthreads();
+                far = stage(from);
+            }
+            if (!on) continue;
+            const int m = min(kBuildCand, total - from);
+            if (!wrap)
+                build_scan<IMG_NONE>(b, g, i, xi, cand, m, skin, L);
+            else if (far || build_far(g, xi))
+                L = build_scan_far(b, g, i, xi, cand, m, skin, L);
+            else
+                build_scan<IMG_NEAR>(b, g, i, xi, cand, m, skin, L);
+        }
+        if (on) build_finish(b, i, skin, L);
     }
-    if (cnt > b.cap) {
-        set_status(b.st, ST_NBR_OVERFLOW);
-        cnt = b.cap;
+}
+// Blocks of `cells` cells: one (the usual density), or 32 W where most cells
+// are empty (a cluster in a large open box), of which the block takes the
+// occupied ones.
+template <int W>
+__global__ void __launch_bounds__(32 * W) k_nbr_build(Bufs b, GeoC g, int force, int cells) {
+    __shared__ BuildShared<W> sh;
+    if (!need_rebuild(b.st, g, force)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.st->nbr_builds += 1;
+    if (cells == 1) {
+        build_cell<W>(b, g, blockIdx.x, sh);
+        return;
     }
-    b.nnbr[i] = cnt;
-    // the FP32 copy of x at this build, for the displacement test of k_update
-    // (with cell lists k_cell_count wrote it already)
-    if (g.brute) b.xf[i] = make_float4((float)xi.x, (float)xi.y, (float)xi.z, 0.f);
+    const int c = blockIdx.x * cells + threadIdx.x;
+    int occupied = c < b.ncell && b.cell_start[c + 1] > b.cell_start[c] ? (int)threadIdx.x : -1;
+    for (;;) {   // the highest cell left
+        __shared__ int top;
+        __syncthreads();
+        if (threadIdx.x == 0) top = -1;
+        __syncthreads();
+        if (occupied >= 0) atomicMax(&top, occupied);
+        __syncthreads();
+        if (top < 0) return;
+        build_cell<W>(b, g, blockIdx.x * cells + top, sh);
+        if (occupied == top) occupied = -1;
+    }
 }
 
 // ---------------------------------------------------------------------------
