@@ -534,7 +534,7 @@ void launch_forces(fire_handle* h, const GeoC& g, cudaStream_t s, bool confirm_p
         k_embed<<<h->b.nb_embed, kElemBlock, 0, s>>>(h->b);
         k_force_rgl<<<h->b.nb_force, kForceBlock, 0, s>>>(h->b, g);
     } else if (h->pot.kind == FIRE_POT_SW) {
-        k_force_sw<<<h->b.nb_force, kForceBlock, 0, s>>>(h->b, h->potc, g);
+        k_force_sw<<<h->b.nb_force, kSwBlock, 0, s>>>(h->b, h->potc, g);
     } else {
         force_lj(h->b, h->potc, g, s);
     }
@@ -988,6 +988,7 @@ static bool fill_potc(fire_handle* h) {
         c.sw_sigma = pot->sigma;
         c.sw_rc = pot->sw_a * pot->sigma;
         c.rc2 = c.sw_rc * c.sw_rc;
+        c.sw_tmax = 600.0 / (pot->sigma * std::max(1.0, pot->sw_gamma));
         c.sw_A = pot->sw_A;
         c.sw_B = pot->sw_B;
         c.sw_p = pot->sw_p;
@@ -1212,7 +1213,8 @@ static fire_status init_handle(fire_handle_t** hp, const fire_system_t* sys,
     // the device on small systems (auto_tpa)
     h->sms = sms;
     b.tpa = tpa_form(*pot) ? auto_tpa(*pot, h->n, sms) : 1;
-    b.nb_force = ceil_div((long long)h->n * b.tpa, kForceBlock);
+    b.nb_force = pot->kind == FIRE_POT_SW ? ceil_div(h->n, kSwBlock)
+                                          : ceil_div((long long)h->n * b.tpa, kForceBlock);
     // blocks per SM of the embedding and the reductions, measured on 1M
     // atoms: embedding 16.4 / 14.3 / 18.4 / 22.1 us at 2 / 4 / 8 / 16;
     // reductions + control 53 / 51 / 57 / 70 us at 1 / 2 / 4 / 8
@@ -2039,7 +2041,7 @@ fire_status fire_profile_stages(fire_handle_t* h, const double* pos, const doubl
         else if (tab) force_ff<false>(h->b, h->potc, g, s);
         else if (rgl && f32) force32(h->b, h->potc, g, s);
         else if (rgl) k_force_rgl<<<h->b.nb_force, kForceBlock, 0, s>>>(h->b, g);
-        else if (h->pot.kind == FIRE_POT_SW) k_force_sw<<<h->b.nb_force, kForceBlock, 0, s>>>(h->b, h->potc, g);
+        else if (h->pot.kind == FIRE_POT_SW) k_force_sw<<<h->b.nb_force, kSwBlock, 0, s>>>(h->b, h->potc, g);
         else force_lj(h->b, h->potc, g, s);
         cudaEventRecord(ev[4], s);
         // the control step runs in the last block of the reductions' launch

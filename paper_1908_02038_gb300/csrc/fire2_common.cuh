@@ -63,7 +63,7 @@ struct PotC {
     // LJ
     double eps, sigma2, lj_shift;
     // SW (eps above): sigma, a sigma, and the published dimensionless set
-    double sw_sigma, sw_rc, sw_A, sw_B, sw_p, sw_q, sw_lambda, sw_gamma;
+    double sw_sigma, sw_rc, sw_tmax, sw_A, sw_B, sw_p, sw_q, sw_lambda, sw_gamma;
     int sw_pi, sw_qi;      // sw_p, sw_q as small non-negative integers, or -1
     // RGL
     double A, xi2, p, q2, r0inv, p_r0, q2_r0, rs, rc, winv;
@@ -99,6 +99,15 @@ __device__ __forceinline__ double max_nonneg(double a, double b) {
 }
 __device__ __forceinline__ double abs_bits(double x) {
     return __longlong_as_double(__double_as_longlong(x) & 0x7fffffffffffffffll);
+}
+
+__device__ __forceinline__ double min_nonneg(double a, double b) {
+    return __longlong_as_double(min(__double_as_longlong(a), __double_as_longlong(b)));
+}
+// a < b of non-negative doubles (NaN fails against a number: its pattern is
+// above every number's).
+__device__ __forceinline__ bool below_nonneg(double a, double b) {
+    return __double_as_longlong(a) < __double_as_longlong(b);
 }
 
 // FP64 instructions issue at 1/58 of the FP32 rate on this part and a warp

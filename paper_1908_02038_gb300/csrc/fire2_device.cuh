@@ -831,59 +831,67 @@ __global__ void __launch_bounds__(kForceBlock) k_force_rgl(Bufs b, GeoC g) {
     f_add(b, i, fx, fy, fz);
 }
 
-// Stillinger-Weber, one pass over the full list (IEEE FP64): the pair term
-// from both ends (half its energy to each atom, its force on i), then the
+// Stillinger-Weber, one pass over the full list (FP64): the pair term from
+// both ends (half its energy to each atom, its force on i), then the
 // three-body terms centred on i for every pair j < k of neighbours within
 // a sigma, their gradients added to i here and to j and k by FP64 atomics:
 //   h = lambda eps (c + 1/3)^2 e_j e_k,  e = exp(gamma sigma / (r - a sigma)),
 //   dh/dx_j = dh/dr_j u_j + dh/dc (u_k - c u_j) / r_j   (u = unit vectors).
-// Everything that depends on one neighbour only (u, 1/r, e, and
-// gamma sigma / (r - a sigma)^2 = -d ln e / dr) is computed once per
-// neighbour, so the triplet loop has no division or exponential.
+// The kernel is bound by the FP64 pipe (1/58 of the FP32 rate), so it keeps
+// its FP64 instructions few.  Everything that depends on one neighbour only
+// (u, 1/r, e, gamma sigma / (r - a sigma)^2 = -d ln e / dr) is computed once
+// per neighbour, without a division, square root or library exponential.
+// With q = lambda eps (c + 1/3) e_j e_k (dh/dc = 2 q, h = q (c + 1/3)) a
+// neighbour's gradient sums to
+//   G_j = -(gd_j S_j + (2 / r_j) C_j) u_j + (2 / r_j) V_j,
+//   S_j = sum_k h, C_j = sum_k q c, V_j = sum_k q u_k,
+// so a triplet costs 17 FP64 instructions (40 with its gradients formed one by
+// one) and each neighbour three atomics (six per triplet before).
+// 32,763-atom Si slab at its displaced start (up to 9 neighbours inside): 208 ->
+// 127 us, 1,394 FP64 instructions per warp against 2,273.
+// Blocks of one warp: 1,024 warps over 152 SMs come out evenly (7 against 6.7
+// on average; with blocks of 128 some SMs had 8 and some 4).
+constexpr int kSwBlock = 32;
 constexpr int kSwMax = 32;   // neighbours within a sigma per atom (a solid has 4)
 
 // x^e for the SW exponents: repeated squaring when e is a small non-negative
 // integer (ei >= 0), pow() otherwise.
 __device__ __forceinline__ double sw_pow(double x, double e, int ei) {
     if (ei < 0) return pow(x, e);
-    double r = 1.0, b = x;
-    for (int n = ei; n > 0; n >>= 1) {
-        if (n & 1) r *= b;
-        b *= b;
+    if (ei == 0) return 1.0;
+    double r = 0.0;
+    bool have = false;
+    for (int n = ei;;) {
+        if (n & 1) {
+            r = have ? r * x : x;
+            have = true;
+        }
+        n >>= 1;
+        if (n == 0) return r;
+        x *= x;
     }
-    return r;
 }
 
-// Pair term phi2(r) and phi2'(r) from invr = 1/r and t = 1/(r - a sigma).
-__device__ __forceinline__ void sw_pair(const PotC& P, double invr, double t, double& e2,
-                                        double& de2) {
-    const double s = P.sw_sigma;
-    const double sr = s * invr;
-    const double bp = P.sw_B * sw_pow(sr, P.sw_p, P.sw_pi), bq = sw_pow(sr, P.sw_q, P.sw_qi);
-    const double ex = exp(s * t);
-    e2 = P.sw_A * P.eps * (bp - bq) * ex;
-    de2 = P.sw_A * P.eps * ex * ((-P.sw_p * bp + P.sw_q * bq) * invr - (bp - bq) * s * t * t);
-}
-
-__global__ void __launch_bounds__(kForceBlock) k_force_sw(Bufs b, PotC P, GeoC g) {
+__global__ void __launch_bounds__(kSwBlock) k_force_sw(Bufs b, PotC P, GeoC g) {
     __shared__ double3 tbl[125];
+    __shared__ double etab[kExpTableSize];
     __shared__ double red[32];
     if (b.st->done) return;
     fill_shift_table(tbl, g);
+    for (int t = threadIdx.x; t < kExpTableSize; t += blockDim.x) etab[t] = b.exp_table[t];
     __syncthreads();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     double e_i = 0.0;
     if (i < b.n) {
         const dvec4 xi = b.x[i];
         const int m = b.nnbr[i];
-        // per neighbour: unit vector, 1/r, exp(gamma sigma / (r - a sigma)) and
-        // gamma sigma / (r - a sigma)^2, so the triplet loop only multiplies
         int nj[kSwMax];
         double ux[kSwMax], uy[kSwMax], uz[kSwMax], ir[kSwMax], eg[kSwMax], gd[kSwMax];
+        double S[kSwMax], C[kSwMax], Vx[kSwMax], Vy[kSwMax], Vz[kSwMax];
         int cnt = 0;
         double fx = 0.0, fy = 0.0, fz = 0.0;
-        const double gs = P.sw_gamma * P.sw_sigma, rc = P.sw_rc;
-        const double le = P.sw_lambda * P.eps;
+        const double s = P.sw_sigma, gs = P.sw_gamma * P.sw_sigma;
+        const double le = P.sw_lambda * P.eps, ae = P.sw_A * P.eps;
         for (int k = 0; k < m; ++k) {
             const uint32_t e = b.nbr[(size_t)k * b.n + i];
             const int j = (int)(e & kIdxMask);
@@ -897,25 +905,31 @@ __global__ void __launch_bounds__(kForceBlock) k_force_sw(Bufs b, PotC P, GeoC g
                 dz -= sh.z;
             }
             const double r2 = dx * dx + dy * dy + dz * dz;
-            if (!(r2 < P.rc2)) continue;
-            const double invr = rsqrt_newton(r2);   // r2 > 0: list pairs are distinct atoms
+            if (!below_nonneg(r2, P.rc2)) continue;
+            const double invr = rsqrt_f64(r2);   // r2 > 0: list pairs are distinct atoms
             const double r = r2 * invr;
-            const double t = 1.0 / (r - rc);
-            double e2, de2;
-            sw_pair(P, invr, t, e2, de2);
-            e_i += 0.5 * e2;
-            const double w = de2 * invr;   // force on i from the pair: +phi2'(r) d / r
+            // t = 1 / (r - a sigma) < 0, no further than where the exponentials
+            // are e^-600 (exp_tang's range; exactly at the cut-off t = -sw_tmax)
+            const double t = -min_nonneg(rcp_f64(abs_bits(r - P.sw_rc)), P.sw_tmax);
+            const double x1 = s * t, sr = s * invr;
+            const double bp = P.sw_B * sw_pow(sr, P.sw_p, P.sw_pi), bq = sw_pow(sr, P.sw_q, P.sw_qi);
+            const double aex = ae * exp_tang(x1, P.ex, etab), d = bp - bq;
+            e_i = fma(0.5 * aex, d, e_i);
+            // force on i from the pair: phi2'(r) d / r
+            const double w = aex * fma(-d, x1 * t, (P.sw_q * bq - P.sw_p * bp) * invr) * invr;
             fx += w * dx;
             fy += w * dy;
             fz += w * dz;
             if (cnt < kSwMax) {
+                const double x2 = gs * t;
                 nj[cnt] = j;
                 ux[cnt] = dx * invr;
                 uy[cnt] = dy * invr;
                 uz[cnt] = dz * invr;
                 ir[cnt] = invr;
-                eg[cnt] = exp(gs * t);
-                gd[cnt] = gs * t * t;
+                eg[cnt] = exp_tang(x2, P.ex, etab);
+                gd[cnt] = x2 * t;
+                S[cnt] = C[cnt] = Vx[cnt] = Vy[cnt] = Vz[cnt] = 0.0;
             }
             ++cnt;
         }
@@ -923,30 +937,35 @@ __global__ void __launch_bounds__(kForceBlock) k_force_sw(Bufs b, PotC P, GeoC g
             set_status(b.st, ST_CROWDED);
             cnt = kSwMax;
         }
-        for (int p = 0; p < cnt; ++p)
+        double sum = 0.0;   // of S: every h twice
+        for (int p = 0; p < cnt; ++p) {
+            const double upx = ux[p], upy = uy[p], upz = uz[p], lep = le * eg[p];
+            double Sp = S[p], Cp = C[p], px = Vx[p], py = Vy[p], pz = Vz[p];
             for (int q = p + 1; q < cnt; ++q) {
-                const double ujx = ux[p], ujy = uy[p], ujz = uz[p];
-                const double ukx = ux[q], uky = uy[q], ukz = uz[q];
-                const double cs = ujx * ukx + ujy * uky + ujz * ukz;   // cos theta_jik
+                const double uqx = ux[q], uqy = uy[q], uqz = uz[q];
+                const double cs = upx * uqx + upy * uqy + upz * uqz;   // cos theta_jik
                 const double wv = cs + 1.0 / 3.0;
-                const double ee = eg[p] * eg[q];
-                const double h = le * wv * wv * ee;
-                e_i += h;
-                const double dh_dc = 2.0 * le * wv * ee;
-                const double dj = -h * gd[p], dk = -h * gd[q];
-                const double cj = dh_dc * ir[p], ck = dh_dc * ir[q];
-                const double gjx = dj * ujx + cj * (ukx - cs * ujx);
-                const double gjy = dj * ujy + cj * (uky - cs * ujy);
-                const double gjz = dj * ujz + cj * (ukz - cs * ujz);
-                const double gkx = dk * ukx + ck * (ujx - cs * ukx);
-                const double gky = dk * uky + ck * (ujy - cs * uky);
-                const double gkz = dk * ukz + ck * (ujz - cs * ukz);
-                fx += gjx + gkx;
-                fy += gjy + gky;
-                fz += gjz + gkz;
-                f_add(b, nj[p], -gjx, -gjy, -gjz);
-                f_add(b, nj[q], -gkx, -gky, -gkz);
+                const double qv = wv * (lep * eg[q]), h = qv * wv;
+                Sp += h;
+                S[q] += h;
+                Cp = fma(qv, cs, Cp);
+                C[q] = fma(qv, cs, C[q]);
+                px = fma(qv, uqx, px);
+                py = fma(qv, uqy, py);
+                pz = fma(qv, uqz, pz);
+                Vx[q] = fma(qv, upx, Vx[q]);
+                Vy[q] = fma(qv, upy, Vy[q]);
+                Vz[q] = fma(qv, upz, Vz[q]);
             }
+            sum += Sp;
+            const double c2 = 2.0 * ir[p], a = -fma(gd[p], Sp, c2 * Cp);
+            const double gx = fma(a, upx, c2 * px), gy = fma(a, upy, c2 * py), gz = fma(a, upz, c2 * pz);
+            fx += gx;
+            fy += gy;
+            fz += gz;
+            f_add(b, nj[p], -gx, -gy, -gz);
+        }
+        e_i = fma(0.5, sum, e_i);
         f_add(b, i, fx, fy, fz);
         if (b.eatom) b.eatom[i] = e_i;
     }

@@ -91,26 +91,10 @@ __device__ __forceinline__ double na_exp(const NaPot& P, double x, const double*
     return FAST ? fire2::exp_tang(x, P.ex, tab) : exp(x);
 }
 
-// 1/sqrt(x) for x in (1e-30, 1e30): the FP32 estimate y0 (conversions on the
-// integer pipes) and one step of third order, y0 + y0 e (1/2 + 3/8 e) with
-// e = 1 - x y0^2 ~ 2^-22: off by 5/16 e^3 ~ 2^-67.
-__device__ __forceinline__ double na_rsqrt(double x) {
-    const double y0 = fire2::f32_to_f64(rsqrtf(fire2::f64_to_f32_trunc(x)));
-    const double e = fma(-x, y0 * y0, 1.0);
-    return fma(y0, fma(e, 0.375, 0.5) * e, y0);
-}
-// Outside that range.
-__device__ __noinline__ double na_rsqrt_any(double x) { return 1.0 / sqrt(x); }
-
 // r and 1/r of a pair.
 __device__ __forceinline__ void na_radius(double r2, double& r, double& rinv) {
-    const bool in = fire2::ff_range(r2);   // 2^-60 .. 2^60, by the bit pattern
-    rinv = in ? na_rsqrt(r2) : 0.0;
-    r = r2 * rinv;
-    if (!in) {
-        rinv = na_rsqrt_any(r2);
-        r = r2 > 0.0 ? r2 * rinv : 0.0;
-    }
+    rinv = fire2::rsqrt_f64(r2);
+    r = __double_as_longlong(r2) > 0 ? r2 * rinv : 0.0;
 }
 
 // RGL pair terms: phi = A e^{-p s} S, g = xi^2 e^{-2q s} S, s = r/r0 - 1, with
@@ -245,12 +229,6 @@ __device__ __forceinline__ double na_sep(const double* __restrict__ pos, const N
     return d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
 }
 
-// a < b of non-negative doubles on the integer pipes (NaN fails: its pattern is
-// above every number's).
-__device__ __forceinline__ bool na_below(double a, double b) {
-    return __double_as_longlong(a) < __double_as_longlong(b);
-}
-
 // Pass 1 (RGL): F'(rho_i) and the per-atom energy, all-pairs.
 // LJ: the whole evaluation (forces and energy) in this one pass.
 template <int A, bool RGL, bool FAST>
@@ -275,7 +253,7 @@ __global__ void __launch_bounds__(kBlock) k_na_pass1(const double* __restrict__ 
     na_walk<A>(pos, n, P, i0, tile, list[w], [&](int u, int j) {
         double d[3];
         const double r2 = na_sep(pos, P, x[u], j, d);
-        if (!na_below(r2, P.rc2)) return;
+        if (!fire2::below_nonneg(r2, P.rc2)) return;
         if (RGL) {
             double r, rinv, phi, dphi, g, dg;
             na_radius(r2, r, rinv);
@@ -336,7 +314,7 @@ __global__ void __launch_bounds__(kBlock) k_na_pass2(const double* __restrict__ 
     na_walk<A>(pos, n, P, i0, tile, list[w], [&](int u, int j) {
         double d[3];
         const double r2 = na_sep(pos, P, x[u], j, d);
-        if (!na_below(r2, P.rc2)) return;
+        if (!fire2::below_nonneg(r2, P.rc2)) return;
         double r, rinv, phi, dphi, g, dg;
         na_radius(r2, r, rinv);
         na_rgl_pair<FAST>(P, r, tab, phi, dphi, g, dg);

@@ -409,6 +409,28 @@ __device__ __forceinline__ bool ff_range(double d) {
     return bits > 0x3C30000000000000ll && bits < 0x43B0000000000000ll;
 }
 
+#ifdef __CUDACC__
+// 1/sqrt(x), x >= 0, in FP64 without a library call: the FP32 estimate y0 (the
+// conversions on the integer pipes) and one step of third order,
+// y0 + y0 e (1/2 + 3/8 e) with e = 1 - x y0^2 ~ 2^-22, off by 5/16 e^3 ~ 2^-67:
+// five FP64 instructions.  Outside ff_range the IEEE operations.
+static __device__ __noinline__ double rsqrt_f64_any(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double rsqrt_f64(double x) {
+    if (!ff_range(x)) return rsqrt_f64_any(x);
+    const double y0 = f32_to_f64(rsqrtf(f64_to_f32_trunc(x)));
+    const double e = fma(-x, y0 * y0, 1.0);
+    return fma(y0, fma(e, 0.375, 0.5) * e, y0);
+}
+// 1/x, x >= 0, the same way (y0 + y0 (e + e^2), e = 1 - x y0): three.
+static __device__ __noinline__ double rcp_f64_any(double x) { return 1.0 / x; }
+__device__ __forceinline__ double rcp_f64(double x) {
+    if (!ff_range(x)) return rcp_f64_any(x);
+    const double y0 = f32_to_f64(__frcp_rn(f64_to_f32_trunc(x)));
+    const double e = fma(-x, y0, 1.0);
+    return fma(y0, fma(e, e, e), y0);
+}
+#endif  // __CUDACC__
+
 // d with ff_range(d) as a float pair without an FP64 instruction: hi is d
 // truncated to 24 significant bits (f64_to_f32_trunc), lo the remaining 29
 // bits of the significand, rem 2^(e - 52), rounded to 24 bits
