@@ -34,8 +34,12 @@ struct GradState {
     int* nnbr = nullptr;
     double *rho = nullptr, *F1 = nullptr, *F2 = nullptr, *drho = nullptr, *dq = nullptr;
     double* part = nullptr;        // 9 x nb block partials
-    double* vec = nullptr;         // 4 work vectors of 3N (r, p, Ap, lambda)
-    double* pcache = nullptr;      // HVP pair coefficients, 3 x cap x N (implicit gradient)
+    dvec4* vec = nullptr;          // 4 work vectors of N quads (r, p, Ap, lambda)
+    // HVP pair cache of the implicit gradient (GradBufs): per slot and per atom
+    dvec4 *dw = nullptr, *wsum = nullptr;
+    double2* fa = nullptr;
+    double *dot = nullptr, *dc = nullptr;
+    int* nin = nullptr;
     size_t pcache_slots = 0;
     CgState* cs = nullptr;         // device scalars of the CG solve
     CgState* h_cs = nullptr;       // pinned copy
@@ -478,21 +482,21 @@ void force32(const Bufs& b, const PotC& P, const GeoC& g, cudaStream_t s) {
     }
 }
 
-// The two passes of the cached Hessian-vector product, TPA threads per atom.
+// The two passes of the cached Hessian-vector product, TPA threads per atom,
+// ending with alpha of the conjugate-gradient step.
+inline int hvp_grid(int n, int tpa) { return ceil_div((long long)n * tpa, kForceBlock); }
 template <int TPA>
-void hvp_cached_t(const GradBufs& b, const double* u, double* hu, const int* skip, int n,
-                  cudaStream_t s) {
-    const int nb = ceil_div((long long)n * TPA, kForceBlock);
-    k_g_hvp1c<TPA><<<nb, kForceBlock, 0, s>>>(b, u, skip);
-    k_g_hvp2c<TPA><<<nb, kForceBlock, 0, s>>>(b, u, hu, skip);
+void hvp_cached_t(const GradBufs& b, const dvec4* p, dvec4* Ap, CgState* cs, cudaStream_t s) {
+    const int nb = hvp_grid(b.n, TPA);
+    k_g_hvp1c<TPA><<<nb, kForceBlock, 0, s>>>(b, p, &cs->done);
+    k_g_hvp2c<TPA><<<nb, kForceBlock, 0, s>>>(b, p, Ap, cs);
 }
-void hvp_cached(const GradBufs& b, const double* u, double* hu, const int* skip, int tpa, int n,
-                cudaStream_t s) {
+void hvp_cached(const GradBufs& b, const dvec4* p, dvec4* Ap, CgState* cs, int tpa, cudaStream_t s) {
     switch (tpa) {
-    case 8: hvp_cached_t<8>(b, u, hu, skip, n, s); break;
-    case 4: hvp_cached_t<4>(b, u, hu, skip, n, s); break;
-    case 2: hvp_cached_t<2>(b, u, hu, skip, n, s); break;
-    default: hvp_cached_t<1>(b, u, hu, skip, n, s);
+    case 8: hvp_cached_t<8>(b, p, Ap, cs, s); break;
+    case 4: hvp_cached_t<4>(b, p, Ap, cs, s); break;
+    case 2: hvp_cached_t<2>(b, p, Ap, cs, s); break;
+    default: hvp_cached_t<1>(b, p, Ap, cs, s);
     }
 }
 
@@ -1325,7 +1329,8 @@ void fire_destroy(fire_handle_t* h) {
     {
         GradState& gs = h->grad;
         void* gp[] = {gs.x, gs.xf, gs.nbr, gs.nnbr, gs.rho, gs.F1, gs.F2, gs.drho,
-                      gs.dq, gs.part, gs.vec, gs.pcache, gs.cs, gs.st};
+                      gs.dq, gs.part, gs.vec, gs.dw, gs.wsum, gs.fa, gs.dot, gs.dc, gs.nin,
+                      gs.cs, gs.st};
         for (void* p : gp)
             if (p) cudaFree(p);
         if (gs.h_part) cudaFreeHost(gs.h_part);
@@ -1643,8 +1648,9 @@ static fire_status grad_setup(fire_handle* h, const double* d_pos, const double 
         CK(h, cudaMalloc(&gs.nnbr, (size_t)n * sizeof(int)));
         for (double** p : {&gs.rho, &gs.F1, &gs.F2, &gs.drho, &gs.dq})
             CK(h, cudaMalloc(p, (size_t)n * sizeof(double)));
-        CK(h, cudaMalloc(&gs.part, (size_t)9 * gs.nb * sizeof(double)));
-        CK(h, cudaMalloc(&gs.vec, (size_t)4 * 3 * n * sizeof(double)));
+        // 9 rows of nb, or 4 of the cached HVP's blocks
+        CK(h, cudaMalloc(&gs.part, (size_t)std::max(9 * gs.nb, 4 * hvp_grid(n, kMaxHvpTpa)) * sizeof(double)));
+        CK(h, cudaMalloc(&gs.vec, (size_t)4 * n * sizeof(dvec4)));
         CK(h, cudaMallocHost(&gs.h_part, (size_t)9 * gs.nb * sizeof(double)));
         CK(h, cudaMalloc(&gs.st, sizeof(DevState)));
     }
@@ -1841,52 +1847,53 @@ fire_status fire_rgl_implicit_grad_dev(fire_handle_t* h, const double* d_pos, co
     GradBufs b;
     fire_status st = grad_setup(h, d_pos, box, theta, s, &g, &pc, &b);
     if (st != FIRE_OK) return st;
-    const int n = h->n, m = 3 * n;
+    const int n = h->n;
     // the positions are fixed for the whole solve: cache the pair
-    // coefficients of the HVP and the separations once (6 doubles per slot)
+    // coefficients of the HVP and the separations once (7 doubles per slot)
+    GradState& gs = h->grad;
     {
-        GradState& gs = h->grad;
         const size_t slots = (size_t)gs.cap * n;
         if (slots > gs.pcache_slots) {
-            cudaFree(gs.pcache);
-            gs.pcache = nullptr;
             gs.pcache_slots = 0;
-            CK(h, cudaMalloc(&gs.pcache, 6 * slots * sizeof(double)));
+            for (void** q : {(void**)&gs.dw, (void**)&gs.fa, (void**)&gs.dot, (void**)&gs.wsum,
+                             (void**)&gs.dc, (void**)&gs.nin}) {
+                cudaFree(*q);
+                *q = nullptr;
+            }
+            CK(h, cudaMalloc(&gs.dw, slots * sizeof(dvec4)));
+            CK(h, cudaMalloc(&gs.fa, slots * sizeof(double2)));
+            CK(h, cudaMalloc(&gs.dot, slots * sizeof(double)));
+            CK(h, cudaMalloc(&gs.wsum, (size_t)n * sizeof(dvec4)));
+            CK(h, cudaMalloc(&gs.dc, (size_t)n * sizeof(double)));
+            CK(h, cudaMalloc(&gs.nin, (size_t)n * sizeof(int)));
             gs.pcache_slots = slots;
         }
-        double* w1 = gs.pcache;
-        double* fsc = w1 + slots;
-        double* a2 = fsc + slots;
-        double* dcx = a2 + slots;
-        double* dcy = dcx + slots;
-        double* dcz = dcy + slots;
+        b.dw = gs.dw;
+        b.fa = gs.fa;
+        b.dot = gs.dot;
+        b.wsum = gs.wsum;
+        b.dc = gs.dc;
+        b.nin = gs.nin;
         GeoL L{{box[0], box[1], box[2]}};
-        k_g_pair_cache<<<gs.nb, kForceBlock, 0, s>>>(b, pc, L, h->b.exp_table, w1, fsc, a2,
-                                                      dcx, dcy, dcz);
+        k_g_pair_cache<<<gs.nb, kForceBlock, 0, s>>>(b, pc, L, h->b.exp_table);
         CK(h, cudaGetLastError());
-        b.w1 = w1;
-        b.fsc = fsc;
-        b.a2 = a2;
-        b.dcx = dcx;
-        b.dcy = dcy;
-        b.dcz = dcz;
     }
-    const size_t bytes = (size_t)m * sizeof(double);
-    double* r = h->grad.vec;
-    double* p = r + m;
-    double* Ap = p + m;
-    double* lam = Ap + m;
-    const int nb = std::min(h->grad.nb, 1024);
-    CK(h, cudaMemcpyAsync(r, d_g, bytes, cudaMemcpyDeviceToDevice, s));
-    if ((st = project_out_translations(h, r, s)) != FIRE_OK) return st;
-    CK(h, cudaMemsetAsync(lam, 0, bytes, s));
-    CK(h, cudaMemcpyAsync(p, r, bytes, cudaMemcpyDeviceToDevice, s));
+    const size_t bytes = (size_t)3 * n * sizeof(double);
+    dvec4* r = gs.vec;
+    dvec4* p = r + n;
+    dvec4* Ap = p + n;
+    dvec4* lam = Ap + n;
+    double* row = reinterpret_cast<double*>(Ap);   // row-major copies, before and after the solve
+    const int ne = ceil_div(n, kElemBlock), nb = std::min(ne, 4 * h->sms);
+    CK(h, cudaMemcpyAsync(row, d_g, bytes, cudaMemcpyDeviceToDevice, s));
+    if ((st = project_out_translations(h, row, s)) != FIRE_OK) return st;
+    k_cg_load<<<ne, kElemBlock, 0, s>>>(n, row, r, p, lam);
+    CK(h, cudaGetLastError());
     double rr = 0.0;
-    if ((st = dev_dot(h, r, r, &rr, s)) != FIRE_OK) return st;
+    if ((st = dev_dot(h, row, row, &rr, s)) != FIRE_OK) return st;
     // the iterations run on device scalars (CgState): the host queues
     // kCgBatch of them at a time and reads the state once per batch; the
     // kernels of iterations after the stop return at once
-    GradState& gs = h->grad;
     if (!gs.cs) {
         CK(h, cudaMalloc(&gs.cs, sizeof(CgState)));
         CK(h, cudaMallocHost(&gs.h_cs, sizeof(CgState)));
@@ -1902,10 +1909,11 @@ fire_status fire_rgl_implicit_grad_dev(fire_handle_t* h, const double* d_pos, co
     *gs.h_cs = c0;
     CK(h, cudaMemcpyAsync(gs.cs, gs.h_cs, sizeof(CgState), cudaMemcpyHostToDevice, s));
     GeoL L{{box[0], box[1], box[2]}};
-    const int* skip = &gs.cs->done;
-    // the cached HVP passes are FP64 pair loops like the force passes: split
-    // each atom's list over several threads on small systems
-    const int tpa = tpa_for(n, h->sms, 1024, kMaxHvpTpa);
+    // split each atom's list over several threads on small systems: 256 threads
+    // per SM keep the FP64 pipe busy, and every doubling adds a step to the
+    // groups' FP64 sums (31,999 atoms, 199 iterations: 16.2 / 16.5 / 20.8 ms at
+    // 2 / 4 / 8 threads per atom)
+    const int tpa = tpa_for(n, h->sms, 256, kMaxHvpTpa);
     constexpr int kCgBatch = 16;
     int done = c0.done;
     // the kCgBatch iterations between two reads of the state form one CUDA
@@ -1915,14 +1923,9 @@ fire_status fire_rgl_implicit_grad_dev(fire_handle_t* h, const double* d_pos, co
         CK(h, cudaStreamSynchronize(s));   // the set-up above is complete before the graph runs
         st = capture_plain(h, &batch, [&](cudaStream_t cs) {
             for (int c = 0; c < kCgBatch; ++c) {
-                hvp_cached(b, p, Ap, skip, tpa, n, cs);
-                k_cg_colsum<<<nb, kElemBlock, 0, cs>>>(n, gs.cs, Ap, gs.part);
-                k_cg_means<<<1, kElemBlock, 0, cs>>>(gs.cs, gs.part, nb, n);
-                k_cg_project_dot<<<nb, kElemBlock, 0, cs>>>(n, gs.cs, Ap, p, gs.part);
-                k_cg_alpha<<<1, kElemBlock, 0, cs>>>(gs.cs, gs.part, nb);
-                k_cg_step<<<nb, kElemBlock, 0, cs>>>(m, gs.cs, p, Ap, lam, r, gs.part);
-                k_cg_beta<<<1, kElemBlock, 0, cs>>>(gs.cs, gs.part, nb);
-                k_cg_dir<<<nb, kElemBlock, 0, cs>>>(m, gs.cs, r, p);
+                hvp_cached(b, p, Ap, gs.cs, tpa, cs);
+                k_cg_step<<<nb, kElemBlock, 0, cs>>>(n, gs.cs, p, Ap, lam, r, gs.part);
+                k_cg_dir<<<nb, kElemBlock, 0, cs>>>(n, gs.cs, r, p);
             }
         });
         if (st != FIRE_OK) return st;
@@ -1942,12 +1945,13 @@ fire_status fire_rgl_implicit_grad_dev(fire_handle_t* h, const double* d_pos, co
     const int64_t it = gs.h_cs->it;
     const int reason = gs.h_cs->reason;
     const double rel_res = rr > 0.0 ? std::sqrt(gs.h_cs->rr / rr) : 0.0;
-    k_g_force<<<h->grad.nb, kForceBlock, 0, s>>>(b, pc, L, h->b.exp_table, nullptr, nullptr, lam);
+    k_cg_export<<<ne, kElemBlock, 0, s>>>(n, lam, row);
+    k_g_force<<<h->grad.nb, kForceBlock, 0, s>>>(b, pc, L, h->b.exp_table, nullptr, nullptr, row);
     CK(h, cudaGetLastError());
     double sums[4];
     if ((st = grad_sums(h, 5, 4, sums, s)) != FIRE_OK) return st;
     for (int k = 0; k < 4; ++k) dL_dtheta[k] = sums[k];
-    if (d_lambda) CK(h, cudaMemcpyAsync(d_lambda, lam, bytes, cudaMemcpyDeviceToDevice, s));
+    if (d_lambda) CK(h, cudaMemcpyAsync(d_lambda, row, bytes, cudaMemcpyDeviceToDevice, s));
     CK(h, cudaStreamSynchronize(s));
     if (cg_iters) *cg_iters = it;
     // the outputs above hold the last iterate in every case; a solve that did

@@ -28,10 +28,31 @@ struct GradBufs {
     const int* nnbr;
     double *rho, *F1, *F2, *drho, *dq;
     double* part;          // block partials
-    // pair coefficients of the HVP at fixed positions (k_g_pair_cache), one
-    // per list slot [k * n + i]; NULL when not computed
-    const double *w1, *fsc, *a2;
-    const double *dcx, *dcy, *dcz;   // cached separation x_j - x_i per list slot
+    // pair quantities of the HVP at fixed positions (k_g_pair_cache), one per
+    // list slot [k * n + i]: the separation x_j - x_i with w1 in its fourth
+    // word, and (fs, a2); per atom the number of slots up to the last pair
+    // inside rc and sum_j w1 (x_j - x_i)
+    dvec4* dw;
+    double2* fa;
+    int* nin;
+    dvec4* wsum;
+    double* dot;           // per slot d.(u_j - u_i), from pass 1 to pass 2
+    double* dc;            // per atom F''_i drho_i
+};
+
+// Scalars of the conjugate-gradient solve, kept on the device so that the
+// iterations run without a host round trip; every kernel of an iteration
+// returns at once when the solve is done (done = 1), so the host can queue
+// several iterations and look at the state once per batch.
+// Why the solve stopped (CgState::reason).
+enum CgReason { CG_RUNNING = 0, CG_CONVERGED = 1, CG_BREAKDOWN = 2, CG_MAXIT = 3 };
+
+struct CgState {
+    double rr, stop2, alpha, beta, m[3];
+    long long it, maxit;
+    int done;
+    int reason;            // CgReason
+    unsigned ticket;       // blocks finished (last-block test)
 };
 
 struct Pair2 {
@@ -299,18 +320,15 @@ __global__ void __launch_bounds__(kForceBlock) k_g_hvp2(GradBufs g, PotC P, GeoL
 
 // Pair coefficients of the HVP at the current positions, for the many
 // products of one conjugate-gradient solve (the positions do not change):
-// per list slot w1 = g'/r, fs = [2 phi' + (F'_i + F'_j) g'] / r and
-// a2 = [2 phi'' + (F'_i + F'_j) g'' - fs] / r^2, zero beyond rc.  With them
-// dfs = a2 d.(u_j - u_i) + (F''_i drho_i + F''_j drho_j) w1 (HVP pass 2) and
-// drho_i = sum_j w1 d.(u_j - u_i) (pass 1) need no pair function.  The
-// separation d = x_j - x_i of each slot is cached too: the HVP passes then
-// stream it instead of gathering x_j and redoing the minimum image (six FP64
-// instructions per pair and pass at 1/58 of the FP32 rate).
+// per list slot d = x_j - x_i, w1 = g'/r, fs = [2 phi' + (F'_i + F'_j) g'] / r
+// and a2 = [2 phi'' + (F'_i + F'_j) g'' - fs] / r^2, zero beyond rc.  With
+// them the two passes need no pair function and no minimum image:
+//   pass 1:  dot = d.(u_j - u_i),  dc_i = F''_i sum_j w1 dot
+//   pass 2:  dF_i = sum_j [(a2 dot + dc_j w1) d + fs (u_j - u_i)]
+//                   + dc_i sum_j w1 d
+// (the last sum is the atom's own and is kept as well).
 __global__ void __launch_bounds__(kForceBlock) k_g_pair_cache(GradBufs g, PotC P, GeoL L,
-                                                              const double* exp_table,
-                                                              double* w1, double* fsc,
-                                                              double* a2, double* dcx,
-                                                              double* dcy, double* dcz) {
+                                                              const double* exp_table) {
     __shared__ double3 tbl[125];
     __shared__ double etab[kExpTableSize];
     grad_tables(tbl, etab, exp_table, L.L);
@@ -320,86 +338,226 @@ __global__ void __launch_bounds__(kForceBlock) k_g_pair_cache(GradBufs g, PotC P
     const dvec4 xi = g.x[i];
     const double f1i = g.F1[i];
     const int m = g.nnbr[i];
+    int nin = 0;
+    double wx = 0.0, wy = 0.0, wz = 0.0;
     for (int k = 0; k < m; ++k) {
         const size_t slot = (size_t)k * g.n + i;
         int j;
         double dx, dy, dz;
         const double r2 = grad_pair_vec(g, tbl, xi, g.nbr[slot], j, dx, dy, dz);
-        dcx[slot] = dx;
-        dcy[slot] = dy;
-        dcz[slot] = dz;
         if (!(r2 < P.rc2)) {
-            w1[slot] = 0.0;
-            fsc[slot] = 0.0;
-            a2[slot] = 0.0;
+            g.dw[slot] = make_dvec4(dx, dy, dz, 0.0);
+            g.fa[slot] = make_double2(0.0, 0.0);
             continue;
         }
+        nin = k + 1;
         Pair2 q;
         rgl_pair_d2(P, r2, etab, q);
         const double c = f1i + g.F1[j];
-        const double fs = (2.0 * q.dphi + c * q.dg) * q.rinv;
-        w1[slot] = q.dg * q.rinv;
-        fsc[slot] = fs;
-        a2[slot] = (2.0 * q.d2phi + c * q.d2g - fs) * q.rinv * q.rinv;
+        const double fs = (2.0 * q.dphi + c * q.dg) * q.rinv, w1 = q.dg * q.rinv;
+        g.dw[slot] = make_dvec4(dx, dy, dz, w1);
+        g.fa[slot] = make_double2(fs, (2.0 * q.d2phi + c * q.d2g - fs) * q.rinv * q.rinv);
+        wx = fma(w1, dx, wx);
+        wy = fma(w1, dy, wy);
+        wz = fma(w1, dz, wz);
     }
+    g.nin[i] = nin;
+    g.wsum[i] = make_dvec4(wx, wy, wz, 0.0);
 }
 
-// HVP pass 1 from the pair cache.
+// HVP pass 1 from the pair cache, u in padded quads.  Both passes are bound by
+// the FP64 pipe (1/58 of the FP32 rate): 7 and 11 FP64 instructions per pair;
+// 31,999 atoms 36 + 74 -> 27 + 50 us (22 FP64 instructions per pair before).
 template <int TPA>
-__global__ void __launch_bounds__(kForceBlock) k_g_hvp1c(GradBufs g, const double* u,
+__global__ void __launch_bounds__(kForceBlock) k_g_hvp1c(GradBufs g, const dvec4* u,
                                                          const int* skip) {
-    if (skip && *skip) return;   // a finished conjugate-gradient solve
+    if (*skip) return;   // a finished conjugate-gradient solve
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = t / TPA, lane = t % TPA;   // TPA threads per atom (group_sum)
     if (i >= g.n) return;
-    const double* ui = u + 3 * (size_t)i;
+    const dvec4 ui = u[i];
     double acc = 0.0;
-    const int m = g.nnbr[i];
+    const int m = g.nin[i];
     for (int k = lane; k < m; k += TPA) {
         const size_t slot = (size_t)k * g.n + i;
-        const double w = g.w1[slot];
-        if (w == 0.0) continue;
-        const int j = (int)(g.nbr[slot] & kIdxMask);
-        const double dx = g.dcx[slot], dy = g.dcy[slot], dz = g.dcz[slot];
-        const double* uj = u + 3 * (size_t)j;
-        acc += w * (dx * (uj[0] - ui[0]) + dy * (uj[1] - ui[1]) + dz * (uj[2] - ui[2]));
+        const dvec4 d = g.dw[slot];
+        const dvec4 uj = u[g.nbr[slot] & kIdxMask];
+        const double dot = d.x * (uj.x - ui.x) + d.y * (uj.y - ui.y) + d.z * (uj.z - ui.z);
+        g.dot[slot] = dot;
+        acc = fma(d.w, dot, acc);
     }
     acc = group_sum<TPA>(acc);
-    if (lane == 0) g.drho[i] = acc;
+    if (lane == 0) g.dc[i] = g.F2[i] * acc;
 }
 
-// HVP pass 2 from the pair cache: (H u)_i = -dF_i.
+// The four sums of a block (each thread's contribution in v) into the partials
+// part[k * gridDim.x + block]; true in every thread of the last block of the
+// grid to come here (ticket), where every block's partials are visible.
+__device__ __forceinline__ bool cg_block_sum4(double v0, double v1, double v2, double v3, double* part,
+                                              unsigned* ticket) {
+    __shared__ double sh[4][32];
+    __shared__ int last;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double s = warp_sum4(v0, v1, v2, v3);
+    if ((lane & 7) == 0) sh[lane >> 3][w] = s;
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        double a = 0.0;
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) a += sh[threadIdx.x][q];
+        part[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = a;
+        __threadfence();   // this block's partials before its ticket
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1 : 0;
+    __syncthreads();
+    if (!last) return false;
+    if (threadIdx.x == 0) *ticket = 0u;
+    __threadfence();
+    return true;
+}
+// The partials of rows 0 .. 3 added up in a fixed order by one block; valid in
+// thread 0.
+__device__ __forceinline__ void cg_final_sum4(const double* part, int nb, double out[4]) {
+    __shared__ double sh[4][32];
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int k = threadIdx.x; k < nb; k += blockDim.x)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) a[r] += part[(size_t)r * nb + k];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double s = warp_sum4(a[0], a[1], a[2], a[3]);
+    if ((lane & 7) == 0) sh[lane >> 3][w] = s;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int r = 0; r < 4; ++r) {
+            out[r] = 0.0;
+            for (int q = 0; q < (int)(blockDim.x >> 5); ++q) out[r] += sh[r][q];
+        }
+}
+
+// HVP pass 2 from the pair cache: Ap = H p (= -dF).  Its last block ends the
+// step's first half: the column means of Ap (the translations that are
+// projected out, H being singular along them) and alpha = r.r / p.Ap (p has no
+// mean, so projecting Ap does not change p.Ap); CG_BREAKDOWN when H is not
+// positive definite along p or p.Ap is not finite.
 template <int TPA>
-__global__ void __launch_bounds__(kForceBlock) k_g_hvp2c(GradBufs g, const double* u, double* hu,
-                                                         const int* skip) {
-    if (skip && *skip) return;
+__global__ void __launch_bounds__(kForceBlock) k_g_hvp2c(GradBufs g, const dvec4* p, dvec4* Ap,
+                                                         CgState* cs) {
+    if (cs->done) return;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = t / TPA, lane = t % TPA;
-    if (i >= g.n) return;
-    const double* ui = u + 3 * (size_t)i;
-    const double dci = g.F2[i] * g.drho[i];
-    double dF[3] = {0, 0, 0};
-    const int m = g.nnbr[i];
-    for (int k = lane; k < m; k += TPA) {
-        const size_t slot = (size_t)k * g.n + i;
-        const double fs = g.fsc[slot];
-        if (fs == 0.0 && g.w1[slot] == 0.0) continue;
-        const int j = (int)(g.nbr[slot] & kIdxMask);
-        const double d[3] = {g.dcx[slot], g.dcy[slot], g.dcz[slot]};
-        const double* uj = u + 3 * (size_t)j;
-        const double du[3] = {uj[0] - ui[0], uj[1] - ui[1], uj[2] - ui[2]};
-        const double dd = d[0] * du[0] + d[1] * du[1] + d[2] * du[2];
-        const double dfs = g.a2[slot] * dd + (dci + g.F2[j] * g.drho[j]) * g.w1[slot];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) dF[a] += dfs * d[a] + fs * du[a];
+    double hx = 0.0, hy = 0.0, hz = 0.0, ph = 0.0;
+    if (i < g.n) {
+        const dvec4 ui = p[i];
+        double fx = 0.0, fy = 0.0, fz = 0.0;
+        const int m = g.nin[i];
+        for (int k = lane; k < m; k += TPA) {
+            const size_t slot = (size_t)k * g.n + i;
+            const int j = (int)(g.nbr[slot] & kIdxMask);
+            const dvec4 d = g.dw[slot], uj = p[j];
+            const double2 fa = g.fa[slot];
+            const double dfs = fma(fa.y, g.dot[slot], g.dc[j] * d.w);
+            fx = fma(dfs, d.x, fma(fa.x, uj.x - ui.x, fx));
+            fy = fma(dfs, d.y, fma(fa.x, uj.y - ui.y, fy));
+            fz = fma(dfs, d.z, fma(fa.x, uj.z - ui.z, fz));
+        }
+        fx = group_sum<TPA>(fx);
+        fy = group_sum<TPA>(fy);
+        fz = group_sum<TPA>(fz);
+        if (lane == 0) {
+            const dvec4 ws = g.wsum[i];
+            const double dci = g.dc[i];
+            hx = -fma(dci, ws.x, fx);
+            hy = -fma(dci, ws.y, fy);
+            hz = -fma(dci, ws.z, fz);
+            Ap[i] = make_dvec4(hx, hy, hz, 0.0);
+            ph = ui.x * hx + ui.y * hy + ui.z * hz;
+        }
     }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) dF[a] = group_sum<TPA>(dF[a]);
-    if (lane != 0) return;
-    double* h = hu + 3 * (size_t)i;
-    h[0] = -dF[0];
-    h[1] = -dF[1];
-    h[2] = -dF[2];
+    __syncwarp();   // lanes past the end rejoin their warp
+    if (!cg_block_sum4(hx, hy, hz, ph, g.part, &cs->ticket)) return;
+    double s[4];
+    cg_final_sum4(g.part, gridDim.x, s);
+    if (threadIdx.x != 0) return;
+    for (int k = 0; k < 3; ++k) cs->m[k] = s[k] / g.n;
+    if (!(s[3] > 0.0) || !isfinite(s[3])) {
+        cs->done = 1;
+        cs->reason = CG_BREAKDOWN;
+    } else {
+        cs->alpha = cs->rr / s[3];
+    }
+}
+
+// lam += alpha p; r -= alpha (Ap - its means); the last block: the new r.r,
+// beta, the iteration count and the stopping test.
+__global__ void __launch_bounds__(kElemBlock) k_cg_step(int n, CgState* cs, const dvec4* p,
+                                                        const dvec4* Ap, dvec4* lam, dvec4* r,
+                                                        double* part) {
+    if (cs->done) return;
+    const double alpha = cs->alpha, m0 = cs->m[0], m1 = cs->m[1], m2 = cs->m[2];
+    double acc = 0.0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const dvec4 pi = p[i], ai = Ap[i];
+        dvec4 l = lam[i], ri = r[i];
+        l.x = fma(alpha, pi.x, l.x);
+        l.y = fma(alpha, pi.y, l.y);
+        l.z = fma(alpha, pi.z, l.z);
+        lam[i] = l;
+        ri.x -= alpha * (ai.x - m0);
+        ri.y -= alpha * (ai.y - m1);
+        ri.z -= alpha * (ai.z - m2);
+        r[i] = ri;
+        acc = fma(ri.z, ri.z, fma(ri.y, ri.y, fma(ri.x, ri.x, acc)));
+    }
+    if (!cg_block_sum4(acc, 0.0, 0.0, 0.0, part, &cs->ticket)) return;
+    double s[4];
+    cg_final_sum4(part, gridDim.x, s);
+    if (threadIdx.x != 0) return;
+    const double rr = s[0];
+    cs->beta = rr / cs->rr;
+    cs->rr = rr;
+    cs->it += 1;
+    if (!isfinite(rr)) {
+        cs->done = 1;
+        cs->reason = CG_BREAKDOWN;
+    } else if (!(rr > cs->stop2)) {
+        cs->done = 1;
+        cs->reason = CG_CONVERGED;
+    } else if (cs->it >= cs->maxit) {
+        cs->done = 1;
+        cs->reason = CG_MAXIT;
+    }
+}
+
+// p = r + beta p
+__global__ void k_cg_dir(int n, const CgState* cs, const dvec4* r, dvec4* p) {
+    if (cs->done) return;
+    const double beta = cs->beta;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const dvec4 ri = r[i];
+        dvec4 pi = p[i];
+        pi.x = fma(beta, pi.x, ri.x);
+        pi.y = fma(beta, pi.y, ri.y);
+        pi.z = fma(beta, pi.z, ri.z);
+        p[i] = pi;
+    }
+}
+
+// r = p = v (row-major), lam = 0; and back.
+__global__ void k_cg_load(int n, const double* v, dvec4* r, dvec4* p, dvec4* lam) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double* q = v + 3 * (size_t)i;
+    r[i] = p[i] = make_dvec4(q[0], q[1], q[2], 0.0);
+    lam[i] = make_dvec4(0.0, 0.0, 0.0, 0.0);
+}
+__global__ void k_cg_export(int n, const dvec4* lam, double* v) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const dvec4 l = lam[i];
+    double* q = v + 3 * (size_t)i;
+    q[0] = l.x;
+    q[1] = l.y;
+    q[2] = l.z;
 }
 
 // Row-major positions into the padded layout used by the list build.
@@ -443,136 +601,6 @@ __global__ void k_g_sub_mean(int n, double* a, double m0, double m1, double m2) 
         a[3 * (size_t)i + 1] -= m1;
         a[3 * (size_t)i + 2] -= m2;
     }
-}
-
-// Scalars of the conjugate-gradient solve, kept on the device so that the
-// iterations run without a host round trip; every kernel of an iteration
-// returns at once when the solve is done (done = 1), so the host can queue
-// several iterations and look at the state once per batch.
-// Why the solve stopped (CgState::reason).
-enum CgReason { CG_RUNNING = 0, CG_CONVERGED = 1, CG_BREAKDOWN = 2, CG_MAXIT = 3 };
-
-struct CgState {
-    double rr, stop2, alpha, beta, m[3];
-    long long it, maxit;
-    int done;
-    int reason;            // CgReason
-};
-
-// Fixed-order sum of cnt partials by one block (result in thread 0).
-__device__ __forceinline__ double cg_sum(const double* a, int cnt, double* red) {
-    double s = 0.0;
-    for (int k = threadIdx.x; k < cnt; k += blockDim.x) s += a[k];
-    return block_sum(s, red);
-}
-
-// Column sums of Ap, as partials (k_g_colsum), unless the solve is done.
-__global__ void k_cg_colsum(int n, const CgState* cs, const double* a, double* part) {
-    __shared__ double red[32];
-    if (cs->done) return;
-    double c[3] = {0.0, 0.0, 0.0};
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        c[0] += a[3 * (size_t)i];
-        c[1] += a[3 * (size_t)i + 1];
-        c[2] += a[3 * (size_t)i + 2];
-    }
-    for (int k = 0; k < 3; ++k) {
-        const double s = block_sum(c[k], red);
-        if (threadIdx.x == 0) part[k * gridDim.x + blockIdx.x] = s;
-    }
-}
-
-// One block: the mean of each Cartesian column of Ap (the translations that
-// are projected out, H being singular along them).
-__global__ void k_cg_means(CgState* cs, const double* part, int nb, int n) {
-    __shared__ double red[32];
-    if (cs->done) return;
-    for (int k = 0; k < 3; ++k) {
-        const double s = cg_sum(part + (size_t)k * nb, nb, red);
-        if (threadIdx.x == 0) cs->m[k] = s / n;
-    }
-}
-
-// Ap -= its column means; partials of p.Ap.
-__global__ void k_cg_project_dot(int n, const CgState* cs, double* ap, const double* p,
-                                 double* part) {
-    __shared__ double red[32];
-    if (cs->done) return;
-    const double m0 = cs->m[0], m1 = cs->m[1], m2 = cs->m[2];
-    double acc = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const size_t k = 3 * (size_t)i;
-        const double a0 = ap[k] - m0, a1 = ap[k + 1] - m1, a2 = ap[k + 2] - m2;
-        ap[k] = a0;
-        ap[k + 1] = a1;
-        ap[k + 2] = a2;
-        acc += p[k] * a0 + p[k + 1] * a1 + p[k + 2] * a2;
-    }
-    acc = block_sum(acc, red);
-    if (threadIdx.x == 0) part[blockIdx.x] = acc;
-}
-
-// One block: alpha = r.r / p.Ap; stops (CG_BREAKDOWN) when H is not
-// positive definite along p or p.Ap is not finite.
-__global__ void k_cg_alpha(CgState* cs, const double* part, int nb) {
-    __shared__ double red[32];
-    if (cs->done) return;
-    const double pAp = cg_sum(part, nb, red);
-    if (threadIdx.x == 0) {
-        if (!(pAp > 0.0) || !isfinite(pAp)) {
-            cs->done = 1;
-            cs->reason = CG_BREAKDOWN;
-        } else {
-            cs->alpha = cs->rr / pAp;
-        }
-    }
-}
-
-// lam += alpha p; r -= alpha Ap; partials of r.r.
-__global__ void k_cg_step(int m, const CgState* cs, const double* p, const double* Ap,
-                          double* lam, double* r, double* part) {
-    __shared__ double red[32];
-    if (cs->done) return;
-    const double alpha = cs->alpha;
-    double acc = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        lam[i] += alpha * p[i];
-        const double ri = r[i] - alpha * Ap[i];
-        r[i] = ri;
-        acc += ri * ri;
-    }
-    acc = block_sum(acc, red);
-    if (threadIdx.x == 0) part[blockIdx.x] = acc;
-}
-
-// One block: the new r.r, beta, the iteration count and the stopping test.
-__global__ void k_cg_beta(CgState* cs, const double* part, int nb) {
-    __shared__ double red[32];
-    if (cs->done) return;
-    const double rr = cg_sum(part, nb, red);
-    if (threadIdx.x == 0) {
-        cs->beta = rr / cs->rr;
-        cs->rr = rr;
-        cs->it += 1;
-        if (!isfinite(rr)) {
-            cs->done = 1;
-            cs->reason = CG_BREAKDOWN;
-        } else if (!(rr > cs->stop2)) {
-            cs->done = 1;
-            cs->reason = CG_CONVERGED;
-        } else if (cs->it >= cs->maxit) {
-            cs->done = 1;
-            cs->reason = CG_MAXIT;
-        }
-    }
-}
-
-// p = r + beta p
-__global__ void k_cg_dir(int m, const CgState* cs, const double* r, double* p) {
-    if (cs->done) return;
-    const double beta = cs->beta;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x)
-        p[i] = r[i] + beta * p[i];
 }
 
 }  // namespace fire2
