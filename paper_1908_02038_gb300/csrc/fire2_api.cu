@@ -15,6 +15,7 @@
 #include "fire2.h"
 #include "fire2_device.cuh"
 #include "fire2_grad.cuh"
+#include "fire2_loop.cuh"
 #include "fire2_neb.cuh"
 #include "fire2_tile.cuh"
 
@@ -110,6 +111,10 @@ struct fire_handle {
     int img_n = 0;                   // atoms per image (n, except for NEB handles)
     bool verify = false;             // FP32-pair: stops on ftol confirmed in FP64
     int sms = 0;                     // SM count of the device
+    bool tpa_set = false;            // threads per atom chosen by the caller
+    bool loop = false;               // make_geo: lists for the resident loop (full)
+    int loop_ok = -1;                // its graph can be made on this device (-1: not tried)
+    double* loop_rows = nullptr;     // the resident loop's partials
     int tile_mode = FIRE_TILES_AUTO; // shared-memory tiles of the FP64 half-list passes
     int stage_cap = 0;               // staged atoms per tile (0 = kStageMax)
     size_t loc_slots = 0;            // allocated nbr_loc entries
@@ -216,6 +221,23 @@ bool tiles_wanted(const fire_handle* h, const GeoC& g) {
     return h->tile_mode == FIRE_TILES_ON;
 }
 
+// Whether relaxations run in the resident loop (fire2_loop.cuh): the default
+// settings of the FP64 table form and LJ, one system, up to kLoopAtoms atoms.
+// What the caller has chosen (newton, threads per atom, tiles, chunked or
+// sized graph bodies, a displacement cap) keeps the kernel chain.  RGL, us per
+// iteration chain / loop: 48,667 atoms 84.5 / 70.5, 62,499 atoms 98 / 77; above,
+// the full list's second evaluation of every pair eats the gain, and for LJ,
+// whose pair terms are FP64 arithmetic, earlier (10,975 atoms 80 / 53).
+constexpr int kLoopAtoms = 65536, kLoopAtomsLj = 16384;
+bool loop_wanted(const fire_handle* h) {
+    const bool form = h->pot.kind == FIRE_POT_LJ ||
+                      (fixed64_form(h->pot) && h->pot.newton == FIRE_NEWTON_AUTO);
+    return form && h->loop_ok != 0 && !h->neb && !h->batch && h->img_n == h->n &&
+           h->n <= (h->pot.kind == FIRE_POT_LJ ? kLoopAtomsLj : kLoopAtoms) && !h->tpa_set &&
+           h->tile_mode != FIRE_TILES_ON && h->exec_mode == FIRE_EXEC_GRAPH_WHILE &&
+           h->body_iters == 0 && !(h->par.dmax > 0.0);
+}
+
 // Neighbour geometry for a box.  The list radius is rc + skin, with the skin
 // reduced where a periodic axis is shorter than 2 (rc + skin) so that the
 // minimum image stays unique within the list radius.
@@ -254,7 +276,7 @@ GeoC make_geo(const fire_handle* h, const double box[3]) {
     const double margin = 1e-3 * rc + 8.0 * 1.2e-7 * (2.0 * lmax);
     g.rlist2f = (float)((rl + margin) * (rl + margin));
     g.full = (h->pot.precision == FIRE_PREC_FP32_PAIR || h->pot.kind == FIRE_POT_SW ||
-              (fixed64_form(h->pot) && !fixed64_half(h->pot))) ? 1 : 0;
+              (fixed64_form(h->pot) && !fixed64_half(h->pot)) || h->loop) ? 1 : 0;
     for (int a = 0; a < 3; ++a) {
         g.Lq[a] = (int)(unsigned)(unsigned long long)std::llrint(box[a] * h->b.qscale);
         g.Lq64[a] = std::llrint(std::ldexp(box[a], kFixedBits64));
@@ -632,7 +654,100 @@ cudaError_t add_conditional(cudaStream_t s, cudaGraphConditionalHandle hc,
 constexpr int kLoopUnroll = 8;
 constexpr int kMaxBodyIters = 64;
 
+// The resident loop's launch for n atoms: blocks (at most one per SM, two atoms
+// or more each), their share, lanes per atom, threads.
+struct LoopShape {
+    int blocks, share, lanes, threads;
+};
+LoopShape loop_shape(const fire_handle* h) {
+    LoopShape q;
+    q.share = std::max(2, ceil_div(h->n, h->sms));
+    q.blocks = ceil_div(h->n, q.share);
+    // lanes per atom, us per iteration at 8 / 16 / 32 (RGL): shares of 2 20.8 / 17.6 /
+    // 16.1, 27 22.6 / 22.0 / 25.7, 46 24.6 / 26.3 / 34.5; at 4 / 8: 130 38.4 / 46.9,
+    // 73 31.6 / 29.0: more lanes shorten the chain of pairs but add FP64 group sums
+    q.lanes = q.share <= 8 ? 32 : q.share <= 32 ? 16 : q.share <= 112 || h->pot.kind == FIRE_POT_LJ ? 8 : 4;
+    q.threads = std::min(kLoopThreads, std::max(256, (q.share * q.lanes + 31) / 32 * 32));
+    return q;
+}
+using LoopKernel = void (*)(Bufs, PotC, GeoC, LoopC, cudaGraphConditionalHandle);
+template <bool RGL, int L>
+LoopKernel loop_kernel_t(int threads) {
+    return threads <= 512 ? k_loop<RGL, L, 512> : threads <= 896 ? k_loop<RGL, L, 896> : k_loop<RGL, L, 1024>;
+}
+LoopKernel loop_kernel(const fire_handle* h, const LoopShape& q) {
+    if (h->pot.kind == FIRE_POT_LJ)
+        return q.lanes == 32 ? loop_kernel_t<false, 32>(q.threads)
+             : q.lanes == 16 ? loop_kernel_t<false, 16>(q.threads)
+                             : loop_kernel_t<false, 8>(q.threads);
+    return q.lanes == 32 ? loop_kernel_t<true, 32>(q.threads)
+         : q.lanes == 16 ? loop_kernel_t<true, 16>(q.threads)
+         : q.lanes == 8 ? loop_kernel_t<true, 8>(q.threads)
+                        : loop_kernel_t<true, 4>(q.threads);
+}
+
+// The resident loop as a graph: prepare; WHILE (not stopped): list build,
+// k_loop (which sets the condition); finalize.
+fire_status build_loop_graph(fire_handle* h, const GeoC& g) {
+    drop_graph(h);
+    const LoopShape q = loop_shape(h);
+    const LoopKernel kern = loop_kernel(h, q);
+    const size_t smem = loop_smem(q.share);
+    CK(h, cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (!h->loop_rows) CK(h, cudaMalloc(&h->loop_rows, (size_t)kLoopRows * h->sms * sizeof(double)));
+    cudaGraph_t graph = nullptr;
+    CK(h, cudaGraphCreate(&graph, 0));
+    cudaGraphConditionalHandle hw;
+    cudaError_t e = cudaGraphConditionalHandleCreate(&hw, graph, 1, cudaGraphCondAssignDefault);
+    if (e == cudaSuccess)
+        e = cudaStreamBeginCaptureToGraph(h->cap0, graph, nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeRelaxed);
+    if (e != cudaSuccess) {
+        cudaGraphDestroy(graph);
+        return fail(h, FIRE_ERR_CUDA, "begin capture: %s", cudaGetErrorString(e));
+    }
+    k_prepare<<<ceil_div(h->n, kElemBlock), kElemBlock, 0, h->cap0>>>(h->b);
+    cudaGraph_t body = nullptr;
+    e = add_conditional(h->cap0, hw, cudaGraphCondTypeWhile, &body);
+    if (e == cudaSuccess)
+        e = cudaStreamBeginCaptureToGraph(h->cap1, body, nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeRelaxed);
+    if (e == cudaSuccess) {
+        launch_build(h, g, 1, h->cap1);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)q.blocks, 1, 1);
+        cfg.blockDim = dim3((unsigned)q.threads, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = h->cap1;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, kern, h->b, h->potc, g, LoopC{h->loop_rows, q.share}, hw);
+        cudaGraph_t body_out = nullptr;
+        const cudaError_t e1 = cudaStreamEndCapture(h->cap1, &body_out);
+        if (e == cudaSuccess) e = e1;
+    }
+    k_finalize<<<ceil_div(h->n, kElemBlock), kElemBlock, 0, h->cap0>>>(h->b);
+    cudaGraph_t out = nullptr;
+    const cudaError_t e2 = cudaStreamEndCapture(h->cap0, &out);
+    if (e == cudaSuccess) e = e2;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&h->exec, graph, 0);
+    if (e != cudaSuccess) {
+        cudaGraphDestroy(graph);
+        h->exec = nullptr;
+        cudaGetLastError();
+        return fail(h, FIRE_ERR_CUDA, "resident loop's graph: %s", cudaGetErrorString(e));
+    }
+    h->graph = graph;
+    h->gkey = g;
+    h->has_graph = true;
+    return FIRE_OK;
+}
+
 fire_status build_graph(fire_handle* h, const GeoC& g) {
+    if (h->loop) return build_loop_graph(h, g);
     drop_graph(h);
     cudaGraph_t graph = nullptr;
     CK(h, cudaGraphCreate(&graph, 0));
@@ -853,6 +968,7 @@ void init_state(fire_handle* h, double ftol, int64_t maxiter) {
     q.alpha0 = p.alpha0;
     q.alphashrink = p.alphashrink;
     q.mass = h->sys.mass;
+    q.minv = 1.0 / h->sys.mass;
     q.delaystep = p.delaystep;
     q.vdfmax = p.vdfmax;
     q.halfstepback = p.halfstepback;
@@ -919,12 +1035,14 @@ fire_status check_params(fire_handle* h, const fire_params_t& p) {
     return FIRE_OK;
 }
 
-fire_status prepare_call(fire_handle* h, const double box[3], GeoC* g, bool neb_call = false) {
+fire_status prepare_call(fire_handle* h, const double box[3], GeoC* g, bool neb_call = false,
+                         bool relax = false) {
     if (h->batch) return fail(h, FIRE_ERR_STATE, "batched handle: use fire_minimize_batch");
     if (h->neb && !neb_call) return fail(h, FIRE_ERR_STATE, "NEB handle: use fire_neb_minimize");
     fire_status st = check_box(h, box);
     if (st != FIRE_OK) return st;
     CK(h, cudaSetDevice(h->device));
+    h->loop = relax && loop_wanted(h);
     *g = make_geo(h, box);
     const int cap = std::max(estimate_cap(h, *g), h->cap);
     return ensure_buffers(h, *g, cap);
@@ -1318,7 +1436,7 @@ void fire_destroy(fire_handle_t* h) {
     void* ptrs[] = {b.x, b.v, b.f, b.xf, b.xq, b.xq64, b.fp32, (void*)b.exp32_table,
                     (void*)b.exp_table, b.rho, b.fp, b.nbr, b.nnbr, b.crep, b.cden,
                     b.cell_of, b.cell_count, b.cell_start, b.cell_atoms, b.xs, b.cell_box, b.epart, b.rpart,
-                    b.st, b.pos_io, b.nbr_loc, b.tile_key, b.tile_ns};
+                    b.st, b.pos_io, b.nbr_loc, b.tile_key, b.tile_ns, h->loop_rows};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (h->batch) fire2_batch_free(h->batch);
@@ -1388,6 +1506,16 @@ fire_status fire_set_dof_mask(fire_handle_t* h, const uint8_t* mask) {
     return FIRE_OK;
 }
 
+// prepare_call for a relaxation: where the resident loop's graph cannot be made
+// (no cooperative launches inside conditional nodes, as under MPS) the kernel
+// chain from then on.
+static fire_status prepare_relax(fire_handle* h, const double box[3], GeoC* g) {
+    fire_status st = prepare_call(h, box, g, false, true);
+    if (st != FIRE_OK || !h->loop || h->loop_ok == 1) return st;
+    h->loop_ok = build_loop_graph(h, *g) == FIRE_OK ? 1 : 0;
+    return h->loop_ok ? FIRE_OK : prepare_call(h, box, g, false, true);
+}
+
 // One relaxation on the device: positions are already in b.pos_io.
 static fire_status run_minimize(fire_handle* h, const GeoC& g, double ftol, int64_t maxiter,
                                 cudaStream_t s) {
@@ -1423,6 +1551,8 @@ fire_status fire_set_threads_per_atom(fire_handle_t* h, int32_t tpa, int32_t* ch
     if (tpa != 0 && tpa != 1 && tpa != 2 && tpa != 4 && tpa != 8 && tpa != 16 && tpa != 32)
         return fail(h, FIRE_ERR_ARG, "threads per atom must be 0 (automatic), 1, 2, 4, 8, 16 or 32");
     const int t = !tpa_form(h->pot) ? 1 : tpa == 0 ? auto_tpa(h->pot, h->n, h->sms) : tpa;
+    if (h->tpa_set != (tpa != 0)) drop_graph(h);   // the resident loop chooses its own
+    h->tpa_set = tpa != 0;
     if (t != h->b.tpa) {
         drop_graph(h);
         h->b.tpa = t;
@@ -1468,7 +1598,7 @@ fire_status fire_minimize_dev(fire_handle_t* h, double* d_pos, const double box[
     if (!d_pos || !out) return fail(h, FIRE_ERR_ARG, "NULL positions or result");
     if (!(ftol >= 0.0) || maxiter < 0) return fail(h, FIRE_ERR_ARG, "need ftol >= 0 and maxiter >= 0");
     GeoC g;
-    fire_status st = prepare_call(h, box, &g);
+    fire_status st = prepare_relax(h, box, &g);
     if (st != FIRE_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
     const size_t bytes = (size_t)3 * h->n * sizeof(double);
@@ -1509,7 +1639,7 @@ fire_status fire_minimize(fire_handle_t* h, double* pos, const double box[3], do
     if (!pos || !out) return fail(h, FIRE_ERR_ARG, "NULL positions or result");
     if (!(ftol >= 0.0) || maxiter < 0) return fail(h, FIRE_ERR_ARG, "need ftol >= 0 and maxiter >= 0");
     GeoC g;
-    fire_status st = prepare_call(h, box, &g);
+    fire_status st = prepare_relax(h, box, &g);
     if (st != FIRE_OK) return st;
     cudaStream_t s = h->stream;
     const size_t bytes = (size_t)3 * h->n * sizeof(double);

@@ -1065,6 +1065,7 @@ static fire_status batch_launch(fire_handle_t* h, fire_batch_state* b, double ft
     q.alpha0 = p.alpha0;
     q.alphashrink = p.alphashrink;
     q.mass = fire2_sys(h).mass;
+    q.minv = 1.0 / fire2_sys(h).mass;
     q.delaystep = p.delaystep;
     q.vdfmax = p.vdfmax;
     q.halfstepback = p.halfstepback;

@@ -157,6 +157,35 @@ __device__ __forceinline__ double group_sum(double v) {
     return v;
 }
 
+// Four (two) sums over the L consecutive lanes of an atom by the transposing
+// butterfly of warp_sum4 (L >= 4): lane l of the group ends with the total of
+// q_k, k = l / (L / 4) (l / (L / 2)).  3 + log2 L - 2 FP64 additions in place of
+// 4 log2 L.
+template <int L>
+__device__ __forceinline__ double group_sum4(double q0, double q1, double q2, double q3) {
+    static_assert(L >= 4 && L <= 32, "lanes per atom");
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned gmask = L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u) << (lane & ~(unsigned)(L - 1));
+    const bool hi = (lane & (L / 2)) != 0u, odd = (lane & (L / 4)) != 0u;
+    const double r0 = __shfl_xor_sync(gmask, hi ? q0 : q2, L / 2);
+    const double r1 = __shfl_xor_sync(gmask, hi ? q1 : q3, L / 2);
+    const double a0 = (hi ? q2 : q0) + r0, a1 = (hi ? q3 : q1) + r1;
+    double v = (odd ? a1 : a0) + __shfl_xor_sync(gmask, odd ? a0 : a1, L / 4);
+#pragma unroll
+    for (int o = L / 8; o > 0; o >>= 1) v += __shfl_xor_sync(gmask, v, o);
+    return v;
+}
+template <int L>
+__device__ __forceinline__ double group_sum2(double q0, double q1) {
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned gmask = L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u) << (lane & ~(unsigned)(L - 1));
+    const bool hi = (lane & (L / 2)) != 0u;
+    double v = (hi ? q1 : q0) + __shfl_xor_sync(gmask, hi ? q0 : q1, L / 2);
+#pragma unroll
+    for (int o = L / 4; o > 0; o >>= 1) v += __shfl_xor_sync(gmask, v, o);
+    return v;
+}
+
 // Block-wide sum; result valid in thread 0.  `sh` holds >= 32 doubles.
 __device__ __forceinline__ double block_sum(double v, double* sh) {
     v = warp_sum(v);
@@ -362,6 +391,7 @@ struct FireParamsD {
     double dt_start, dtmax, dtmin, dtgrow, dtshrink, alpha0, alphashrink, mass;
     int delaystep, vdfmax, halfstepback, initialdelay, norm, integrator, variant, pad;
     double dmax;           // maximum displacement per step, 0 = no cap
+    double minv;           // 1 / mass
 };
 
 // Scalar state of Algorithms 1/2 plus the coefficients the next element-wise
@@ -410,15 +440,28 @@ __host__ __device__ inline void fire_scal_init(const FireParamsD& p, FireScal& s
 //    Leapfrog initialisation v(-dt/2) = -dt/2 F / m at the first iteration.
 // Norms of mixed velocities come from the reductions:
 // |v + c F|^2 = |v|^2 + 2 c P + c^2 |F|^2.  Returns true to stop.
+// Square roots and quotients by sqrt_f64 and div_f64 (fire2_table.cuh): one
+// thread runs this while everything waits, and the library's sequences are
+// about 20 dependent FP64 instructions each (255 LJ atoms in the resident loop:
+// 12.5 -> 12.3 us per iteration).
+__device__ __forceinline__ double sqrt_f64(double x);
+__device__ __forceinline__ double rcp_f64(double x);
+// a / b from y = 1 / b, the residual put back
+__device__ __forceinline__ double div_by(double a, double b, double y) {
+    const double q = a * y;
+    return fma(fma(-q, b, a), y, q);
+}
 // The stopping norm of Sec. 3.4 (fire_norm) from the reductions.
 __device__ __forceinline__ double force_norm(int norm, double F2, double fa2, double fin) {
-    return norm == 1 ? sqrt(F2) : (norm == 2 ? fin : sqrt(fa2));
+    return norm == 2 ? fin : sqrt_f64(norm == 1 ? F2 : fa2);
 }
 
 __device__ inline bool fire_control_step(const FireParamsD& p, FireScal& s, double P, double F2,
                                          double V2, double fa2, double fin) {
     s.evals += 1;
-    const double fn = force_norm(p.norm, F2, fa2, fin);
+    // what needs no branch first: independent chains overlap
+    const double fnorm = sqrt_f64(F2), fnorm_inv = rcp_f64(fnorm), fatom = sqrt_f64(fa2);
+    const double fn = p.norm == 2 ? fin : (p.norm == 1 ? fnorm : fatom);
     if (fn < p.ftol) {
         s.stop = STOP_FTOL;
         return true;
@@ -431,11 +474,10 @@ __device__ inline bool fire_control_step(const FireParamsD& p, FireScal& s, doub
     s.lf_init = 0;
     if (p.integrator == INT_LEAPFROG && i == 1) {
         s.lf_init = 1;
-        s.lf_c = -0.5 * p.dt_start / p.mass;
+        s.lf_c = div_by(-0.5 * p.dt_start, p.mass, p.minv);
         P = s.lf_c * F2;                 // F . v(-dt/2)
         V2 = s.lf_c * s.lf_c * F2;
     }
-    const double fnorm = sqrt(F2);
     s.zero_v = 0;
     s.halfstep = 0.0;
     s.premix = 0;
@@ -446,7 +488,7 @@ __device__ inline bool fire_control_step(const FireParamsD& p, FireScal& s, doub
             s.npos += 1;
             s.premix = fnorm > 0.0;
             s.mix_a = s.alpha;
-            s.mix_fv_pre = fnorm > 0.0 ? sqrt(V2) / fnorm : 0.0;
+            s.mix_fv_pre = fnorm > 0.0 ? div_by(sqrt_f64(V2), fnorm, fnorm_inv) : 0.0;
             if (s.npos > p.delaystep) {
                 s.dt = fmin(s.dt * p.dtgrow, p.dtmax);
                 s.alpha *= p.alphashrink;
@@ -480,7 +522,7 @@ __device__ inline bool fire_control_step(const FireParamsD& p, FireScal& s, doub
         s.zero_v = 1;
         s.halfstep = p.halfstepback ? 0.5 * s.dt : 0.0;
     }
-    const double dtm = s.dt / p.mass;
+    const double dtm = div_by(s.dt, p.mass, p.minv);
     s.dtm = dtm;
     s.dt_cur = s.dt;
     s.kick_pre = p.integrator == INT_EULER_EXPLICIT ? 0.0
@@ -492,11 +534,11 @@ __device__ inline bool fire_control_step(const FireParamsD& p, FireScal& s, doub
         s.mix_a = s.alpha;
         if (p.integrator == INT_EULER_EXPLICIT) {
             s.premix = 1;
-            s.mix_fv_pre = sqrt(V2) / fnorm;
+            s.mix_fv_pre = div_by(sqrt_f64(V2), fnorm, fnorm_inv);
         } else {
             const double c = s.kick_pre;
             s.postmix = 1;
-            s.mix_fv_post = sqrt(fmax(V2 + 2.0 * c * P + c * c * F2, 0.0)) / fnorm;
+            s.mix_fv_post = div_by(sqrt_f64(fmax(V2 + 2.0 * c * P + c * c * F2, 0.0)), fnorm, fnorm_inv);
             s.post_v = 1.0 - s.alpha;
             s.post_f = s.post_v * c + s.alpha * s.mix_fv_post;
         }

@@ -86,6 +86,10 @@ struct DevState {
     double ftol_user, fn32, fsw;
     unsigned int red_blocks;   // k_reduce_ctl / k_neb_project blocks finished (last-block test)
     unsigned int neb_blocks;   // k_neb_sums blocks finished (last-block test)
+    // the resident loop (fire2_loop.cuh): its barrier's arrivals (and votes) since
+    // the last list build, its abort flag
+    unsigned long long bar;
+    unsigned int bar_abort;
 };
 
 struct Bufs {
@@ -382,6 +386,12 @@ __device__ __forceinline__ float4 xf_of(const Bufs& b, int j) {
     return make_float4((float)x.x, (float)x.y, (float)x.z, 0.f);
 }
 
+// One list build more; the resident loop that may follow starts anew.
+__device__ __forceinline__ void build_count(DevState* st) {
+    st->nbr_builds += 1;
+    st->bar = 0ull;
+}
+
 // List order: the pairs inside rc come first and the skin pairs (rc up to
 // rc + skin, which the force kernels test and skip) after them, so that
 // the lanes of a warp evaluate their in-range pairs together and skip their
@@ -533,7 +543,7 @@ __device__ __forceinline__ void build_pad(float4* cand, int m) {
 __global__ void __launch_bounds__(32 * kBuildWarps) k_nbr_build_all(Bufs b, GeoC g, int force) {
     __shared__ BuildShared<kBuildWarps> sh;
     if (!need_rebuild(b.st, g, force)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) b.st->nbr_builds += 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) build_count(b.st);
     const int w = threadIdx.x >> 5;
     // blocks of one image only, so that they share its candidates
     const int per_img = (g.img_n + kBuildWarps - 1) / kBuildWarps;
@@ -672,7 +682,7 @@ template <int W>
 __global__ void __launch_bounds__(32 * W) k_nbr_build(Bufs b, GeoC g, int force, int cells) {
     __shared__ BuildShared<W> sh;
     if (!need_rebuild(b.st, g, force)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) b.st->nbr_builds += 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) build_count(b.st);
     if (cells == 1) {
         build_cell<W>(b, g, blockIdx.x, sh);
         return;

@@ -410,13 +410,18 @@ __device__ __forceinline__ bool ff_range(double d) {
 }
 
 #ifdef __CUDACC__
+// Whether 2^-120 < d < 2^120, on the integer pipes.
+__device__ __forceinline__ bool f32_exponent(double d) {
+    const long long bits = __double_as_longlong(d);
+    return bits > (903ll << 52) && bits < (1143ll << 52);
+}
 // 1/sqrt(x), x >= 0, in FP64 without a library call: the FP32 estimate y0 (the
 // conversions on the integer pipes) and one step of third order,
 // y0 + y0 e (1/2 + 3/8 e) with e = 1 - x y0^2 ~ 2^-22, off by 5/16 e^3 ~ 2^-67:
-// five FP64 instructions.  Outside ff_range the IEEE operations.
+// five FP64 instructions.  Outside FP32's exponents the IEEE operations.
 static __device__ __noinline__ double rsqrt_f64_any(double x) { return 1.0 / sqrt(x); }
 __device__ __forceinline__ double rsqrt_f64(double x) {
-    if (!ff_range(x)) return rsqrt_f64_any(x);
+    if (!f32_exponent(x)) return rsqrt_f64_any(x);
     const double y0 = f32_to_f64(rsqrtf(f64_to_f32_trunc(x)));
     const double e = fma(-x, y0 * y0, 1.0);
     return fma(y0, fma(e, 0.375, 0.5) * e, y0);
@@ -424,10 +429,19 @@ __device__ __forceinline__ double rsqrt_f64(double x) {
 // 1/x, x >= 0, the same way (y0 + y0 (e + e^2), e = 1 - x y0): three.
 static __device__ __noinline__ double rcp_f64_any(double x) { return 1.0 / x; }
 __device__ __forceinline__ double rcp_f64(double x) {
-    if (!ff_range(x)) return rcp_f64_any(x);
+    if (!f32_exponent(x)) return rcp_f64_any(x);
     const double y0 = f32_to_f64(__frcp_rn(f64_to_f32_trunc(x)));
     const double e = fma(-x, y0, 1.0);
     return fma(y0, fma(e, e, e), y0);
+}
+// sqrt(x) from these with the residual x - s^2 (exact in an FMA) put back: the
+// IEEE result but for rare last-bit ties, in a third of the dependent FP64
+// instructions of the library's.
+static __device__ __noinline__ double sqrt_f64_any(double x) { return sqrt(x); }
+__device__ __forceinline__ double sqrt_f64(double x) {
+    if (!f32_exponent(x)) return sqrt_f64_any(x);
+    const double y = rsqrt_f64(x), s = x * y;
+    return fma(fma(-s, s, x), 0.5 * y, s);
 }
 #endif  // __CUDACC__
 
