@@ -110,16 +110,16 @@ __device__ __forceinline__ double loop_density(const Bufs& b, const PotC& P, con
         const int i = i0 + a, m = b.nnbr[i];
         const lvec4 qi = ld_lvec4_l2(b.xq64 + i);
         ffloat2 acc = {{0.f, 0.f}, {0.f, 0.f}};   // repulsive energy, density
-        // the next entry's atom loads while this pair is evaluated
+        // the atom one pair ahead and the entry two ahead load meanwhile
         uint32_t e_nx = lane < m ? b.nbr[(size_t)lane * b.n + i] : (uint32_t)i;
+        uint32_t e_n2 = lane + L < m ? b.nbr[(size_t)(lane + L) * b.n + i] : (uint32_t)i;
         lvec4 q_nx = ld_lvec4_l2(b.xq64 + (e_nx & kIdxMask));
         for (int k = lane; k < m; k += L) {
             const uint32_t en = e_nx;
             const lvec4 qj = q_nx;
-            if (k + L < m) {
-                e_nx = b.nbr[(size_t)(k + L) * b.n + i];
-                q_nx = ld_lvec4_l2(b.xq64 + (e_nx & kIdxMask));
-            }
+            e_nx = e_n2;
+            if (k + L < m) q_nx = ld_lvec4_l2(b.xq64 + (e_nx & kIdxMask));
+            if (k + 2 * L < m) e_n2 = b.nbr[(size_t)(k + 2 * L) * b.n + i];
             const ffloat r2 = ff_norm2(pair_sep_ff(qt, qi, qj, en));
             if (!(r2.hi < P.rc2_f)) continue;
             ffloat2 v;
@@ -169,14 +169,14 @@ __device__ __forceinline__ void loop_force(const Bufs& b, const PotC& P, const l
         ffloat2 fxy = {{0.f, 0.f}, {0.f, 0.f}};
         ffloat fz = {0.f, 0.f};
         uint32_t e_nx = lane < m ? b.nbr[(size_t)lane * b.n + i] : (uint32_t)i;
+        uint32_t e_n2 = lane + L < m ? b.nbr[(size_t)(lane + L) * b.n + i] : (uint32_t)i;
         lvec4 q_nx = ld_lvec4_l2(b.xq64 + (e_nx & kIdxMask));
         for (int k = lane; k < m; k += L) {
             const uint32_t en = e_nx;
             const lvec4 qj = q_nx;
-            if (k + L < m) {
-                e_nx = b.nbr[(size_t)(k + L) * b.n + i];
-                q_nx = ld_lvec4_l2(b.xq64 + (e_nx & kIdxMask));
-            }
+            e_nx = e_n2;
+            if (k + L < m) q_nx = ld_lvec4_l2(b.xq64 + (e_nx & kIdxMask));
+            if (k + 2 * L < m) e_n2 = b.nbr[(size_t)(k + 2 * L) * b.n + i];
             const ffvec d = pair_sep_ff(qt, qi, qj, en);
             const ffloat r2 = ff_norm2(d);
             if (!(r2.hi < P.rc2_f)) continue;
