@@ -686,14 +686,35 @@ LoopKernel loop_kernel(const fire_handle* h, const LoopShape& q) {
                         : loop_kernel_t<true, 4>(q.threads);
 }
 
+// Launches the resident loop on s (directly or under capture).
+cudaError_t launch_loop(fire_handle* h, const GeoC& g, cudaStream_t s, bool eval,
+                        cudaGraphConditionalHandle hw) {
+    const LoopShape q = loop_shape(h);
+    const LoopKernel kern = loop_kernel(h, q);
+    const size_t smem = loop_smem(q.share);
+    cudaError_t e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e == cudaSuccess && !h->loop_rows)
+        e = cudaMalloc(&h->loop_rows, (size_t)kLoopRows * h->sms * sizeof(double));
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)q.blocks, 1, 1);
+    cfg.blockDim = dim3((unsigned)q.threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, h->b, h->potc, g, LoopC{h->loop_rows, q.share, eval ? 1 : 0},
+                              hw);
+}
+
 // The resident loop as a graph: prepare; WHILE (not stopped): list build,
 // k_loop (which sets the condition); finalize.
 fire_status build_loop_graph(fire_handle* h, const GeoC& g) {
     drop_graph(h);
-    const LoopShape q = loop_shape(h);
-    const LoopKernel kern = loop_kernel(h, q);
-    const size_t smem = loop_smem(q.share);
-    CK(h, cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (!h->loop_rows) CK(h, cudaMalloc(&h->loop_rows, (size_t)kLoopRows * h->sms * sizeof(double)));
     cudaGraph_t graph = nullptr;
     CK(h, cudaGraphCreate(&graph, 0));
@@ -714,17 +735,7 @@ fire_status build_loop_graph(fire_handle* h, const GeoC& g) {
                                           cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
         launch_build(h, g, 1, h->cap1);
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)q.blocks, 1, 1);
-        cfg.blockDim = dim3((unsigned)q.threads, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = h->cap1;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeCooperative;
-        attr[0].val.cooperative = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, kern, h->b, h->potc, g, LoopC{h->loop_rows, q.share}, hw);
+        e = launch_loop(h, g, h->cap1, false, hw);
         cudaGraph_t body_out = nullptr;
         const cudaError_t e1 = cudaStreamEndCapture(h->cap1, &body_out);
         if (e == cudaSuccess) e = e1;
@@ -1516,6 +1527,22 @@ static fire_status prepare_relax(fire_handle* h, const double box[3], GeoC* g) {
     return h->loop_ok ? FIRE_OK : prepare_call(h, box, g, false, true);
 }
 
+// The same before an evaluation, which launches the kernel itself: whether a
+// cooperative launch of it fits (loop_ok stays untried for the graph).
+static fire_status prepare_eval(fire_handle* h, const double box[3], GeoC* g) {
+    fire_status st = prepare_call(h, box, g, false, true);
+    if (st != FIRE_OK || !h->loop) return st;
+    int coop = 0, occ = 0;
+    const LoopShape q = loop_shape(h);
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device) == cudaSuccess && coop &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)loop_kernel(h, q), q.threads,
+                                                      loop_smem(q.share)) == cudaSuccess && occ >= 1)
+        return FIRE_OK;
+    cudaGetLastError();
+    h->loop_ok = 0;
+    return prepare_call(h, box, g, false, true);
+}
+
 // One relaxation on the device: positions are already in b.pos_io.
 static fire_status run_minimize(fire_handle* h, const GeoC& g, double ftol, int64_t maxiter,
                                 cudaStream_t s) {
@@ -1672,9 +1699,13 @@ static fire_status run_eval_unmasked(fire_handle* h, const GeoC& g, cudaStream_t
     CK(h, cudaMemcpyAsync(h->b.st, h->h_state, sizeof(DevState), cudaMemcpyHostToDevice, s));
     k_prepare<<<ceil_div(h->n, kElemBlock), kElemBlock, 0, s>>>(h->b);
     launch_build(h, g, 1, s);
-    launch_forces(h, g, s);
-    launch_reduce_control(h, g, s, CTL_EVAL, cudaGraphConditionalHandle{}, 0);
-    k_export_forces<<<ceil_div(h->n, kElemBlock), kElemBlock, 0, s>>>(h->b);
+    if (h->loop) {   // both passes, the sums and the export in one launch
+        CK(h, launch_loop(h, g, s, true, cudaGraphConditionalHandle{}));
+    } else {
+        launch_forces(h, g, s);
+        launch_reduce_control(h, g, s, CTL_EVAL, cudaGraphConditionalHandle{}, 0);
+        k_export_forces<<<ceil_div(h->n, kElemBlock), kElemBlock, 0, s>>>(h->b);
+    }
     CK(h, cudaGetLastError());
     CK(h, cudaMemcpyAsync(h->h_state, h->b.st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
     CK(h, cudaStreamSynchronize(s));
@@ -1686,7 +1717,7 @@ fire_status fire_energy_forces_dev(fire_handle_t* h, const double* d_pos, const 
     if (!h) return FIRE_ERR_ARG;
     if (!d_pos) return fail(h, FIRE_ERR_ARG, "NULL positions");
     GeoC g;
-    fire_status st = prepare_call(h, box, &g);
+    fire_status st = prepare_eval(h, box, &g);
     if (st != FIRE_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
     const size_t bytes = (size_t)3 * h->n * sizeof(double);
@@ -1709,7 +1740,7 @@ fire_status fire_energy_forces(fire_handle_t* h, const double* pos, const double
     if (!h) return FIRE_ERR_ARG;
     if (!pos) return fail(h, FIRE_ERR_ARG, "NULL positions");
     GeoC g;
-    fire_status st = prepare_call(h, box, &g);
+    fire_status st = prepare_eval(h, box, &g);
     if (st != FIRE_OK) return st;
     cudaStream_t s = h->stream;
     const size_t bytes = (size_t)3 * h->n * sizeof(double);

@@ -41,6 +41,7 @@ constexpr unsigned long long kLoopWaitNs = 5000000000ull;
 struct LoopC {
     double* rows;          // kLoopRows x gridDim.x partials
     int share;             // atoms per block (the last block may have fewer)
+    int eval;              // 1: one evaluation (F to b.f and b.f_out, E to b.e_out)
 };
 
 // Shared-memory bytes of a block that owns `share` atoms.
@@ -310,6 +311,24 @@ static __device__ __noinline__ void loop_control(LoopShared& sh) {
     sh.stop = stop ? 1 : 0;
 }
 
+// The end of one evaluation: forces, energy and state out.
+__device__ __forceinline__ void loop_export(const Bufs& b, int i0, int own, int share, const double* f,
+                                            const LoopShared& sh) {
+    for (int a = threadIdx.x; a < own; a += blockDim.x)
+        f_store(b, i0 + a, f[a], f[share + a], f[2 * share + a]);
+    if (b.f_out)
+        for (int k = threadIdx.x; k < 3 * own; k += blockDim.x)
+            b.f_out[3 * (size_t)i0 + k] = f[(k % 3) * share + k / 3];
+    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+    const double E = sh.sum[3], F2 = sh.sum[1];
+    if (b.e_out) *b.e_out = E;
+    b.st->energy = E;
+    b.st->F2 = F2;
+    b.st->fmax2 = sh.sum[4];
+    b.st->finf = sh.sum[5];
+    if (b.st->status == ST_OK && (!isfinite(E) || !isfinite(F2))) b.st->status = ST_NONFINITE;
+}
+
 // The element-wise step of the block's atoms; returns this thread's largest
 // squared displacement since the list build.
 template <bool RGL, bool KICK>
@@ -416,6 +435,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_loop(Bufs b, PotC P, GeoC g, LoopC 
         loop_partials(acc, status, c, sh);
         if (!(ok = loop_barrier(st, target, sh, false, votes))) break;
         loop_sums(c, sh);
+        if (c.eval) {
+            loop_export(b, i0, own, share, f, sh);
+            return;
+        }
         if (threadIdx.x == 0) loop_control(sh);
         __syncthreads();
         if (sh.stop) break;
