@@ -424,7 +424,7 @@ void launch_lists(const Bufs& b, const GeoC& g, int sms, int force, cudaStream_t
     k_cell_fill<<<ceil_div(n, kElemBlock), kElemBlock, 0, s>>>(b, g, force);
     k_cell_sort<<<ceil_div(32ll * b.ncell, kElemBlock), kElemBlock, 0, s>>>(b, g, force);
     // a block per cell; 16 warps where the cells do not give every SM four blocks
-    // of 4 (497 atoms 51 -> 37 us, 3,960 atoms 55 -> 39 us the whole build)
+    // of 4 (497 atoms 51 -> 36 us, 3,960 atoms 55 -> 39 us the whole build)
     constexpr int W = kBuildWarps, WS = kBuildWarpsSmall;
     if (b.ncell < 4 * sms) {
         k_nbr_build<WS><<<b.ncell, 32 * WS, 0, s>>>(b, g, force, 1);

@@ -404,10 +404,11 @@ __device__ __forceinline__ void build_count(DevState* st) {
 // shared memory by the block, and ballots give the entries their places in
 // candidate order.  With a thread per atom (each lane walking cells of its own)
 // the lanes diverged at every cell and small systems had a few dozen warps;
-// the whole build, thread / warp per atom: 255 LJ atoms (all pairs) 111 / 9 us,
-// 497 atoms 177 / 37, 3,960 atoms 203 / 40, 31,680 atoms 228 / 74, 119,023
-// atoms 248 / 138, 997,450 atoms 1422 / 924 (half list) and 1467 / 1114 us
-// (full list).  Bound by the issue of the FP32 tests (67 % of the slots).
+// the whole build, thread per atom / now: 255 LJ atoms (all pairs) 111 / 9 us,
+// 497 atoms 177 / 36, 3,960 atoms 203 / 39, 31,680 atoms 228 / 69, 119,023
+// atoms 248 / 115, 997,450 atoms 1422 / 718 (half list) and 1467 / 921 us (full
+// list).  Bound by the issue of the FP32 tests; 9 blocks of 4 warps per SM (56
+// registers; 8, 10 or 12 blocks 1-3 % slower at 1M atoms).
 constexpr int kSkinBuf = 24;
 constexpr int kBuildWarps = 4;       // warps per block, and on small systems (few
 constexpr int kBuildWarpsSmall = 16; // blocks): an atom per warp
@@ -443,73 +444,113 @@ __device__ __forceinline__ bool build_far(const GeoC& g, float4 x) {
            !(fabsf(x.z) * build_linv(g, 2) < 0x1p19f);
 }
 
+// Separation of candidate xj from the atom at xi (minimum image) and its square.
+struct BuildSep {
+    float dx, dy, dz, sx, sy, sz, r2;
+};
+template <int MODE>
+__device__ __forceinline__ BuildSep build_sep(const GeoC& g, float4 xi, float4 xj) {
+    BuildSep d;
+    d.dx = build_image<MODE>(xj.x - xi.x, g.Lf[0], build_linv(g, 0), d.sx);
+    d.dy = build_image<MODE>(xj.y - xi.y, g.Lf[1], build_linv(g, 1), d.sy);
+    d.dz = build_image<MODE>(xj.z - xi.z, g.Lf[2], build_linv(g, 2), d.sz);
+    d.r2 = __fmaf_rn(d.dz, d.dz, __fmaf_rn(d.dy, d.dy, __fmul_rn(d.dx, d.dx)));
+    return d;
+}
+
+// Writes the list entries of the accepted candidates hit[0, m), m <= 32, of
+// atom i, one per lane, in their order; drops the atom itself and, of a half
+// list, the pairs in its plane that are the other atom's.
+template <int MODE>
+__device__ __forceinline__ void build_emit(const Bufs& b, const GeoC& g, int i, float4 xi,
+                                           const float4* cand, const uint16_t* hit, int m,
+                                           uint32_t* skin, ListState& L) {
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    bool ok = lane < m;
+    const float4 xj = cand[ok ? hit[lane] : hit[0]];
+    const BuildSep d = build_sep<MODE>(g, xi, xj);
+    const int j = __float_as_int(xj.w);
+    ok = ok && j != i && (g.full || upper_half(d.dx, d.dy, d.dz));
+    // image codes cover shifts of -2..2 box lengths; atoms further apart than
+    // that in raw coordinates are a caller error (positions far outside the box)
+    if (MODE != IMG_NONE) {
+        const bool range = ok && !(fmaxf(fabsf(d.sx), fmaxf(fabsf(d.sy), fabsf(d.sz))) <= 2.f);
+        if (range) set_status(b.st, ST_RANGE);
+        ok = ok && !range;
+    }
+    const bool in = ok && d.r2 < g.rc2f;
+    const unsigned bi = __ballot_sync(0xffffffffu, in);
+    const unsigned bs = __ballot_sync(0xffffffffu, ok) & ~bi;
+    // exact in FP32; the integer is in the sum's low bits
+    const uint32_t code =
+        (uint32_t)__float_as_int(d.sx + 5.f * d.sy + 25.f * d.sz + (62.f + 0x1p23f)) & 0x7fu;
+    const uint32_t e = (code << kIdxBits) | (uint32_t)j;
+    uint32_t* out = b.nbr + i;
+    if (L.skin + __popc(bs) <= kSkinBuf) {
+        const int at = (in ? L.cnt : L.skin) + __popc((in ? bi : bs) & below);
+        if (in) {
+            if (at < b.cap) out[(size_t)at * b.n] = e;
+        } else if (ok) {
+            skin[at] = e;
+        }
+        L.cnt += __popc(bi);
+        L.skin += __popc(bs);
+    } else {   // the buffer is full: the rest among the in-range ones
+        const int rank = L.skin + __popc(bs & below);
+        const bool now = in || (ok && rank >= kSkinBuf);
+        const unsigned bn = __ballot_sync(0xffffffffu, now);
+        const int at = L.cnt + __popc(bn & below);
+        if (ok && !now) skin[rank] = e;
+        if (now && at < b.cap) out[(size_t)at * b.n] = e;
+        L.cnt += __popc(bn);
+        L.skin = kSkinBuf;
+    }
+}
+
 // Candidate test in FP32 (the FP64 unit is ~58x slower on this part): the
 // list radius carries a margin larger than the FP32 rounding of the
 // positions, so every pair closer than rc + skin is kept; the force kernels
 // test r < rc again.  The warp's lanes test candidates [0, m) (position, index
-// in w; NaN up to the next multiple of 32) against atom i at xi.
+// in w; NaN up to the next multiple of 32) against atom i at xi.  Accepted
+// ones (15 % of a stencil, so that nearly every set of 32 holds some) queue up
+// in hit and their entries are written 32 at a time (the build of the 1M-atom box
+// 924 -> 857 us; 718 with the tests of the own index and of the half space's
+// boundary plane left to the accepted ones and the staging below).
 template <int MODE>
 __device__ __forceinline__ void build_scan(const Bufs& b, const GeoC& g, int i, float4 xi,
-                                           const float4* cand, int m, uint32_t* skin,
-                                           ListState& L) {
-    const int lane = threadIdx.x & 31, full = g.full;
+                                           const float4* cand, int m, uint16_t* hit,
+                                           uint32_t* skin, ListState& L) {
+    const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
-    const float lx = build_linv(g, 0), ly = build_linv(g, 1), lz = build_linv(g, 2);
-    const float Lx = g.Lf[0], Ly = g.Lf[1], Lz = g.Lf[2], rl2 = g.rlist2f, rc2 = g.rc2f;
-    uint32_t* out = b.nbr + i;
+    const float rl2 = g.rlist2f, zmin = g.full ? -INFINITY : 0.f;
+    int q = 0;
     for (int k = lane; k < m + lane; k += 32) {   // the warp stays together
         const float4 xj = cand[k];
-        const int j = __float_as_int(xj.w);
-        float sx, sy, sz;
-        const float dx = build_image<MODE>(xj.x - xi.x, Lx, lx, sx);
-        const float dy = build_image<MODE>(xj.y - xi.y, Ly, ly, sy);
-        const float dz = build_image<MODE>(xj.z - xi.z, Lz, lz, sz);
-        const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
-        bool ok = r2 < rl2 && j != i && (full || upper_half(dx, dy, dz));   // NaN fails
+        const BuildSep d = build_sep<MODE>(g, xi, xj);
+        const bool ok = d.r2 < rl2 && d.dz >= zmin;   // NaN fails
         const unsigned any = __ballot_sync(0xffffffffu, ok);
-        if (any == 0u) continue;
-        // image codes cover shifts of -2..2 box lengths; atoms further apart than
-        // that in raw coordinates are a caller error (positions far outside the box)
-        if (MODE != IMG_NONE) {
-            const bool range = ok && !(fmaxf(fabsf(sx), fmaxf(fabsf(sy), fabsf(sz))) <= 2.f);
-            if (__any_sync(0xffffffffu, range)) {
-                if (range) set_status(b.st, ST_RANGE);
-                ok = ok && !range;
-            }
-        }
-        const bool in = ok && r2 < rc2;
-        const unsigned bi = __ballot_sync(0xffffffffu, in);
-        const unsigned bs = __ballot_sync(0xffffffffu, ok) & ~bi;
-        // exact in FP32; the integer is in the sum's low bits
-        const uint32_t code = (uint32_t)__float_as_int(sx + 5.f * sy + 25.f * sz + (62.f + 0x1p23f)) & 0x7fu;
-        const uint32_t e = (code << kIdxBits) | (uint32_t)j;
-        if (L.skin + __popc(bs) <= kSkinBuf) {
-            const int at = (in ? L.cnt : L.skin) + __popc((in ? bi : bs) & below);
-            if (in) {
-                if (at < b.cap) out[(size_t)at * b.n] = e;
-            } else if (ok) {
-                skin[at] = e;
-            }
-            L.cnt += __popc(bi);
-            L.skin += __popc(bs);
-        } else {   // the buffer is full: the rest among the in-range ones
-            const int rank = L.skin + __popc(bs & below);
-            const bool now = in || (ok && rank >= kSkinBuf);
-            const unsigned bn = __ballot_sync(0xffffffffu, now);
-            const int at = L.cnt + __popc(bn & below);
-            if (ok && !now) skin[rank] = e;
-            if (now && at < b.cap) out[(size_t)at * b.n] = e;
-            L.cnt += __popc(bn);
-            L.skin = kSkinBuf;
-        }
+        if (ok) hit[q + __popc(any & below)] = (uint16_t)k;
+        q += __popc(any);
+        if (q < 32) continue;
+        __syncwarp();
+        build_emit<MODE>(b, g, i, xi, cand, hit, 32, skin, L);
+        q -= 32;
+        const uint16_t rest = hit[32 + lane];
+        __syncwarp();
+        if (lane < q) hit[lane] = rest;
     }
+    if (q == 0) return;
+    __syncwarp();
+    build_emit<MODE>(b, g, i, xi, cand, hit, q, skin, L);
+    __syncwarp();
 }
 
 // The rare form, out of line.
 __device__ __noinline__ ListState build_scan_far(const Bufs& b, const GeoC& g, int i, float4 xi,
-                                                 const float4* cand, int m, uint32_t* skin,
-                                                 ListState L) {
-    build_scan<IMG_FAR>(b, g, i, xi, cand, m, skin, L);
+                                                 const float4* cand, int m, uint16_t* hit,
+                                                 uint32_t* skin, ListState L) {
+    build_scan<IMG_FAR>(b, g, i, xi, cand, m, hit, skin, L);
     return L;
 }
 
@@ -531,6 +572,7 @@ template <int W>
 struct BuildShared {
     float4 cand[kBuildCand];
     uint32_t skin[W][kSkinBuf];
+    uint16_t hit[W][64];
     int beg[27], off[28], wrap;   // wrap: a pair of the stencil may be across a face
 };
 // NaN candidates after m up to the next multiple of 32 (kBuildCand is one).
@@ -566,9 +608,9 @@ __global__ void __launch_bounds__(32 * kBuildWarps) k_nbr_build_all(Bufs b, GeoC
         far = __syncthreads_or(far);
         if (!on) continue;
         if (far)
-            L = build_scan_far(b, g, i, xi, sh.cand, m, sh.skin[w], L);
+            L = build_scan_far(b, g, i, xi, sh.cand, m, sh.hit[w], sh.skin[w], L);
         else
-            build_scan<IMG_NEAR>(b, g, i, xi, sh.cand, m, sh.skin[w], L);
+            build_scan<IMG_NEAR>(b, g, i, xi, sh.cand, m, sh.hit[w], sh.skin[w], L);
     }
     if (!on) return;
     build_finish(b, i, sh.skin[w], L);
@@ -583,9 +625,9 @@ __device__ __forceinline__ void build_cell(const Bufs& b, const GeoC& g, int c, 
     float4* cand = sh.cand;
     int *beg = sh.beg, *off = sh.off;
     const int p0 = b.cell_start[c], na = b.cell_start[c + 1] - p0;
-    if (na == 0) return;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t* skin = sh.skin[w];
+    uint16_t* hit = sh.hit[w];
     if (w == 0) {
         // this cell's coordinates (the inverse of cell_index), its stencil's
         // runs in the order (x, y, z) of the offsets
@@ -602,20 +644,26 @@ __device__ __forceinline__ void build_cell(const Bufs& b, const GeoC& g, int c, 
             const int az = cell_step(cz, lane % 3 - 1, g.nc[2], g.per[2]);
             if (ax >= 0 && ay >= 0 && az >= 0) {
                 const int nb = cell_index(g, img, ax, ay, az);
-                beg[lane] = b.cell_start[nb];
-                len = b.cell_start[nb + 1] - beg[lane];
+                // all loads at once (an empty cell's extremes are not used)
+                const int p = b.cell_start[nb], q = b.cell_start[nb + 1];
+                float2 xi[3], xj[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    xi[a] = b.cell_box[3 * (size_t)c + a];
+                    xj[a] = b.cell_box[3 * (size_t)nb + a];
+                }
+                beg[lane] = p;
+                len = q - p;
                 // FP32 subtraction, multiplication and rounding are monotonic:
                 // every pair's separation and image lie between those of the
                 // two cells' extremes.
-                if (len > 0) {
+                if (len > 0 && na > 0) {
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
-                        const float2 xi = b.cell_box[3 * (size_t)c + a];
-                        const float2 xj = b.cell_box[3 * (size_t)nb + a];
                         const float li = build_linv(g, a);
                         float s0, s1;
-                        const float d0 = build_image<IMG_FAR>(xj.x - xi.y, g.Lf[a], li, s0);
-                        const float d1 = build_image<IMG_FAR>(xj.y - xi.x, g.Lf[a], li, s1);
+                        const float d0 = build_image<IMG_FAR>(xj[a].x - xi[a].y, g.Lf[a], li, s0);
+                        const float d1 = build_image<IMG_FAR>(xj[a].y - xi[a].x, g.Lf[a], li, s1);
                         wrap = wrap || s0 != 0.f || s1 != 0.f;
                         // half list: a run whose atoms all lie below this
                         // cell's (the layer under it, as a rule) has no pair in
@@ -637,18 +685,35 @@ __device__ __forceinline__ void build_cell(const Bufs& b, const GeoC& g, int c, 
     }
     __syncthreads();
     const int total = off[27];
-    // candidates [from, from + kBuildCand) of the stencil; whether any is far
+    if (na == 0) return;
+    // candidates [from, from + kBuildCand) of the stencil; whether any is far.
+    // A thread loads two at once (one in blocks of 16 warps), the run found by
+    // bisection; a run per warp, one after another, waits for 27 / W loads in turn.
     auto stage = [&](int from) {
+        constexpr int T = 32 * W, U = W >= 16 ? 1 : 2;
+        const int m = min(kBuildCand, total - from);
         bool far = false;
-        for (int r = w; r < 27; r += W) {
-            const int lo = max(off[r], from), hi = min(off[r + 1], from + kBuildCand);
-            for (int k = lo + lane; k < hi; k += 32) {
-                const float4 x = b.xs[beg[r] + k - off[r]];
-                cand[k - from] = x;
-                far = far || build_far(g, x);
+        for (int k0 = threadIdx.x; k0 < m; k0 += U * T) {
+            float4 x[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int k = k0 + u * T, t = from + k;
+                if (k >= m) continue;
+                int r = 0;   // the last run that starts at t or before
+#pragma unroll
+                for (int st = 16; st > 0; st >>= 1)
+                    if (r + st < 27 && off[r + st] <= t) r += st;
+                x[u] = b.xs[beg[r] + t - off[r]];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int k = k0 + u * T;
+                if (k >= m) continue;
+                cand[k] = x[u];
+                far = far || build_far(g, x[u]);
             }
         }
-        build_pad(cand, min(kBuildCand, total - from));
+        build_pad(cand, m);
         return __syncthreads_or(far) != 0;
     };
     const bool once = total <= kBuildCand, wrap = sh.wrap != 0;
@@ -666,11 +731,11 @@ __device__ __forceinline__ void build_cell(const Bufs& b, const GeoC& g, int c, 
             if (!on) continue;
             const int m = min(kBuildCand, total - from);
             if (!wrap)
-                build_scan<IMG_NONE>(b, g, i, xi, cand, m, skin, L);
+                build_scan<IMG_NONE>(b, g, i, xi, cand, m, hit, skin, L);
             else if (far || build_far(g, xi))
-                L = build_scan_far(b, g, i, xi, cand, m, skin, L);
+                L = build_scan_far(b, g, i, xi, cand, m, hit, skin, L);
             else
-                build_scan<IMG_NEAR>(b, g, i, xi, cand, m, skin, L);
+                build_scan<IMG_NEAR>(b, g, i, xi, cand, m, hit, skin, L);
         }
         if (on) build_finish(b, i, skin, L);
     }
@@ -679,7 +744,7 @@ __device__ __forceinline__ void build_cell(const Bufs& b, const GeoC& g, int c, 
 // are empty (a cluster in a large open box), of which the block takes the
 // occupied ones.
 template <int W>
-__global__ void __launch_bounds__(32 * W) k_nbr_build(Bufs b, GeoC g, int force, int cells) {
+__global__ void __launch_bounds__(32 * W, W == kBuildWarps ? 9 : 2) k_nbr_build(Bufs b, GeoC g, int force, int cells) {
     __shared__ BuildShared<W> sh;
     if (!need_rebuild(b.st, g, force)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) build_count(b.st);
@@ -1275,7 +1340,7 @@ __global__ void __launch_bounds__(BLK) k_force32(Bufs b, PotC P, GeoC g) {
 }
 
 // ---------------------------------------------------------------------------
-// Tabulated RGL passes (quintic Hermite tables in u = r^2 - r0^2, held in
+// Tabulated RGL passes (FP32: quintic Hermite tables in u = r^2 - r0^2, held in
 // shared memory; persistent grids stride over the atoms so each block loads
 // the table once).  Pairs closer than r0/2 fall back to the analytic terms.
 
@@ -1287,7 +1352,7 @@ __device__ __forceinline__ void load_table(T* dst, const T* src, int count) {
 // ---------------------------------------------------------------------------
 // FP64 form, tabulated RGL on the full list with no FP64 instruction per
 // pair (fire2_table.cuh): exact fixed-point separations, double-float r^2,
-// interval offsets, quintics and per-atom sums.  One atom per thread, no
+// interval offsets, quartics and per-atom sums.  One atom per thread, no
 // atomics: every atom's sums are complete in its own thread.
 
 __device__ __forceinline__ void fill_qshift64_table(long long* qt, const GeoC& g) {
