@@ -97,7 +97,7 @@ def parse():
     ap.add_argument("--config", default="rgl1m", choices=sorted(CONFIGS))
     ap.add_argument("--form", default="fp64", choices=["fp64", "fp32pair"])
     ap.add_argument("--pair", default=None, choices=["table", "analytic"],
-                    help="RGL pair functions: quintic tables or exponentials (default: "
+                    help="RGL pair functions: tables or exponentials (default: "
                          "tables for fp64, exponentials for fp32pair, the faster of each)")
     ap.add_argument("--newton", default="auto", choices=["auto", "on", "off"],
                     help="FP64 tabulated form: half list + atomics (on) or full list (off)")
@@ -351,6 +351,15 @@ def tiles_active(args, form, pair, n):
     return args.tiles == "on"
 
 
+def resident_active(args, form, pair, n, is_rgl):
+    """Whether the library relaxes the system in its resident loop kernel."""
+    if args.exec == "chunked" or form != "fp64":
+        return False
+    if not is_rgl:
+        return n <= 16384
+    return pair == "table" and args.newton == "auto" and args.tiles != "on" and n <= 65536
+
+
 def default_pair(form):
     return "analytic" if form == "fp32pair" else "table"
 
@@ -402,7 +411,8 @@ class _NoClock:
         return None
 
 
-def launches_of(results, is_rgl, fp32, cell_mode, chunked=False, tiled=False, body=8, chunk=32):
+def launches_of(results, is_rgl, fp32, cell_mode, chunked=False, tiled=False, body=8, chunk=32,
+                resident=False):
     """Kernels one relaxation launches: prepare, list build, forces, the
     reductions with the control step (one launch), finalize once; then the
     loop passes, launched a whole WHILE body (`body` iterations, graph mode)
@@ -414,9 +424,13 @@ def launches_of(results, is_rgl, fp32, cell_mode, chunked=False, tiled=False, bo
     FP32-pair form also has the two FP64 confirming passes: launched once in
     the set-up, then in the graph loop only in the passes that confirm a
     stop (an IF node), in the chunked loop with every pass.  Each
-    confirmation is one more loop pass (force evaluations - iterations - 1)."""
+    confirmation is one more loop pass (force evaluations - iterations - 1).
+    The resident loop (small systems) launches prepare and finalize, and the
+    build chain and the loop kernel once per list."""
     build_k = (6 + (1 if tiled else 0)) if cell_mode else 1
     force_k = (2 if fp32 else 3) if is_rgl else 1
+    if resident:
+        return sum(2 + rr["nbr_builds"] * (build_k + 1) for rr in results)
     per = chunk if chunked else body
     total = 0
     for rr in results:
@@ -1094,7 +1108,8 @@ def run_gpu(args):
                       "nbr_builds": [rr["nbr_builds"] for rr in results],
                       "l2": "inputs larger than L2 (working set > 1 GB at 1M atoms)"},
            "gpu_launches": launches_of(results, is_rgl, fp32, cell_mode, args.exec == "chunked",
-                                       tiles_active(args, args.form, pair, n)),
+                                       tiles_active(args, args.form, pair, n),
+                                       resident=resident_active(args, args.form, pair, n, is_rgl)),
            "clocks": m["clocks"]}
 
     # per-stage device times (CUDA events) for the roofline of the dominant kernel

@@ -94,7 +94,8 @@ typedef enum {
  * FIRE_NEWTON_ON: each pair once (half list), its terms added to both atoms
  * by FP64 atomics.  FIRE_NEWTON_OFF: full list, every pair from both ends,
  * no atomics (results reproducible bit for bit).  FIRE_NEWTON_AUTO: the
- * library's default for this part (FIRE_NEWTON_ON). */
+ * faster of the two at the handle's size: full lists in the resident loop
+ * (up to 65,536 atoms; fire_set_exec_mode), half lists otherwise. */
 typedef enum {
     FIRE_NEWTON_AUTO = 0,
     FIRE_NEWTON_ON = 1,
@@ -281,7 +282,12 @@ typedef enum {
  * passes of FP32-pair handles under conditional IF nodes (an all-pairs list
  * build, used for boxes under three cells per axis, is launched in every
  * iteration and returns at once unless due; iterations past the stop return
- * at once too); 0 (the default) takes 8.  Results do not depend on the mode.
+ * at once too); 0 (the default) takes 8, and relaxes small single systems in
+ * one resident kernel per neighbour list instead: LJ up to 16,384 atoms, the
+ * FP64 table form with FIRE_NEWTON_AUTO up to 65,536, without a maximum
+ * displacement, pair tiles or a set number of threads per atom (energies and
+ * forces alone run there too).  Results do not depend on the mode, but for the
+ * rounding of sums.
  * The paper has no counterpart (it describes the loop of Algorithm 2, not how
  * it is driven).  Errors: FIRE_ERR_ARG. */
 fire_status fire_set_exec_mode(fire_handle_t* h, int32_t mode, int32_t chunk);
@@ -297,7 +303,8 @@ fire_status fire_set_exec_mode(fire_handle_t* h, int32_t mode, int32_t chunk);
  * take every tpa-th entry of its neighbour list and their partial sums are
  * added in FP64, so results change only in the rounding of the per-atom sums
  * (far below the FP64 form's 1e-10 relative force error).  Other forms run
- * one thread per atom and report 1.  *chosen (may be NULL) receives the value
+ * one thread per atom and report 1; a set tpa also keeps small systems out of
+ * the resident loop (fire_set_exec_mode).  *chosen (may be NULL) receives the value
  * in effect.  Applies to later calls on h; the paper has no counterpart (it
  * does not say how force evaluation is parallelised).
  * Errors: FIRE_ERR_ARG (another tpa; batched handles, which take their launch
