@@ -62,14 +62,12 @@ struct BArgs {
     int4* xq;
     float4* xf;
     lvec4* xq64;            // FP64 table form: positions in 2^-44 A units
-    float2* fpff;           // FP64 table form: F'(rho) as a float pair
     const float *tab_ffd, *tab_fff;   // FP64 table form: density / force rows
     int ff;                 // 1: FP64 table passes available (FP64 table form, or the
                             //    FP32-pair form confirming its stops)
     int confirm;            // FP32-pair form: FP64 check of its stops (confirm64 != 0)
     int vmode;              // fire_fp64_check: 1 confirm, 2 finish in FP64 below 3 ftol
-    double* fp64;           // F'(rho) (FP64 form)
-    float* fp32;            // F'(rho) (FP32-pair form)
+    double* fp64;           // F'(rho) (IEEE-FP64 form; the others keep it in xq.w, xq64.w)
     uint32_t* nbr;
     int* nnbr;
     double* pos_io;         // packed N x 3, in/out
@@ -248,17 +246,42 @@ static __device__ __noinline__ int b_build(const BArgs& a, const BInst& I, int l
     return (int)bmax((double)(bad != ST_OK ? bad : (over ? ST_NBR_OVERFLOW : 0)), red);
 }
 
+// F'(rho) of the FP64 table form from the record's fourth word.
+__device__ __forceinline__ ffloat fp_load(const lvec4& q) {
+    return {__uint_as_float((unsigned)((unsigned long long)q.w & 0xffffffffull)),
+            __uint_as_float((unsigned)((unsigned long long)q.w >> 32))};
+}
+
+// Image shifts by code in fixed point, in the shared memory that the list build
+// has left (kShiftInts ints).  Small boxes put wrapped pairs into nearly every
+// warp, and decoding the code took some 25 integer instructions each time: 512
+// systems, FP32-pair, 92 -> 83 ms together with F' in the position records.
+constexpr int kShiftInts = 376 + 750;
+struct BShift {
+    const int* q;
+    const long long* q64;
+};
+__device__ __forceinline__ void b_shifts(const BInst& I, int* smem) {
+    long long* q64 = reinterpret_cast<long long*>(smem + 376);
+    for (int t = threadIdx.x; t < 375; t += blockDim.x) {
+        const int c = t / 3, d = t % 3;
+        const int s = (d == 0 ? c % 5 : d == 1 ? c / 5 % 5 : c / 25) - 2;
+        smem[t] = (int)((unsigned)s * (unsigned)I.Lq[d]);
+        q64[t] = (long long)s * I.Lq64[d];
+    }
+    __syncthreads();
+}
+
 // Separation x_j - x_i - shift of list entry e in the FP64 table form: exact
 // in 2^-44 A fixed point, split into float pairs.
-__device__ __forceinline__ ffvec b_sep_ff(const BArgs& a, const BInst& I, const lvec4& qi,
+__device__ __forceinline__ ffvec b_sep_ff(const BShift& S, const lvec4& qi, const lvec4& qj,
                                           uint32_t e) {
-    const int j = (int)(e & kIdxMask), code = (int)(e >> kIdxBits);
-    const lvec4 qj = a.xq64[I.off + j];
+    const int code = (int)(e >> kIdxBits);
     long long ix = qj.x - qi.x, iy = qj.y - qi.y, iz = qj.z - qi.z;
     if (code != kCodeZero) {
-        ix -= (long long)(code % 5 - 2) * I.Lq64[0];
-        iy -= (long long)((code / 5) % 5 - 2) * I.Lq64[1];
-        iz -= (long long)(code / 25 - 2) * I.Lq64[2];
+        ix -= S.q64[3 * code];
+        iy -= S.q64[3 * code + 1];
+        iz -= S.q64[3 * code + 2];
     }
     return {fixed_to_ff2(ix, iy), fixed_to_ff(iz)};
 }
@@ -269,8 +292,10 @@ __device__ __forceinline__ ffvec b_sep_ff(const BArgs& a, const BInst& I, const 
 // every CTA's F'(rho) visible to the others.
 template <bool F32, bool CL>
 __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int lo, int hi,
-                                           const double* etab, const float* et32, double* red) {
+                                           const double* etab, const float* et32, const int* smem,
+                                         double* red) {
     const PotC& P = a.P;
+    const BShift S = {smem, reinterpret_cast<const long long*>(smem + 376)};
     const int T = blockDim.x, t = threadIdx.x;
     double e_sum = 0.0;
     // pass 1: densities, embedding derivative, atom energies
@@ -288,9 +313,9 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
                 const int4 qj = a.xq[I.off + j];
                 int dx = wrap_sub(qj.x, qi.x), dy = wrap_sub(qj.y, qi.y), dz = wrap_sub(qj.z, qi.z);
                 if (code != kCodeZero) {
-                    dx = wrap_sub(dx, (int)((unsigned)(code % 5 - 2) * (unsigned)I.Lq[0]));
-                    dy = wrap_sub(dy, (int)((unsigned)((code / 5) % 5 - 2) * (unsigned)I.Lq[1]));
-                    dz = wrap_sub(dz, (int)((unsigned)(code / 25 - 2) * (unsigned)I.Lq[2]));
+                    dx = wrap_sub(dx, S.q[3 * code]);
+                    dy = wrap_sub(dy, S.q[3 * code + 1]);
+                    dz = wrap_sub(dz, S.q[3 * code + 2]);
                 }
                 const long long r2q = (long long)dx * dx + (long long)dy * dy + (long long)dz * dz;
                 if (r2q >= P.rc2q) continue;
@@ -301,7 +326,8 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
             }
             const float rf = (float)rho.value();
             const float sq = sqrtf(rf);
-            a.fp32[gi] = rf > 0.f ? -0.5f / sq : 0.f;
+            // F' beside the position: one gather per pair in the force pass
+            a.xq[gi].w = __float_as_int(rf > 0.f ? -0.5f / sq : 0.f);
             e_sum += erep.value() - (double)sq;
         } else if (a.ff) {   // FP64 table form: double-float pair terms, FP64 embedding
             const lvec4 qi = a.xq64[gi];
@@ -310,7 +336,8 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
             for (int k = 0; k < m; ++k) {
                 const uint32_t e = e_nx;
                 if (k + 1 < m) e_nx = a.nbr[I.list_off + (long long)(k + 1) * I.n + i];
-                const ffloat r2 = ff_norm2(b_sep_ff(a, I, qi, e));
+                const lvec4 qj = a.xq64[I.off + (int)(e & kIdxMask)];
+                const ffloat r2 = ff_norm2(b_sep_ff(S, qi, qj, e));
                 if (!(r2.hi < P.rc2_f)) continue;
                 ffloat2 w;
                 if (r2.hi >= P.ff.r2_lo) {
@@ -326,8 +353,8 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
             double sq, fp;
             ffloat fpf;
             rgl_embed_dd(ff_to_f64(ff_second(acc)), sq, fp, fpf);
-            a.fp64[gi] = fp;
-            a.fpff[gi] = make_float2(fpf.hi, fpf.lo);
+            a.xq64[gi].w = (long long)((unsigned long long)__float_as_uint(fpf.hi) |
+                                       ((unsigned long long)__float_as_uint(fpf.lo) << 32));
             e_sum += ff_to_f64(ff_first(acc)) - sq;
         } else {
             const dvec4 xi = a.x[gi];
@@ -365,7 +392,7 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
         const int m = a.nnbr[gi];
         if (F32) {
             const int4 qi = a.xq[gi];
-            const float fpi = a.fp32[gi];
+            const float fpi = __int_as_float(qi.w);
             Kahan32 fx, fy, fz;
             uint32_t e_nx = m > 0 ? a.nbr[I.list_off + i] : 0u;   // the next entry loads ahead
             for (int k = 0; k < m; ++k) {
@@ -375,15 +402,15 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
                 const int4 qj = a.xq[I.off + j];
                 int dx = wrap_sub(qj.x, qi.x), dy = wrap_sub(qj.y, qi.y), dz = wrap_sub(qj.z, qi.z);
                 if (code != kCodeZero) {
-                    dx = wrap_sub(dx, (int)((unsigned)(code % 5 - 2) * (unsigned)I.Lq[0]));
-                    dy = wrap_sub(dy, (int)((unsigned)((code / 5) % 5 - 2) * (unsigned)I.Lq[1]));
-                    dz = wrap_sub(dz, (int)((unsigned)(code / 25 - 2) * (unsigned)I.Lq[2]));
+                    dx = wrap_sub(dx, S.q[3 * code]);
+                    dy = wrap_sub(dy, S.q[3 * code + 1]);
+                    dz = wrap_sub(dz, S.q[3 * code + 2]);
                 }
                 const long long r2q = (long long)dx * dx + (long long)dy * dy + (long long)dz * dz;
                 if (r2q >= P.rc2q) continue;
                 float rinv, phi, dphi, g, dg;
                 rgl_pair32(P, r2q, et32, rinv, phi, dphi, g, dg);
-                const float fs = (2.f * dphi + (fpi + a.fp32[I.off + j]) * dg) * rinv * P.qinv;
+                const float fs = (2.f * dphi + (fpi + __int_as_float(qj.w)) * dg) * rinv * P.qinv;
                 fx.add(fs * (float)dx);
                 fy.add(fs * (float)dy);
                 fz.add(fs * (float)dz);
@@ -391,15 +418,15 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
             a.f[gi] = make_dvec4(fx.value(), fy.value(), fz.value(), 0.0);
         } else if (a.ff) {
             const lvec4 qi = a.xq64[gi];
-            const float2 fpi2 = a.fpff[gi];
-            const ffloat fpi = {fpi2.x, fpi2.y};
+            const ffloat fpi = fp_load(qi);
             ffloat2 fxy = {{0.f, 0.f}, {0.f, 0.f}};
             ffloat fz = {0.f, 0.f};
             uint32_t e_nx = m > 0 ? a.nbr[I.list_off + i] : 0u;   // the next entry loads ahead
             for (int k = 0; k < m; ++k) {
                 const uint32_t e = e_nx;
                 if (k + 1 < m) e_nx = a.nbr[I.list_off + (long long)(k + 1) * I.n + i];
-                const ffvec d = b_sep_ff(a, I, qi, e);
+                const lvec4 qj = a.xq64[I.off + (int)(e & kIdxMask)];
+                const ffvec d = b_sep_ff(S, qi, qj, e);
                 const ffloat r2 = ff_norm2(d);
                 if (!(r2.hi < P.rc2_f)) continue;
                 ffloat c0, c1;
@@ -413,8 +440,7 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
                     c0 = f64_to_ff(2.0 * dphi * rinv);
                     c1 = f64_to_ff(dg * rinv);
                 }
-                const float2 fpj2 = a.fpff[I.off + (int)(e & kIdxMask)];
-                const ffloat fs = ff_madd(ff_add(fpi, {fpj2.x, fpj2.y}), c1, c0);
+                const ffloat fs = ff_madd(ff_add(fpi, fp_load(qj)), c1, c0);
                 const ffloat2 t = ff_mul2_neg(fs, d.xy);
                 fxy = ff_acc2_neg(fxy, t.hi, t.lo);
                 fz = ff_acc(fz, ff_mul_nn(fs, d.z));
@@ -630,8 +656,8 @@ __device__ __noinline__ void b_reduce_control(const BArgs& a, const BInst& I, in
 template <bool CL>
 __device__ __noinline__ double b_forces_confirm(const BArgs& a, const BInst& I, int lo, int hi,
                                                 const double* etab, const float* et32,
-                                                double* red) {
-    return b_forces<false, CL>(a, I, lo, hi, etab, et32, red);
+                                                const int* smem, double* red) {
+    return b_forces<false, CL>(a, I, lo, hi, etab, et32, smem, red);
 }
 
 // The batched relaxation.  CL = false: one CTA per system.  CL = true: the
@@ -649,7 +675,7 @@ __device__ __noinline__ double b_forces_confirm(const BArgs& a, const BInst& I, 
 template <bool F32, bool CL, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_batch_relax(BArgs a) {
     namespace cg = cooperative_groups;
-    extern __shared__ int smem[];
+    extern __shared__ __align__(16) int smem[];
     __shared__ double etab[kExpTableSize];
     __shared__ float et32[kExp32TableSize];
     __shared__ double red[32];
@@ -716,11 +742,12 @@ __global__ void __launch_bounds__(MAXT, 1) k_batch_relax(BArgs a) {
         if (CL) cg::this_cluster().sync();   // every CTA's positions before the list build
         else __syncthreads();
         int bst = b_build(a, I, lo, hi, s_count, s_start, s_atoms, red);
+        b_shifts(I, smem);
         if (threadIdx.x == 0) {
             if (bst != ST_OK && sh.status == ST_OK) sh.status = bst;
             sh.builds += 1;
         }
-        double E = b_forces<F32, CL>(a, I, lo, hi, etab, et32, red);
+        double E = b_forces<F32, CL>(a, I, lo, hi, etab, et32, smem, red);
         b_reduce_control<CL>(a, I, lo, hi, sh, X, E, red, t0);
         while (!sh.done) {
             if (F32 && sh.vstate == 2) {
@@ -733,7 +760,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_batch_relax(BArgs a) {
                 }
                 if (CL) cg::this_cluster().sync();
                 else __syncthreads();
-                E = b_forces_confirm<CL>(a, I, lo, hi, etab, et32, red);
+                E = b_forces_confirm<CL>(a, I, lo, hi, etab, et32, smem, red);
                 b_reduce_control<CL>(a, I, lo, hi, sh, X, E, red, t0);
                 continue;
             }
@@ -764,13 +791,14 @@ __global__ void __launch_bounds__(MAXT, 1) k_batch_relax(BArgs a) {
             cl_combine<CL>(X, &db, 0, 1);
             if (X.res[0] > I.half_skin2) {
                 bst = b_build(a, I, lo, hi, s_count, s_start, s_atoms, red);
+                b_shifts(I, smem);
                 if (threadIdx.x == 0) {
                     if (bst != ST_OK && sh.status == ST_OK) sh.status = bst;
                     sh.builds += 1;
                 }
             }
-            E = fp64_phase ? b_forces_confirm<CL>(a, I, lo, hi, etab, et32, red)
-                           : b_forces<F32, CL>(a, I, lo, hi, etab, et32, red);
+            E = fp64_phase ? b_forces_confirm<CL>(a, I, lo, hi, etab, et32, smem, red)
+                           : b_forces<F32, CL>(a, I, lo, hi, etab, et32, smem, red);
             b_reduce_control<CL>(a, I, lo, hi, sh, X, E, red, t0);
         }
         // write back
@@ -858,7 +886,7 @@ cudaStream_t fire2_stream(fire_handle_t* h);
 static void free_batch(fire_batch_state* b) {
     if (!b) return;
     BArgs& a = b->args;
-    void* ptrs[] = {a.x, a.v, a.f, a.xref, a.xq, a.xf, a.xq64, a.fpff, a.fp64, a.fp32, a.nbr,
+    void* ptrs[] = {a.x, a.v, a.f, a.xref, a.xq, a.xf, a.xq64, a.fp64, a.nbr,
                     a.nnbr, a.pos_io,
                     b->d_inst, b->d_res, b->d_order, b->d_queue};
     for (void* p : ptrs)
@@ -922,7 +950,7 @@ static fire_status batch_geometry(fire_handle_t* h, fire_batch_state* b, const d
     }
     b->args.max_cells = max_cells;
     b->args.max_atoms_smem = max_atoms;
-    b->smem_bytes = (size_t)(2 * max_cells + 1 + max_atoms) * sizeof(int);
+    b->smem_bytes = (size_t)std::max(2 * max_cells + 1 + max_atoms, kShiftInts) * sizeof(int);
     if (slots > b->list_slots) {
         cudaFree(b->args.nbr);
         b->args.nbr = nullptr;
@@ -961,19 +989,13 @@ FIRE2_HIDDEN fire_status fire2_batch_create(fire_handle_t* h, int32_t n_sys,
     BA(a.f, n * sizeof(dvec4));
     BA(a.xref, n * sizeof(dvec4));
     BA(a.xf, n * sizeof(float4));
-    if (f32) {
-        BA(a.xq, n * sizeof(int4));
-        BA(a.fp32, n * sizeof(float));
-    } else {
-        BA(a.fp64, n * sizeof(double));
-    }
+    if (f32) BA(a.xq, n * sizeof(int4));
     a.confirm = f32 && fire2_params(h).confirm64 != 0 ? 1 : 0;
     a.vmode = a.confirm ? fire2_params(h).confirm64 : 0;
     a.ff = fire2_tab_ffd(h) != nullptr && (!f32 || a.confirm) ? 1 : 0;
-    if (a.ff && f32) BA(a.fp64, n * sizeof(double));
+    if (!a.ff) BA(a.fp64, n * sizeof(double));
     if (a.ff) {
         BA(a.xq64, n * sizeof(lvec4));
-        BA(a.fpff, n * sizeof(float2));
         a.tab_ffd = fire2_tab_ffd(h);
         a.tab_fff = fire2_tab_fff(h);
     }
