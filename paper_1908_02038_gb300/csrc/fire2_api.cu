@@ -214,8 +214,9 @@ int auto_tpa(const fire_potential_t& p, long long n, int sms) {
 // the FP64 additions and L2 atomics of the neighbour terms (FP64 pipe 62 % ->
 // 3 %, L2 40 % -> 8 % in the force pass) but both passes are bound by the
 // issue of their double-float arithmetic, and the tiles' staging, barriers
-// and fixed-point splits cost more issue than they save (1M-atom box: force
-// 0.49 ms against 0.41, density 0.38 against 0.29).
+// and fixed-point splits cost more issue than they save (1M-atom box, both on
+// the quintic tables: force 0.49 ms against 0.41, density 0.38 against 0.29; the
+// untiled passes take 0.344 and 0.245 since).
 bool tiles_wanted(const fire_handle* h, const GeoC& g) {
     if (!fixed64_half(h->pot) || g.brute || h->neb || g.img_n != h->n) return false;
     return h->tile_mode == FIRE_TILES_ON;
