@@ -2143,9 +2143,10 @@ fire_status fire_diag_rgl_table(const fire_potential_t* pot, int64_t n, const do
         double* o = out + 4 * i;
         // the FP64 kernels' arithmetic from r^2 on (r^2 as a float pair)
         const ffloat r2 = f64_to_ff(r[i] * r[i]);
-        if (!(r2.hi < rc2_f)) {
+        const bool rows = ff_in_rows(T, r2.hi);
+        if (!rows && !(r2.hi < rc2_f)) {
             o[0] = o[1] = o[2] = o[3] = 0.0;
-        } else if (r2.hi >= T.r2_lo) {
+        } else if (rows) {
             ffloat d[2], f[2];
             ff_eval(ffd, T, r2, d);
             ff_eval(fff, T, r2, f);

@@ -338,11 +338,12 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
                 if (k + 1 < m) e_nx = a.nbr[I.list_off + (long long)(k + 1) * I.n + i];
                 const lvec4 qj = a.xq64[I.off + (int)(e & kIdxMask)];
                 const ffloat r2 = ff_norm2(b_sep_ff(S, qi, qj, e));
-                if (!(r2.hi < P.rc2_f)) continue;
+                const bool rows = ff_in_rows(P.ff, r2.hi);
+                if (!rows && !(r2.hi < P.rc2_f)) continue;
                 ffloat2 w;
-                if (r2.hi >= P.ff.r2_lo) {
+                if (rows) {
                     w = ff_eval2(a.tab_ffd, P.ff, r2);
-                } else {   // compressed below the table: FP64 exponentials
+                } else {   // outside the rows: FP64 exponentials
                     double rinv, phi, dphi, g, dg;
                     rgl_pair64(P, ff_to_f64(r2), etab, rinv, phi, dphi, g, dg);
                     const ffloat p = f64_to_ff(phi), q = f64_to_ff(g);
@@ -428,9 +429,10 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
                 const lvec4 qj = a.xq64[I.off + (int)(e & kIdxMask)];
                 const ffvec d = b_sep_ff(S, qi, qj, e);
                 const ffloat r2 = ff_norm2(d);
-                if (!(r2.hi < P.rc2_f)) continue;
+                const bool rows = ff_in_rows(P.ff, r2.hi);
+                if (!rows && !(r2.hi < P.rc2_f)) continue;
                 ffloat c0, c1;
-                if (r2.hi >= P.ff.r2_lo) {
+                if (rows) {
                     const ffloat2 c = ff_eval2(a.tab_fff, P.ff, r2);
                     c0 = ff_first(c);
                     c1 = ff_second(c);

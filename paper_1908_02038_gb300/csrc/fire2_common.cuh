@@ -50,9 +50,10 @@ struct TabMeta {
 };
 
 // Intervals of the FP64 form's pair tables (fire2_table.cuh): width h in r^2,
-// from row 0 = [j_lo h, (j_lo + 1) h); rs2 = rs^2, r2_lo = j_lo h.
+// from row 0 = [j_lo h, (j_lo + 1) h); rs2 = rs^2.  The rows serve r2_lo = j_lo h
+// up to r2_hi: rc^2, or rs^2 where the taper is too narrow for them.
 struct FFTab {
-    float h, hinv, r2_lo, rs2;
+    float h, hinv, r2_lo, r2_hi, rs2;
     int j_lo, last;
 };
 

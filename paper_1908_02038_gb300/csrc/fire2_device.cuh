@@ -1411,9 +1411,10 @@ __device__ __forceinline__ void density_ff_body(const Bufs& b, const PotC& P, co
             const lvec4 qj = b.xq64[j];
             if (k + TPA < m) e_nx = b.nbr[(size_t)(k + TPA) * b.n + i];
             const ffloat r2 = ff_norm2(pair_sep_ff(qt, qi, qj, e));
-            if (!(r2.hi < P.rc2_f)) continue;
+            const bool rows = ff_in_rows(P.ff, r2.hi);
+            if (!rows && !(r2.hi < P.rc2_f)) continue;
             ffloat2 v;   // phi (doubled at the end on the half list), g
-            if (r2.hi >= P.ff.r2_lo) {
+            if (rows) {
                 v = ff_eval2(b.tab_ffd, P.ff, r2);
                 if (HALF) atomicAdd(&b.rho[j], ff_to_f64(ff_second(v)));
             } else {
@@ -1496,9 +1497,10 @@ __global__ void __launch_bounds__(BLK) k_force_ff(Bufs b, PotC P, GeoC g) {
         if (k + 2 * TPA < m) e_n2 = b.nbr[(size_t)(k + 2 * TPA) * b.n + i];
         const ffvec d = pair_sep_ff(qt, qi, qj, e);
         const ffloat r2 = ff_norm2(d);
-        if (!(r2.hi < P.rc2_f)) continue;
+        const bool rows = ff_in_rows(P.ff, r2.hi);
+        if (!rows && !(r2.hi < P.rc2_f)) continue;
         ffloat c0, c1;
-        if (r2.hi >= P.ff.r2_lo) {
+        if (rows) {
             const ffloat2 c = ff_eval2(b.tab_fff, P.ff, r2);
             c0 = ff_first(c);
             c1 = ff_second(c);

@@ -125,9 +125,10 @@ __device__ __forceinline__ double loop_density(const Bufs& b, const PotC& P, con
             if (k + L < m) q_nx = ld_lvec4_l2(b.xq64 + (e_nx & kIdxMask));
             if (k + 2 * L < m) e_n2 = b.nbr[(size_t)(k + 2 * L) * b.n + i];
             const ffloat r2 = ff_norm2(pair_sep_ff(qt, qi, qj, en));
-            if (!(r2.hi < P.rc2_f)) continue;
+            const bool rows = ff_in_rows(P.ff, r2.hi);
+            if (!rows && !(r2.hi < P.rc2_f)) continue;
             ffloat2 v;
-            if (r2.hi >= P.ff.r2_lo) {
+            if (rows) {
                 v = ff_eval2(b.tab_ffd, P.ff, r2);
             } else {
                 double rinv, phi, dphi, gg, dg;
@@ -183,9 +184,10 @@ __device__ __forceinline__ void loop_force(const Bufs& b, const PotC& P, const l
             if (k + 2 * L < m) e_n2 = b.nbr[(size_t)(k + 2 * L) * b.n + i];
             const ffvec d = pair_sep_ff(qt, qi, qj, en);
             const ffloat r2 = ff_norm2(d);
-            if (!(r2.hi < P.rc2_f)) continue;
+            const bool rows = ff_in_rows(P.ff, r2.hi);
+            if (!rows && !(r2.hi < P.rc2_f)) continue;
             ffloat c0, c1;
-            if (r2.hi >= P.ff.r2_lo) {
+            if (rows) {
                 const ffloat2 c = ff_eval2(b.tab_fff, P.ff, r2);
                 c0 = ff_first(c);
                 c1 = ff_second(c);

@@ -238,6 +238,7 @@ namespace fire2 {
 // 288 / 385 us and were 10 times less accurate.
 
 constexpr int kFFRow = 16;
+constexpr double kTaperRows = 8.0;   // intervals below which the taper is analytic
 constexpr int kFixedBits64 = 44;   // fixed-point positions of the FP64 form: 2^44 per A
 
 
@@ -480,7 +481,15 @@ __host__ __device__ __forceinline__ ffloat ff_poly(const float* c, ffloat s) {
     return ff_madd(s, r, {c[0], c[2]});
 }
 
-// Row of r^2 (its FP32 high part, at least t.r2_lo) and the middle of its
+// Whether a pair at r^2 (its FP32 high part) is evaluated from the rows; one
+// inside the cut-off that is not takes the analytic functions.  Tested before the
+// cut-off, so that a pair in the rows meets two comparisons, as with a lower
+// bound alone.
+__host__ __device__ __forceinline__ bool ff_in_rows(const FFTab& t, float r2) {
+    return r2 < t.r2_hi && r2 >= t.r2_lo;
+}
+
+// Row of r^2 (its FP32 high part, in the rows) and the middle of its
 // interval.  r2 >= rs2 implies j >= floor(rs^2 / h), whose multiple of h is an
 // FP32 number that rs^2 cannot round below; the last row is a bound only.
 __host__ __device__ __forceinline__ int ff_row_of(const FFTab& t, float r2, float& mid) {
@@ -657,6 +666,12 @@ inline FFTab build_ff_tables(double A, double xi, double p, double q, double r0,
     t.j_lo = std::max(1, (int)std::floor(0.25 * r0 * r0 / h));
     t.r2_lo = (float)(t.j_lo * h);
     t.rs2 = (float)(rs * rs);
+    // The taper is a quintic in (r - rs) / (rc - rs): economised over n intervals
+    // it is off by about 6 / 512 n^-5 of the function, 4e-7 at 8; over fewer the
+    // rows are soon useless (n = 1/2: off by more than the function), and such a
+    // thin shell holds few pairs.  Pairs that round to rs^2 or just below go with the taper.
+    const bool taper_rows = rc * rc - rs * rs >= kTaperRows * h;
+    t.r2_hi = taper_rows ? (float)(rc * rc) : std::nextafterf(t.rs2, 0.f);
     const int j_rs = (int)std::floor(rs * rs / h), j_rc = (int)std::floor(rc * rc / h);
     const int rows = std::max(j_rc - t.j_lo, 0) + 2;
     t.last = rows - 1;
@@ -704,7 +719,7 @@ inline FFTab build_ff_tables(double A, double xi, double p, double q, double r0,
     };
     const int jb = std::max(t.j_lo, j_rs);
     region(t.j_lo, std::min(j_rs, j_rc), 0, 0);
-    region(jb, j_rc, 3, jb - t.j_lo + 1);
+    if (taper_rows) region(jb, j_rc, 3, jb - t.j_lo + 1);
     return t;
 }
 

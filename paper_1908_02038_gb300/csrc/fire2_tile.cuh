@@ -339,9 +339,10 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_density_tile(B
                 }
                 ffloat dx, dy, dz;
                 const ffloat r2 = tile_sep(qjx - qix, qjy - qiy, qjz - qiz, dx, dy, dz);
-                if (!(r2.hi < P.rc2_f)) continue;
+                const bool rows = ff_in_rows(P.ff, r2.hi);
+                if (!rows && !(r2.hi < P.rc2_f)) continue;
                 ffloat v[2];
-                if (r2.hi >= P.ff.r2_lo) {
+                if (rows) {
                     const ffloat2 w = ff_eval2(b.tab_ffd, P.ff, r2);
                     v[0] = ff_first(w);
                     v[1] = ff_second(w);
@@ -460,9 +461,10 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_force_tile(Buf
                 }
                 ffloat dx, dy, dz;
                 const ffloat r2 = tile_sep(qjx - qix, qjy - qiy, qjz - qiz, dx, dy, dz);
-                if (!(r2.hi < P.rc2_f)) continue;
+                const bool rows = ff_in_rows(P.ff, r2.hi);
+                if (!rows && !(r2.hi < P.rc2_f)) continue;
                 ffloat c[2];
-                if (r2.hi >= P.ff.r2_lo) {
+                if (rows) {
                     const ffloat2 w = ff_eval2(b.tab_fff, P.ff, r2);
                     c[0] = ff_first(w);
                     c[1] = ff_second(w);
