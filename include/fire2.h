@@ -77,7 +77,8 @@ typedef enum {
  * evaluated.  FIRE_PAIR_TABLE: piecewise polynomials in r^2, no square root
  * or exponential per pair; pairs closer than r0/2 use the analytic functions.
  * In the FP64 precision: quartics on intervals of r0^2/326 or less (a power of
- * two; the taper's third-derivative jumps at rs and rc on row boundaries;
+ * two, at least rc^2/65536; the taper's third-derivative jumps at rs and rc on
+ * row boundaries, a taper of fewer than 8 intervals by the analytic functions;
  * interpolation error ~1e-13 relative for values, ~1e-12 for derivatives,
  * largest near r0/2), computed from exact fixed-point separations (2^-44 A)
  * in double-float arithmetic (float pairs, ~2^-44 relative), with FP64 sums,

@@ -14,8 +14,8 @@
 // r0, where the forces are stiffest, keep the full precision of u even in
 // FP32), region B x = (u - u_rs) / hB.
 //
-// FP64 form (build_ff_tables below): intervals of a power of two, about
-// r0^2 / 420, in r^2 itself.
+// FP64 form (build_ff_tables below): intervals of a power of two, r0^2 / 652 to
+// r0^2 / 326 in Angstrom (ff_interval), in r^2 itself.
 //
 // In both u_lo = -0.75 r0^2 (r = r0/2); closer pairs fall back to the
 // analytic functions.  Each interval's quintic matches the function and its
@@ -207,8 +207,8 @@ namespace fire2 {
 //       r^2 = dx^2 + dy^2 + dz^2,  s = r^2 - (middle of its interval),
 //       f = c0 + s (c1 + s (c2 + s q)),   q = c3 + s c4
 //     with c0..c2 and s as float pairs, q in plain FP32 and the product s q
-//     added to c2's low part: an interval spans ~r0^2 / 420, so that
-//     |s c_{j+1} / c_j| is below ~0.01 / (j + 1) on the Cu parameters, s q is
+//     added to c2's low part: an interval spans r0^2 / 418 on the Cu
+//     parameters, so that |s c_{j+1} / c_j| is below ~0.01 / (j + 1), s q is
 //     below 2^-8 of c2 and its rounding 2^-32 of c2, ~2^-48 of f;
 //   * the cut-off test and the interval index use the FP32 high part of r^2:
 //     the taper makes phi, g and their first two derivatives vanish at rc,
@@ -651,6 +651,26 @@ inline void ff_eval(const std::vector<float>& tab, const FFTab& t, ffloat r2, ff
     out[1] = ff_poly(row + 1, s);
 }
 
+// Width of the intervals, a power of two.  The largest at or below r0^2 / 326
+// gives the errors quoted at build_ff_tables below near r0 and 32 times those at
+// r0 / 2, where a steep phi's slope is twice as large.  Where lengths are larger
+// numbers than in Angstrom (r0^2 / 326 >= 2^-5) a quarter of that, and no more
+// than 1/256 of the taper, puts both under the arithmetic's own 2^-44 (r0 = 4.83,
+// the Cu set in bohr, phi' at r0 / 2: 7e-13 -> 1e-14); but no finer than 2^-6, at
+// which the Angstrom sets run.  At most 2^16 rows where that is wider than
+// 2^-6, and 2^22 in any case: row numbers and the middles of the intervals have
+// to be exact in FP32, and the rows of an r0 far below rc, of which few are
+// ever met, would fill the memory.
+inline double ff_interval(double r0, double rs, double rc) {
+    auto below = [](double x) { return std::exp2(std::floor(std::log2(x))); };
+    double h = below(r0 * r0 / 326.0);
+    if (h > 0x1p-6)
+        h = std::max(0x1p-6, std::min(0.25 * h, below((rc - rs) * (rc + rs) / 256.0)));
+    const double rows = rc * rc;   // over 2^k rows: the width 2^-k rc^2
+    const double least = std::max(std::min(0x1p-6, 0x1p-16 * rows), 0x1p-22 * rows);
+    return std::max(h, std::exp2(std::ceil(std::log2(least))));
+}
+
 // Density rows (phi, g) and force rows (2 phi'/r, g'/r).  Each polynomial is
 // the quintic Hermite interpolant of its interval, moved to the interval's
 // middle, with its fifth-degree term replaced by the Chebyshev-economised
@@ -659,11 +679,15 @@ inline void ff_eval(const std::vector<float>& tab, const FFTab& t, ffloat r2, ff
 // the Cu phi near r0.
 inline FFTab build_ff_tables(double A, double xi, double p, double q, double r0, double rs,
                              double rc, std::vector<float>& dens, std::vector<float>& force) {
-    const double h = std::exp2(std::floor(std::log2(r0 * r0 / 326.0)));
+    const double h = ff_interval(r0, rs, rc);
     FFTab t;
     t.h = (float)h;
     t.hinv = (float)(1.0 / h);
-    t.j_lo = std::max(1, (int)std::floor(0.25 * r0 * r0 / h));
+    const int j_rs = (int)std::floor(rs * rs / h), j_rc = (int)std::floor(rc * rc / h);
+    // from r0 / 2 (beyond rc where that is); never below 81 h, which it is where
+    // h is not limited by the number of rows: closer to 0 the functions, smooth in
+    // r, are no polynomials in r^2
+    t.j_lo = std::max(81, (int)std::min(std::floor(0.25 * r0 * r0 / h), j_rc + 1.0));
     t.r2_lo = (float)(t.j_lo * h);
     t.rs2 = (float)(rs * rs);
     // The taper is a quintic in (r - rs) / (rc - rs): economised over n intervals
@@ -672,7 +696,6 @@ inline FFTab build_ff_tables(double A, double xi, double p, double q, double r0,
     // thin shell holds few pairs.  Pairs that round to rs^2 or just below go with the taper.
     const bool taper_rows = rc * rc - rs * rs >= kTaperRows * h;
     t.r2_hi = taper_rows ? (float)(rc * rc) : std::nextafterf(t.rs2, 0.f);
-    const int j_rs = (int)std::floor(rs * rs / h), j_rc = (int)std::floor(rc * rc / h);
     const int rows = std::max(j_rc - t.j_lo, 0) + 2;
     t.last = rows - 1;
     dens.assign((size_t)rows * kFFRow, 0.f);
