@@ -422,6 +422,12 @@ fire_status fire_energy_forces_noalloc(const fire_potential_t* pot, int64_t n_at
                                        const double box[3], double* d_forces, double* d_energy,
                                        void* stream);
 
+/* Diagnostic: *used receives 1 if the last relaxation or energy-force evaluation
+ * on h ran in the resident kernel (fire_set_exec_mode), 0 if it ran in the chain
+ * of kernels (also where the device cannot run the resident one), -1 before the
+ * first.  The paper has no counterpart.  Errors: FIRE_ERR_ARG (NULL). */
+fire_status fire_diag_resident_loop(const fire_handle_t* h, int32_t* used);
+
 /* Diagnostic: evaluates the library's FP64 exponential (the table-driven
  * method of P. T. P. Tang, ACM TOMS 15(2), 1989, used by the RGL pair terms)
  * at n points: d_x and d_out are device arrays of n doubles; valid for

@@ -114,6 +114,7 @@ struct fire_handle {
     bool tpa_set = false;            // threads per atom chosen by the caller
     bool loop = false;               // make_geo: lists for the resident loop (full)
     int loop_ok = -1;                // its graph can be made on this device (-1: not tried)
+    int ran_loop = -1;               // the last relaxation or evaluation ran there (-1: none yet)
     double* loop_rows = nullptr;     // the resident loop's partials
     int tile_mode = FIRE_TILES_AUTO; // shared-memory tiles of the FP64 half-list passes
     int stage_cap = 0;               // staged atoms per tile (0 = kStageMax)
@@ -693,8 +694,7 @@ cudaError_t launch_loop(fire_handle* h, const GeoC& g, cudaStream_t s, bool eval
     const LoopShape q = loop_shape(h);
     const LoopKernel kern = loop_kernel(h, q);
     const size_t smem = loop_smem(q.share);
-    cudaError_t e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = raise_smem((const void*)kern, smem);
     if (e == cudaSuccess && !h->loop_rows)
         e = cudaMalloc(&h->loop_rows, (size_t)kLoopRows * h->sms * sizeof(double));
     if (e != cudaSuccess) return e;
@@ -1223,8 +1223,8 @@ static fire_status upload_tables(fire_handle* h) {
     const int block = kTabBlock;
     const void* kd = (const void*)k_density32_tab;
     const void* kf = (const void*)k_force32_tab;
-    CK(h, cudaFuncSetAttribute(kd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem_d));
-    CK(h, cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem_f));
+    CK(h, raise_smem(kd, h->smem_d));
+    CK(h, raise_smem(kf, h->smem_f));
     int sms = 0, occ_d = 0, occ_f = 0;
     CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     CK(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_d, kd, block, h->smem_d));
@@ -1536,6 +1536,7 @@ static fire_status prepare_eval(fire_handle* h, const double box[3], GeoC* g) {
     int coop = 0, occ = 0;
     const LoopShape q = loop_shape(h);
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device) == cudaSuccess && coop &&
+        raise_smem((const void*)loop_kernel(h, q), loop_smem(q.share)) == cudaSuccess &&
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)loop_kernel(h, q), q.threads,
                                                       loop_smem(q.share)) == cudaSuccess && occ >= 1)
         return FIRE_OK;
@@ -1547,6 +1548,7 @@ static fire_status prepare_eval(fire_handle* h, const double box[3], GeoC* g) {
 // One relaxation on the device: positions are already in b.pos_io.
 static fire_status run_minimize(fire_handle* h, const GeoC& g, double ftol, int64_t maxiter,
                                 cudaStream_t s) {
+    h->ran_loop = h->loop ? 1 : 0;
     const bool chunked = h->exec_mode == FIRE_EXEC_CHUNKED;
     const bool have = chunked ? h->exec_chunk != nullptr : h->exec != nullptr;
     if (!h->has_graph || !have || !same_geo(h->gkey, g)) {
@@ -1617,6 +1619,12 @@ fire_status fire_set_exec_mode(fire_handle_t* h, int32_t mode, int32_t chunk) {
     h->exec_mode = mode;
     if (mode == FIRE_EXEC_CHUNKED) h->chunk = chunk;
     else h->body_iters = chunk;
+    return FIRE_OK;
+}
+
+fire_status fire_diag_resident_loop(const fire_handle_t* h, int32_t* used) {
+    if (!h || !used) return FIRE_ERR_ARG;
+    *used = h->ran_loop;
     return FIRE_OK;
 }
 
@@ -1696,6 +1704,7 @@ static fire_status run_eval(fire_handle* h, const GeoC& g, cudaStream_t s) {
 }
 
 static fire_status run_eval_unmasked(fire_handle* h, const GeoC& g, cudaStream_t s) {
+    h->ran_loop = h->loop ? 1 : 0;
     init_state(h, 0.0, 0);
     CK(h, cudaMemcpyAsync(h->b.st, h->h_state, sizeof(DevState), cudaMemcpyHostToDevice, s));
     k_prepare<<<ceil_div(h->n, kElemBlock), kElemBlock, 0, s>>>(h->b);

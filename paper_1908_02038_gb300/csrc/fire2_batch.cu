@@ -1033,9 +1033,7 @@ static int maxt_of(const fire_batch_tuning_t& t) {
 
 template <bool F32, int MAXT>
 static fire_status launch_plain(fire_batch_state* b, int grid, int threads, cudaStream_t s) {
-    if (cudaFuncSetAttribute(k_batch_relax<F32, false, MAXT>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)b->smem_bytes) != cudaSuccess)
+    if (raise_smem((const void*)k_batch_relax<F32, false, MAXT>, b->smem_bytes) != cudaSuccess)
         return FIRE_ERR_CUDA;
     k_batch_relax<F32, false, MAXT><<<grid, threads, b->smem_bytes, s>>>(b->args);
     return cudaGetLastError() == cudaSuccess ? FIRE_OK : FIRE_ERR_CUDA;
@@ -1061,8 +1059,7 @@ static fire_status launch_shape(fire_handle_t* h, fire_batch_state* b, cudaStrea
         return FIRE_OK;
     }
     const int clusters = std::max(1, std::min(b->n_sys, b->sms * b->tune.ctas_per_sm / C));
-    BCK(cudaFuncSetAttribute(k_batch_relax<F32, true, 512>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem_bytes));
+    BCK(raise_smem((const void*)k_batch_relax<F32, true, 512>, b->smem_bytes));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * C), 1, 1);
     cfg.blockDim = dim3((unsigned)threads, 1, 1);
@@ -1084,9 +1081,7 @@ template <bool F32>
 static bool cluster_fits(const fire_batch_state* b, const fire_batch_tuning_t& t) {
     const int C = cluster_of(t);
     if (C == 1) return true;
-    if (cudaFuncSetAttribute(k_batch_relax<F32, true, 512>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)b->smem_bytes) != cudaSuccess) {
+    if (raise_smem((const void*)k_batch_relax<F32, true, 512>, b->smem_bytes) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }

@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "fire2_math.cuh"
 
 namespace fire2 {
@@ -56,6 +58,18 @@ struct FFTab {
     float h, hinv, r2_lo, r2_hi, rs2;
     int j_lo, last;
 };
+
+// Dynamic shared memory of a kernel: its limit belongs to the process, not to a
+// handle, so it is only ever raised, by whoever needs more than it stands at
+// (launches of other handles and threads rely on what they raised it to).
+inline cudaError_t raise_smem(const void* kernel, size_t bytes) {
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess || bytes <= (size_t)a.maxDynamicSharedSizeBytes) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
 
 // Potential constants, passed by value.
 struct PotC {
