@@ -114,6 +114,7 @@ struct fire_handle {
     bool tpa_set = false;            // threads per atom chosen by the caller
     bool loop = false;               // make_geo: lists for the resident loop (full)
     int loop_ok = -1;                // its graph can be made on this device (-1: not tried)
+    bool loop_fits = false;          // the device can hold a block of it per SM
     int ran_loop = -1;               // the last relaxation or evaluation ran there (-1: none yet)
     double* loop_rows = nullptr;     // the resident loop's partials
     int tile_mode = FIRE_TILES_AUTO; // shared-memory tiles of the FP64 half-list passes
@@ -693,9 +694,9 @@ cudaError_t launch_loop(fire_handle* h, const GeoC& g, cudaStream_t s, bool eval
                         cudaGraphConditionalHandle hw) {
     const LoopShape q = loop_shape(h);
     const LoopKernel kern = loop_kernel(h, q);
-    const size_t smem = loop_smem(q.share);
-    cudaError_t e = raise_smem((const void*)kern, smem);
-    if (e == cudaSuccess && !h->loop_rows)
+    const size_t smem = loop_smem(q.share);   // prepare_eval has raised the kernel's limit
+    cudaError_t e = cudaSuccess;
+    if (!h->loop_rows)
         e = cudaMalloc(&h->loop_rows, (size_t)kLoopRows * h->sms * sizeof(double));
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -714,7 +715,7 @@ cudaError_t launch_loop(fire_handle* h, const GeoC& g, cudaStream_t s, bool eval
 
 // The resident loop as a graph: prepare; WHILE (not stopped): list build,
 // k_loop (which sets the condition); finalize.
-fire_status build_loop_graph(fire_handle* h, const GeoC& g) {
+fire_status build_loop_graph(fire_handle* h, const GeoC& g, cudaError_t* why = nullptr) {
     drop_graph(h);
     if (!h->loop_rows) CK(h, cudaMalloc(&h->loop_rows, (size_t)kLoopRows * h->sms * sizeof(double)));
     cudaGraph_t graph = nullptr;
@@ -750,7 +751,9 @@ fire_status build_loop_graph(fire_handle* h, const GeoC& g) {
         cudaGraphDestroy(graph);
         h->exec = nullptr;
         cudaGetLastError();
-        return fail(h, FIRE_ERR_CUDA, "resident loop's graph: %s", cudaGetErrorString(e));
+        if (why) *why = e;
+        return fail(h, e == cudaErrorMemoryAllocation ? FIRE_ERR_NOMEM : FIRE_ERR_CUDA,
+                    "resident loop's graph: %s", cudaGetErrorString(e));
     }
     h->graph = graph;
     h->gkey = g;
@@ -1518,31 +1521,47 @@ fire_status fire_set_dof_mask(fire_handle_t* h, const uint8_t* mask) {
     return FIRE_OK;
 }
 
-// prepare_call for a relaxation: where the resident loop's graph cannot be made
-// (no cooperative launches inside conditional nodes, as under MPS) the kernel
-// chain from then on.
-static fire_status prepare_relax(fire_handle* h, const double box[3], GeoC* g) {
-    fire_status st = prepare_call(h, box, g, false, true);
-    if (st != FIRE_OK || !h->loop || h->loop_ok == 1) return st;
-    h->loop_ok = build_loop_graph(h, *g) == FIRE_OK ? 1 : 0;
-    return h->loop_ok ? FIRE_OK : prepare_call(h, box, g, false, true);
+// prepare_call for an evaluation or a relaxation.  Where the device cannot run
+// the resident loop (no cooperative launches, or none of this size: MPS with a
+// share of the SMs) the handle takes the kernel chain from then on; any other
+// error is the call's.
+static bool loop_unsupported(cudaError_t e) {
+    return e == cudaErrorNotSupported || e == cudaErrorCooperativeLaunchTooLarge ||
+           e == cudaErrorStreamCaptureUnsupported;
+}
+static fire_status prepare_chain(fire_handle* h, const double box[3], GeoC* g) {
+    h->loop_ok = 0;
+    h->err.clear();
+    return prepare_call(h, box, g, false, true);
 }
 
-// The same before an evaluation, which launches the kernel itself: whether a
-// cooperative launch of it fits (loop_ok stays untried for the graph).
 static fire_status prepare_eval(fire_handle* h, const double box[3], GeoC* g) {
     fire_status st = prepare_call(h, box, g, false, true);
     if (st != FIRE_OK || !h->loop) return st;
-    int coop = 0, occ = 0;
+    if (h->loop_fits) return FIRE_OK;
+    int coop = 0, occ = 0, room = 0;
     const LoopShape q = loop_shape(h);
-    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device) == cudaSuccess && coop &&
-        raise_smem((const void*)loop_kernel(h, q), loop_smem(q.share)) == cudaSuccess &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)loop_kernel(h, q), q.threads,
-                                                      loop_smem(q.share)) == cudaSuccess && occ >= 1)
-        return FIRE_OK;
-    cudaGetLastError();
-    h->loop_ok = 0;
-    return prepare_call(h, box, g, false, true);
+    const void* kern = (const void*)loop_kernel(h, q);
+    cudaFuncAttributes a;
+    CK(h, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
+    CK(h, cudaDeviceGetAttribute(&room, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
+    CK(h, cudaFuncGetAttributes(&a, kern));
+    if (!coop || a.sharedSizeBytes + loop_smem(q.share) > (size_t)room) return prepare_chain(h, box, g);
+    CK(h, raise_smem(kern, loop_smem(q.share)));
+    CK(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, q.threads, loop_smem(q.share)));
+    if (occ < 1) return prepare_chain(h, box, g);
+    h->loop_fits = true;
+    return FIRE_OK;
+}
+
+// A relaxation's launch is a node of a graph, which is made here the first time.
+static fire_status prepare_relax(fire_handle* h, const double box[3], GeoC* g) {
+    fire_status st = prepare_eval(h, box, g);
+    if (st != FIRE_OK || !h->loop || h->loop_ok == 1) return st;
+    cudaError_t why = cudaSuccess;
+    st = build_loop_graph(h, *g, &why);
+    if (st == FIRE_OK) h->loop_ok = 1;
+    return loop_unsupported(why) ? prepare_chain(h, box, g) : st;
 }
 
 // One relaxation on the device: positions are already in b.pos_io.
