@@ -428,6 +428,12 @@ fire_status fire_energy_forces_noalloc(const fire_potential_t* pot, int64_t n_at
  * first.  The paper has no counterpart.  Errors: FIRE_ERR_ARG (NULL). */
 fire_status fire_diag_resident_loop(const fire_handle_t* h, int32_t* used);
 
+/* Diagnostic: the longest wait of the resident kernel's blocks for one another
+ * (5 s by default, at most 60) on later calls of h, after which the call returns
+ * FIRE_ERR_TIMEOUT; 0 lets every wait run out.  The paper has no counterpart.
+ * Errors: FIRE_ERR_ARG. */
+fire_status fire_diag_set_loop_wait(fire_handle_t* h, double seconds);
+
 /* Diagnostic: evaluates the library's FP64 exponential (the table-driven
  * method of P. T. P. Tang, ACM TOMS 15(2), 1989, used by the RGL pair terms)
  * at n points: d_x and d_out are device arrays of n doubles; valid for

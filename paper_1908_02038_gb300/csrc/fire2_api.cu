@@ -117,6 +117,7 @@ struct fire_handle {
     bool loop_fits = false;          // the device can hold a block of it per SM
     int ran_loop = -1;               // the last relaxation or evaluation ran there (-1: none yet)
     double* loop_rows = nullptr;     // the resident loop's partials
+    unsigned long long loop_wait_ns = kLoopWaitNs;
     int tile_mode = FIRE_TILES_AUTO; // shared-memory tiles of the FP64 half-list passes
     int stage_cap = 0;               // staged atoms per tile (0 = kStageMax)
     size_t loc_slots = 0;            // allocated nbr_loc entries
@@ -709,8 +710,7 @@ cudaError_t launch_loop(fire_handle* h, const GeoC& g, cudaStream_t s, bool eval
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, h->b, h->potc, g, LoopC{h->loop_rows, q.share, eval ? 1 : 0},
-                              hw);
+    return cudaLaunchKernelEx(&cfg, kern, h->b, h->potc, g, LoopC{h->loop_rows, q.share, eval ? 1 : 0, h->loop_wait_ns}, hw);
 }
 
 // The resident loop as a graph: prepare; WHILE (not stopped): list build,
@@ -1013,6 +1013,13 @@ fire_status status_to_error(fire_handle* h, int st) {
                         "more than %d atoms within the Stillinger-Weber cut-off of one atom", kSwMax);
         default: return fail(h, FIRE_ERR_CUDA, "unknown device status %d", st);
     }
+}
+
+// How the device work of a call ended, from its state copied to the host.
+fire_status end_status(fire_handle* h) {
+    if (h->h_state->bar_abort)
+        return fail(h, FIRE_ERR_TIMEOUT, "a wait between the blocks of the resident kernel ran out");
+    return status_to_error(h, h->h_state->status);
 }
 
 void fill_result(const fire_handle* h, fire_result_t* out) {
@@ -1591,7 +1598,7 @@ static fire_status run_minimize(fire_handle* h, const GeoC& g, double ftol, int6
     }
     CK(h, cudaMemcpyAsync(h->h_state, h->b.st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
     CK(h, cudaStreamSynchronize(s));
-    return status_to_error(h, h->h_state->status);
+    return end_status(h);
 }
 
 fire_status fire_set_threads_per_atom(fire_handle_t* h, int32_t tpa, int32_t* chosen) {
@@ -1638,6 +1645,14 @@ fire_status fire_set_exec_mode(fire_handle_t* h, int32_t mode, int32_t chunk) {
     h->exec_mode = mode;
     if (mode == FIRE_EXEC_CHUNKED) h->chunk = chunk;
     else h->body_iters = chunk;
+    return FIRE_OK;
+}
+
+fire_status fire_diag_set_loop_wait(fire_handle_t* h, double seconds) {
+    if (!h) return FIRE_ERR_ARG;
+    if (!(seconds >= 0.0 && seconds <= 60.0)) return fail(h, FIRE_ERR_ARG, "need 0 <= seconds <= 60");
+    drop_graph(h);   // holds the limit by value
+    h->loop_wait_ns = (unsigned long long)(seconds * 1e9);
     return FIRE_OK;
 }
 
@@ -1738,7 +1753,7 @@ static fire_status run_eval_unmasked(fire_handle* h, const GeoC& g, cudaStream_t
     CK(h, cudaGetLastError());
     CK(h, cudaMemcpyAsync(h->h_state, h->b.st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
     CK(h, cudaStreamSynchronize(s));
-    return status_to_error(h, h->h_state->status);
+    return end_status(h);
 }
 
 fire_status fire_energy_forces_dev(fire_handle_t* h, const double* d_pos, const double box[3],

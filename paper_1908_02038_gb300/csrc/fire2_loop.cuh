@@ -19,9 +19,11 @@
 // velocity.  L lanes share an atom (group sums in FP64).
 //
 // A barrier is one atomic and a poll per block.  The launch is cooperative, so
-// every block is resident; each wait ends after kLoopWaitNs all the same, with
-// an abort flag that every other wait sees, and the call returns
-// FIRE_ERR_TIMEOUT.
+// every block is resident; each wait ends after LoopC::wait_ns all the same, with
+// an abort flag that every other wait and every later launch of the call sees.
+// A block that finds its count complete goes on, whatever others have done by
+// then, so it is the host that looks at the flag after the last launch: the call
+// returns FIRE_ERR_TIMEOUT.
 //
 // One evaluation (LoopC::eval) is the same passes and sums, then the export: 497
 // atoms 130 -> 102 us a call, list build and copies included.
@@ -45,6 +47,7 @@ struct LoopC {
     double* rows;          // kLoopRows x gridDim.x partials
     int share;             // atoms per block (the last block may have fewer)
     int eval;              // 1: one evaluation (F to b.f and b.f_out, E to b.e_out)
+    unsigned long long wait_ns;   // limit of a wait; 0: every wait runs out (tests)
 };
 
 // Shared-memory bytes of a block that owns `share` atoms.
@@ -63,7 +66,7 @@ struct LoopShared {
 // that came with them; votes receives whether there was any.  False once any
 // wait of the grid has run out.
 __device__ __forceinline__ bool loop_barrier(DevState* st, unsigned& target, LoopShared& sh,
-                                             bool vote, bool& votes) {
+                                             unsigned long long wait_ns, bool vote, bool& votes) {
     target += gridDim.x;
     const int mine = __syncthreads_or(vote);
     if (threadIdx.x == 0) {
@@ -73,11 +76,11 @@ __device__ __forceinline__ bool loop_barrier(DevState* st, unsigned& target, Loo
         int ok = 1;
         for (int n = 0;; ++n) {
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&st->bar) : "memory");
-            if ((int)((unsigned)v - target) >= 0) break;
+            if ((int)((unsigned)v - target) >= 0 && wait_ns != 0ull) break;
             if ((n & 255) != 255) continue;
             const unsigned long long t = globaltimer_ns();
             if (t0 == 0ull) t0 = t;
-            if (*(volatile unsigned*)&st->bar_abort != 0u || t - t0 > kLoopWaitNs) {
+            if (*(volatile unsigned*)&st->bar_abort != 0u || t - t0 >= wait_ns) {
                 atomicExch(&st->bar_abort, 1u);
                 ok = 0;
                 break;
@@ -380,6 +383,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_loop(Bufs b, PotC P, GeoC g, LoopC 
         sh.fs = st->fs;
         sh.stop = 0;
         sh.status = st->status;
+        sh.ok = *(volatile unsigned*)&st->bar_abort == 0u;
     }
     if (RGL)
         fill_qshift64_table(qt, g);
@@ -403,12 +407,12 @@ __global__ void __launch_bounds__(MAXT, 1) k_loop(Bufs b, PotC P, GeoC g, LoopC 
     __syncthreads();
     const int status0 = sh.status;   // of the list build, the same for every block
     unsigned target = 0u;
-    bool ok = true, rebuild = false, votes;
-    for (;;) {
+    bool ok = sh.ok != 0, rebuild = false, votes;
+    while (ok) {
         RedAcc acc;
         if (RGL) {
             acc.E = loop_density<L>(b, P, qt, i0, own);
-            if (!(ok = loop_barrier(st, target, sh, false, votes))) break;
+            if (!(ok = loop_barrier(st, target, sh, c.wait_ns, false, votes))) break;
             loop_force<L>(b, P, qt, i0, own, share, f);
         } else {
             acc.E = loop_force_lj<L>(b, P, tbl, i0, own, share, x, f);
@@ -438,7 +442,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_loop(Bufs b, PotC P, GeoC g, LoopC 
         if (blockIdx.x == 0 && budget && globaltimer_ns() - t_start > budget && status == ST_OK)
             status = ST_TIMEOUT;
         loop_partials(acc, status, c, sh);
-        if (!(ok = loop_barrier(st, target, sh, false, votes))) break;
+        if (!(ok = loop_barrier(st, target, sh, c.wait_ns, false, votes))) break;
         loop_sums(c, sh);
         if (c.eval) {
             loop_export(b, i0, own, share, f, sh);
@@ -452,12 +456,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_loop(Bufs b, PotC P, GeoC g, LoopC 
                              : loop_update<RGL, false>(b, sh.fs, i0, own, share, x, v, f, xr);
         // an atom further than skin / 2 from where the lists were built: every
         // block leaves for a new list
-        if (!(ok = loop_barrier(st, target, sh, d2 > skin2, votes))) break;
+        if (!(ok = loop_barrier(st, target, sh, c.wait_ns, d2 > skin2, votes))) break;
         if (votes) {
             rebuild = true;
             break;
         }
     }
+    if (c.eval) return;   // a wait has run out
     // positions and velocities back (the list build reads x; the next launch
     // both), the state by block 0
     for (int a = threadIdx.x; a < own; a += blockDim.x) {
@@ -465,15 +470,16 @@ __global__ void __launch_bounds__(MAXT, 1) k_loop(Bufs b, PotC P, GeoC g, LoopC 
         b.v[i0 + a] = make_dvec4(v[a], v[share + a], v[2 * share + a], 0.0);
     }
     if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    st->fs = sh.fs;
-    st->P = sh.sum[0];
-    st->F2 = sh.sum[1];
-    st->V2 = sh.sum[2];
-    st->energy = sh.sum[3];
-    st->fmax2 = sh.sum[4];
-    st->finf = sh.sum[5];
-    if (!ok) sh.status = ST_TIMEOUT;
-    if (sh.status != ST_OK) st->status = sh.status;
+    if (ok) {
+        st->fs = sh.fs;
+        st->P = sh.sum[0];
+        st->F2 = sh.sum[1];
+        st->V2 = sh.sum[2];
+        st->energy = sh.sum[3];
+        st->fmax2 = sh.sum[4];
+        st->finf = sh.sum[5];
+        if (sh.status != ST_OK) st->status = sh.status;
+    }
     st->done = rebuild ? 0 : 1;
     cudaGraphSetConditional(hw, rebuild ? 1u : 0u);
 }
