@@ -434,6 +434,12 @@ fire_status fire_diag_resident_loop(const fire_handle_t* h, int32_t* used);
  * Errors: FIRE_ERR_ARG. */
 fire_status fire_diag_set_loop_wait(fire_handle_t* h, double seconds);
 
+/* Diagnostic: arrivals at the resident kernel's barriers (one per block, three
+ * barriers per iteration; two for LJ) after which a relaxation on h builds new
+ * lists whether or not they are due; 2^31 by default, so that the count does not
+ * overflow.  The paper has no counterpart.  Errors: FIRE_ERR_ARG. */
+fire_status fire_diag_set_loop_span(fire_handle_t* h, int64_t arrivals);
+
 /* Diagnostic: evaluates the library's FP64 exponential (the table-driven
  * method of P. T. P. Tang, ACM TOMS 15(2), 1989, used by the RGL pair terms)
  * at n points: d_x and d_out are device arrays of n doubles; valid for

@@ -44,6 +44,7 @@ EXPORTED = ("fire_abi_version", "fire_default_params", "fire_init", "fire_minimi
             "fire_set_time_budget", "fire_profile_stages", "fire_diag_fma_peak",
             "fire_energy_forces_noalloc", "fire_set_exec_mode", "fire_set_threads_per_atom",
             "fire_diag_exp", "fire_diag_resident_loop", "fire_diag_set_loop_wait",
+            "fire_diag_set_loop_span",
             "fire_batch_init", "fire_minimize_batch", "fire_minimize_batch_dev",
             "fire_batch_set_tuning", "fire_batch_autotune", "fire_set_rgl_params",
             "fire_rgl_energy_grad_dev", "fire_rgl_hvp_dev", "fire_rgl_implicit_grad_dev",
@@ -136,6 +137,7 @@ def load_library(path: str | None = None):
                                           C.POINTER(C.c_int32), C.c_void_p]
     lib.fire_diag_exp.argtypes = [C.c_int64, C.c_void_p, C.c_void_p, C.c_void_p]
     lib.fire_diag_set_loop_wait.argtypes = [H, C.c_double]
+    lib.fire_diag_set_loop_span.argtypes = [H, C.c_int64]
     lib.fire_diag_resident_loop.argtypes = [H, C.POINTER(C.c_int32)]
     lib.fire_batch_init.argtypes = [C.POINTER(H), C.c_int32, C.c_void_p, C.POINTER(fire_system_t),
                                     C.POINTER(fire_potential_t), C.POINTER(fire_params_t)]
@@ -314,6 +316,11 @@ def fire_diag_resident_loop(handle) -> int:
 def fire_diag_set_loop_wait(handle, seconds: float) -> None:
     """Longest wait between blocks of the resident kernel (diagnostic)."""
     _check(load_library().fire_diag_set_loop_wait(handle, float(seconds)), handle)
+
+
+def fire_diag_set_loop_span(handle, arrivals: int) -> None:
+    """Barrier arrivals after which the resident kernel leaves for new lists (diagnostic)."""
+    _check(load_library().fire_diag_set_loop_span(handle, int(arrivals)), handle)
 
 
 def fire_diag_fma_peak(which: int) -> float:

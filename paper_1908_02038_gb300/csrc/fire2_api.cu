@@ -118,6 +118,7 @@ struct fire_handle {
     int ran_loop = -1;               // the last relaxation or evaluation ran there (-1: none yet)
     double* loop_rows = nullptr;     // the resident loop's partials
     unsigned long long loop_wait_ns = kLoopWaitNs;
+    unsigned loop_span = kLoopSpan;
     int tile_mode = FIRE_TILES_AUTO; // shared-memory tiles of the FP64 half-list passes
     int stage_cap = 0;               // staged atoms per tile (0 = kStageMax)
     size_t loc_slots = 0;            // allocated nbr_loc entries
@@ -710,7 +711,8 @@ cudaError_t launch_loop(fire_handle* h, const GeoC& g, cudaStream_t s, bool eval
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, h->b, h->potc, g, LoopC{h->loop_rows, q.share, eval ? 1 : 0, h->loop_wait_ns}, hw);
+    return cudaLaunchKernelEx(&cfg, kern, h->b, h->potc, g, LoopC{h->loop_rows, q.share, eval ? 1 : 0, h->loop_wait_ns, h->loop_span},
+                              hw);
 }
 
 // The resident loop as a graph: prepare; WHILE (not stopped): list build,
@@ -1653,6 +1655,15 @@ fire_status fire_diag_set_loop_wait(fire_handle_t* h, double seconds) {
     if (!(seconds >= 0.0 && seconds <= 60.0)) return fail(h, FIRE_ERR_ARG, "need 0 <= seconds <= 60");
     drop_graph(h);   // holds the limit by value
     h->loop_wait_ns = (unsigned long long)(seconds * 1e9);
+    return FIRE_OK;
+}
+
+fire_status fire_diag_set_loop_span(fire_handle_t* h, int64_t arrivals) {
+    if (!h) return FIRE_ERR_ARG;
+    if (arrivals < 1 || arrivals > (int64_t)kLoopSpan)
+        return fail(h, FIRE_ERR_ARG, "arrivals must be in [1, %u]", kLoopSpan);
+    drop_graph(h);   // holds the limit by value
+    h->loop_span = (unsigned)arrivals;
     return FIRE_OK;
 }
 

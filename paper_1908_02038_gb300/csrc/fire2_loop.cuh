@@ -42,12 +42,14 @@ namespace fire2 {
 constexpr int kLoopThreads = 1024;
 constexpr int kLoopRows = 7;   // P, |F|^2, |v|^2, E, max |F_i|^2, max |F_i,d|, status
 constexpr unsigned long long kLoopWaitNs = 5000000000ull;
+constexpr unsigned kLoopSpan = 1u << 31;   // half of what the low half holds
 
 struct LoopC {
     double* rows;          // kLoopRows x gridDim.x partials
     int share;             // atoms per block (the last block may have fewer)
     int eval;              // 1: one evaluation (F to b.f and b.f_out, E to b.e_out)
     unsigned long long wait_ns;   // limit of a wait; 0: every wait runs out (tests)
+    unsigned span;         // arrivals after which the blocks leave for a list, due or not
 };
 
 // Shared-memory bytes of a block that owns `share` atoms.
@@ -62,9 +64,11 @@ struct LoopShared {
 };
 
 // All blocks' writes before the barrier are visible after it (to loads that
-// bypass L1).  The counter's low half counts arrivals, its high half the votes
-// that came with them; votes receives whether there was any.  False once any
-// wait of the grid has run out.
+// bypass L1).  The counter's low half counts arrivals since the last list build,
+// its high half the votes that came with them; votes receives whether there was
+// any.  The arrivals must not carry into the votes, which some blocks would see
+// and others not: the blocks leave for a list (which resets the counter) beyond
+// LoopC::span.  False once any wait of the grid has run out.
 __device__ __forceinline__ bool loop_barrier(DevState* st, unsigned& target, LoopShared& sh,
                                              unsigned long long wait_ns, bool vote, bool& votes) {
     target += gridDim.x;
@@ -454,9 +458,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_loop(Bufs b, PotC P, GeoC g, LoopC 
         const float d2 = sh.fs.kick_after != 0.0
                              ? loop_update<RGL, true>(b, sh.fs, i0, own, share, x, v, f, xr)
                              : loop_update<RGL, false>(b, sh.fs, i0, own, share, x, v, f, xr);
-        // an atom further than skin / 2 from where the lists were built: every
-        // block leaves for a new list
-        if (!(ok = loop_barrier(st, target, sh, c.wait_ns, d2 > skin2, votes))) break;
+        // an atom further than skin / 2 from where the lists were built, or the
+        // barrier's count used up (the same in every block): all leave for a new list
+        if (!(ok = loop_barrier(st, target, sh, c.wait_ns, d2 > skin2 || target > c.span, votes))) break;
         if (votes) {
             rebuild = true;
             break;
