@@ -96,7 +96,7 @@ typedef enum {
  * by FP64 atomics.  FIRE_NEWTON_OFF: full list, every pair from both ends,
  * no atomics (results reproducible bit for bit).  FIRE_NEWTON_AUTO: the
  * faster of the two at the handle's size: full lists in the resident loop
- * (up to 65,536 atoms; fire_set_exec_mode), half lists otherwise. */
+ * (fire_set_exec_mode), half lists otherwise. */
 typedef enum {
     FIRE_NEWTON_AUTO = 0,
     FIRE_NEWTON_ON = 1,
@@ -284,8 +284,9 @@ typedef enum {
  * build, used for boxes under three cells per axis, is launched in every
  * iteration and returns at once unless due; iterations past the stop return
  * at once too); 0 (the default) takes 8, and relaxes small single systems in
- * one resident kernel per neighbour list instead: LJ up to 16,384 atoms, the
- * FP64 table form with FIRE_NEWTON_AUTO up to 65,536, without a maximum
+ * one resident kernel per neighbour list instead: the FP64 table form with
+ * FIRE_NEWTON_AUTO up to 65,536 atoms and 10 million expected list entries, LJ up
+ * to 16,384 atoms, 3.5 million entries and 400 per atom, without a maximum
  * displacement, pair tiles or a set number of threads per atom (energies and
  * forces alone run there too).  Results do not depend on the mode, but for the
  * rounding of sums.

@@ -226,34 +226,54 @@ bool tiles_wanted(const fire_handle* h, const GeoC& g) {
     return h->tile_mode == FIRE_TILES_ON;
 }
 
-// Whether relaxations run in the resident loop (fire2_loop.cuh): the default
-// settings of the FP64 table form and LJ, one system, up to kLoopAtoms atoms.
-// What the caller has chosen (newton, threads per atom, tiles, chunked or
-// sized graph bodies, a displacement cap) keeps the kernel chain.  RGL, us per
-// iteration chain / loop: 48,667 atoms 84.5 / 70.5, 62,499 atoms 98 / 77; above,
-// the full list's second evaluation of every pair eats the gain, and for LJ,
-// whose pair terms are FP64 arithmetic, earlier (10,975 atoms 80 / 53).
-constexpr int kLoopAtoms = 65536, kLoopAtomsLj = 16384;
-bool loop_wanted(const fire_handle* h) {
-    const bool form = h->pot.kind == FIRE_POT_LJ ||
-                      (fixed64_form(h->pot) && h->pot.newton == FIRE_NEWTON_AUTO);
-    return form && h->loop_ok != 0 && !h->neb && !h->batch && h->img_n == h->n &&
-           h->n <= (h->pot.kind == FIRE_POT_LJ ? kLoopAtomsLj : kLoopAtoms) && !h->tpa_set &&
-           h->tile_mode != FIRE_TILES_ON && h->exec_mode == FIRE_EXEC_GRAPH_WHILE &&
-           h->body_iters == 0 && !(h->par.dmax > 0.0);
-}
-
-// Neighbour geometry for a box.  The list radius is rc + skin, with the skin
-// reduced where a periodic axis is shorter than 2 (rc + skin) so that the
-// minimum image stays unique within the list radius.
-GeoC make_geo(const fire_handle* h, const double box[3]) {
-    GeoC g{};
+// Radius of the neighbour lists in a box: rc + skin, with the skin reduced where
+// a periodic axis is shorter than 2 (rc + skin) so that the minimum image stays
+// unique within the list radius.
+double list_skin(const fire_handle* h, const double box[3]) {
     const double rc = cutoff(h->pot);
     double skin = h->pot.skin;
     for (int a = 0; a < 3; ++a)
         if (h->sys.periodic[a]) skin = std::min(skin, 0.5 * box[a] * (1.0 - 1e-12) - rc);
-    skin = std::max(skin, 0.0);
-    const double rl = rc + skin;
+    return std::max(skin, 0.0);
+}
+
+// Whether relaxations and evaluations run in the resident loop (fire2_loop.cuh):
+// the default settings of the FP64 table form and LJ, one system, up to kLoopAtoms
+// atoms and kLoopEntries list entries.  What the caller has chosen (newton,
+// threads per atom, tiles, chunked or sized graph bodies, a displacement cap)
+// keeps the kernel chain.  The loop saves the chain's launches, some 45 us per
+// iteration, and pays for them with a full list, every pair from both ends.  us
+// per iteration chain / loop:
+//   RGL, 5.0 A (53 entries per atom): 48,667 atoms 84.5 / 70.5, 62,499 98 / 77
+//   RGL, 7.2 A (150): 54,000 atoms 204 / 194, 65,000 (9.7 M entries) 217 / 205
+//   RGL, 10 A (388): 15,900 atoms 168 / 160, 31,680 (12.3 M) 302 / 304, 48,000
+//     (18.6 M) 402 / 505 -- in between a shell at the cut-off or between it and
+//     the list radius moves the line by a third (6.5 A, 54,000 atoms, 6.0 M:
+//     150 / 160)
+//   LJ, whose pair terms are FP64 arithmetic: 2.5 sigma (92) 10,975 atoms 80 / 53;
+//     4.0 (333) 6,911 atoms (2.3 M) 133 / 131, 10,975 (3.7 M) 188 / 192; 5.0 (624)
+//     1,371 atoms 65 / 68, 13,499 379 / 434
+constexpr int kLoopAtoms = 65536, kLoopAtomsLj = 16384;
+constexpr double kLoopEntries = 10e6, kLoopEntriesLj = 3.5e6, kLoopListLj = 400.0;
+bool loop_wanted(const fire_handle* h, const double box[3]) {
+    const bool lj = h->pot.kind == FIRE_POT_LJ;
+    const bool form = lj || (fixed64_form(h->pot) && h->pot.newton == FIRE_NEWTON_AUTO);
+    if (!form || h->loop_ok == 0 || h->neb || h->batch || h->img_n != h->n || h->tpa_set ||
+        h->n > (lj ? kLoopAtomsLj : kLoopAtoms) || h->tile_mode == FIRE_TILES_ON ||
+        h->exec_mode != FIRE_EXEC_GRAPH_WHILE || h->body_iters != 0 || h->par.dmax > 0.0)
+        return false;
+    // expected list at the mean density
+    const double rl = cutoff(h->pot) + list_skin(h, box);
+    const double list = std::min(h->n - 1.0, 4.0 / 3.0 * M_PI * rl * rl * rl * h->n /
+                                                 (box[0] * box[1] * box[2]));
+    return h->n * list <= (lj ? kLoopEntriesLj : kLoopEntries) && !(lj && list > kLoopListLj);
+}
+
+// Neighbour geometry for a box.
+GeoC make_geo(const fire_handle* h, const double box[3]) {
+    GeoC g{};
+    const double rc = cutoff(h->pot);
+    const double skin = list_skin(h, box), rl = rc + skin;
     g.rlist2 = rl * rl;
     g.half_skin2 = 0.25 * skin * skin;
     g.rc2f = (float)(rc * rc);
@@ -1066,7 +1086,7 @@ fire_status prepare_call(fire_handle* h, const double box[3], GeoC* g, bool neb_
     fire_status st = check_box(h, box);
     if (st != FIRE_OK) return st;
     CK(h, cudaSetDevice(h->device));
-    h->loop = relax && loop_wanted(h);
+    h->loop = relax && loop_wanted(h, box);
     *g = make_geo(h, box);
     const int cap = std::max(estimate_cap(h, *g), h->cap);
     return ensure_buffers(h, *g, cap);
