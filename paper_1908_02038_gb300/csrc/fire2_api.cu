@@ -269,6 +269,11 @@ bool loop_wanted(const fire_handle* h, const double box[3]) {
     return h->n * list <= (lj ? kLoopEntriesLj : kLoopEntries) && !(lj && list > kLoopListLj);
 }
 
+// Cells of all images together, 4 GB of counts, starts and extents: a cluster in an
+// open box of more than 512 cells per axis, nearly all of them empty, gets larger
+// ones (their number is 32-bit, and the scan goes over all).
+constexpr double kMaxCells = 134217728.0;
+
 // Neighbour geometry for a box.
 GeoC make_geo(const fire_handle* h, const double box[3]) {
     GeoC g{};
@@ -284,8 +289,13 @@ GeoC make_geo(const fire_handle* h, const double box[3]) {
         g.per[a] = h->sys.periodic[a] ? 1 : 0;
         // a periodic axis needs 3 cells for a stencil without repeats; an
         // open axis takes any count (at least one), its cells clamped
-        g.nc[a] = std::max((int)std::floor(box[a] / rl), g.per[a] ? 0 : 1);
+        g.nc[a] = std::max((int)std::min(std::floor(box[a] / rl), kMaxCells), g.per[a] ? 0 : 1);
         if (g.per[a] && g.nc[a] < 3) g.brute = 1;
+    }
+    const double images = h->img_n > 0 ? (double)(h->n / h->img_n) : 1.0;
+    while (!g.brute && images * g.nc[0] * g.nc[1] * g.nc[2] > kMaxCells) {
+        int& most = *std::max_element(g.nc, g.nc + 3);
+        most = (most + 1) / 2;   // from more than 3
     }
     if (g.brute)
         for (int a = 0; a < 3; ++a) g.nc[a] = 1;

@@ -342,7 +342,8 @@ __global__ void k_cell_fill(Bufs b, GeoC g, int force) {
 // build reads its candidates from consecutive addresses.
 __global__ void __launch_bounds__(kElemBlock) k_cell_sort(Bufs b, GeoC g, int force) {
     if (!need_rebuild(b.st, g, force)) return;
-    const int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    // (a thread index over all cells would not fit 32 bits)
+    const int c = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
     if (c >= b.ncell) return;
     const int k0 = b.cell_start[c], m = b.cell_start[c + 1] - k0;
     int* a = b.cell_atoms + k0;
