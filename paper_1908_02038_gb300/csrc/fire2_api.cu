@@ -370,9 +370,12 @@ int tile_grid(const fire_handle* h, const GeoC& g) {
     return std::max(1, std::min(std::min(g.ntile, kTileMinBlocks * h->sms), nb_max));
 }
 
+// (An array is counted as allocated once it is: where cudaMalloc fails, the next
+// call finds a count of 0 and allocates again.)
 fire_status ensure_buffers(fire_handle* h, const GeoC& g, int cap) {
     if (cap > h->cap) {
         drop_graph(h);
+        h->cap = 0;
         cudaFree(h->b.nbr);
         cudaFree(h->b.crep);
         cudaFree(h->b.cden);
@@ -391,6 +394,7 @@ fire_status ensure_buffers(fire_handle* h, const GeoC& g, int cap) {
     const int ncell = (h->n / g.img_n) * g.ncell_img;
     if (ncell > h->ncell_alloc) {
         drop_graph(h);
+        h->ncell_alloc = 0;
         cudaFree(h->b.cell_count);
         cudaFree(h->b.cell_start);
         cudaFree(h->b.cell_box);
@@ -1887,22 +1891,24 @@ static fire_status grad_setup(fire_handle* h, const double* d_pos, const double 
     GradState& gs = h->grad;
     const int n = h->n;
     const int cap = std::min(std::max(n - 1, 1), 2 * estimate_cap(h, make_geo(h, box)) + 16);
-    if (!gs.x) {
+    if (!gs.st) {   // the last of them
         gs.nb = ceil_div(n, kForceBlock);
-        CK(h, cudaMalloc(&gs.x, (size_t)n * sizeof(dvec4)));
-        CK(h, cudaMalloc(&gs.xf, (size_t)n * sizeof(float4)));
-        CK(h, cudaMalloc(&gs.nnbr, (size_t)n * sizeof(int)));
+        auto get = [](auto** p, size_t bytes) { return *p ? cudaSuccess : cudaMalloc(p, bytes); };
+        CK(h, get(&gs.x, (size_t)n * sizeof(dvec4)));
+        CK(h, get(&gs.xf, (size_t)n * sizeof(float4)));
+        CK(h, get(&gs.nnbr, (size_t)n * sizeof(int)));
         for (double** p : {&gs.rho, &gs.F1, &gs.F2, &gs.drho, &gs.dq})
-            CK(h, cudaMalloc(p, (size_t)n * sizeof(double)));
+            CK(h, get(p, (size_t)n * sizeof(double)));
         // 9 rows of nb, or 4 of the cached HVP's blocks
-        CK(h, cudaMalloc(&gs.part, (size_t)std::max(9 * gs.nb, 4 * hvp_grid(n, kMaxHvpTpa)) * sizeof(double)));
-        CK(h, cudaMalloc(&gs.vec, (size_t)4 * n * sizeof(dvec4)));
-        CK(h, cudaMallocHost(&gs.h_part, (size_t)9 * gs.nb * sizeof(double)));
-        CK(h, cudaMalloc(&gs.st, sizeof(DevState)));
+        CK(h, get(&gs.part, (size_t)std::max(9 * gs.nb, 4 * hvp_grid(n, kMaxHvpTpa)) * sizeof(double)));
+        CK(h, get(&gs.vec, (size_t)4 * n * sizeof(dvec4)));
+        if (!gs.h_part) CK(h, cudaMallocHost(&gs.h_part, (size_t)9 * gs.nb * sizeof(double)));
+        CK(h, get(&gs.st, sizeof(DevState)));
     }
     if (cap > gs.cap) {
         cudaFree(gs.nbr);
         gs.nbr = nullptr;
+        gs.cap = 0;
         CK(h, cudaMalloc(&gs.nbr, (size_t)cap * n * sizeof(uint32_t)));
         gs.cap = cap;
     }
@@ -2140,10 +2146,8 @@ fire_status fire_rgl_implicit_grad_dev(fire_handle_t* h, const double* d_pos, co
     // the iterations run on device scalars (CgState): the host queues
     // kCgBatch of them at a time and reads the state once per batch; the
     // kernels of iterations after the stop return at once
-    if (!gs.cs) {
-        CK(h, cudaMalloc(&gs.cs, sizeof(CgState)));
-        CK(h, cudaMallocHost(&gs.h_cs, sizeof(CgState)));
-    }
+    if (!gs.cs) CK(h, cudaMalloc(&gs.cs, sizeof(CgState)));
+    if (!gs.h_cs) CK(h, cudaMallocHost(&gs.h_cs, sizeof(CgState)));
     CgState c0{};
     c0.rr = rr;
     c0.stop2 = tol * tol * rr;

@@ -956,6 +956,7 @@ static fire_status batch_geometry(fire_handle_t* h, fire_batch_state* b, const d
     if (slots > b->list_slots) {
         cudaFree(b->args.nbr);
         b->args.nbr = nullptr;
+        b->list_slots = 0;
         BCK(cudaMalloc(&b->args.nbr, (size_t)slots * sizeof(uint32_t)));
         b->list_slots = slots;
     }
