@@ -1168,7 +1168,10 @@ static bool fill_potc(fire_handle* h) {
         c.sw_sigma = pot->sigma;
         c.sw_rc = pot->sw_a * pot->sigma;
         c.rc2 = c.sw_rc * c.sw_rc;
-        c.sw_tmax = 600.0 / (pot->sigma * std::max(1.0, pot->sw_gamma));
+        // |1 / (r - a sigma)| where the pair's and the triplets' exponentials are
+        // e^-600, each by its own argument (finite also for a gamma near 0)
+        c.sw_tmax = 600.0 / pot->sigma;
+        c.sw_tmax3 = std::min(600.0 / (pot->sigma * pot->sw_gamma), 1e150);
         c.sw_A = pot->sw_A;
         c.sw_B = pot->sw_B;
         c.sw_p = pot->sw_p;

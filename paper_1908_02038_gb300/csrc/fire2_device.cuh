@@ -984,12 +984,15 @@ __global__ void __launch_bounds__(kSwBlock) k_force_sw(Bufs b, PotC P, GeoC g) {
             if (!below_nonneg(r2, P.rc2)) continue;
             const double invr = rsqrt_f64(r2);   // r2 > 0: list pairs are distinct atoms
             const double r = r2 * invr;
-            // t = 1 / (r - a sigma) < 0, no further than where the exponentials
-            // are e^-600 (exp_tang's range; exactly at the cut-off t = -sw_tmax)
-            const double t = -min_nonneg(rcp_f64(abs_bits(r - P.sw_rc)), P.sw_tmax);
+            // t = 1 / (r - a sigma) < 0, for each exponential no further than where
+            // it is e^-600 (exp_tang's range; infinite exactly at the cut-off)
+            const double tabs = rcp_f64(abs_bits(r - P.sw_rc));
+            const double t = -min_nonneg(tabs, P.sw_tmax);
             const double x1 = s * t, sr = s * invr;
             const double bp = P.sw_B * sw_pow(sr, P.sw_p, P.sw_pi), bq = sw_pow(sr, P.sw_q, P.sw_qi);
-            const double aex = ae * exp_tang(x1, P.ex, etab), d = bp - bq;
+            // nothing beyond (a library exponential underflows there too)
+            const double aex = below_nonneg(P.sw_tmax, tabs) ? 0.0 : ae * exp_tang(x1, P.ex, etab);
+            const double d = bp - bq;
             e_i = fma(0.5 * aex, d, e_i);
             // force on i from the pair: phi2'(r) d / r
             const double w = aex * fma(-d, x1 * t, (P.sw_q * bq - P.sw_p * bp) * invr) * invr;
@@ -997,14 +1000,14 @@ __global__ void __launch_bounds__(kSwBlock) k_force_sw(Bufs b, PotC P, GeoC g) {
             fy += w * dy;
             fz += w * dz;
             if (cnt < kSwMax) {
-                const double x2 = gs * t;
+                const double t3 = -min_nonneg(tabs, P.sw_tmax3), x2 = gs * t3;
                 nj[cnt] = j;
                 ux[cnt] = dx * invr;
                 uy[cnt] = dy * invr;
                 uz[cnt] = dz * invr;
                 ir[cnt] = invr;
-                eg[cnt] = exp_tang(x2, P.ex, etab);
-                gd[cnt] = x2 * t;
+                eg[cnt] = below_nonneg(P.sw_tmax3, tabs) ? 0.0 : exp_tang(x2, P.ex, etab);
+                gd[cnt] = x2 * t3;
                 S[cnt] = C[cnt] = Vx[cnt] = Vy[cnt] = Vz[cnt] = 0.0;
             }
             ++cnt;
