@@ -91,10 +91,13 @@ __device__ __forceinline__ double na_exp(const NaPot& P, double x, const double*
     return FAST ? fire2::exp_tang(x, P.ex, tab) : exp(x);
 }
 
-// r and 1/r of a pair.
+// r and 1/r of a pair.  The exponentials multiply r's error by up to p r / r0, so
+// r2 / sqrt(r2) gets its residual put back, which rounds it as sqrt does: forces
+// of 3,960 Cu atoms off by 2.15e-15 as with the IEEE operations, 2.71e-15 without.
 __device__ __forceinline__ void na_radius(double r2, double& r, double& rinv) {
     rinv = fire2::rsqrt_f64(r2);
-    r = __double_as_longlong(r2) > 0 ? r2 * rinv : 0.0;
+    const double s = r2 * rinv;
+    r = __double_as_longlong(r2) > 0 ? fma(fma(-s, s, r2), 0.5 * rinv, s) : 0.0;
 }
 
 // RGL pair terms: phi = A e^{-p s} S, g = xi^2 e^{-2q s} S, s = r/r0 - 1, with
