@@ -314,7 +314,7 @@ GeoC make_geo(const fire_handle* h, const double box[3]) {
               (fixed64_form(h->pot) && !fixed64_half(h->pot)) || h->loop) ? 1 : 0;
     for (int a = 0; a < 3; ++a) {
         g.Lq[a] = (int)(unsigned)(unsigned long long)std::llrint(box[a] * h->b.qscale);
-        g.Lq64[a] = std::llrint(std::ldexp(box[a], kFixedBits64));
+        g.Lq64[a] = std::llrint(std::ldexp(box[a], h->potc.fbits));
     }
     g.img_n = h->img_n > 0 ? h->img_n : h->n;
     // bricks of cells: the tiles of the FP64 half-list passes (fire2_tile.cuh);
@@ -1198,6 +1198,9 @@ static bool fill_potc(fire_handle* h) {
     c.rc2 = pot->rc * pot->rc;
     c.r0sq = pot->r0 * pot->r0;
     c.rc2_f = (float)c.rc2;
+    c.fbits = h->b.fbits = fixed_bits(pot->rc);
+    c.lam = std::exp2(kFixedBits64 - c.fbits);
+    c.lam2 = c.lam * c.lam;
     c.A = pot->A;
     c.xi2 = pot->xi * pot->xi;
     c.xi_inv = 1.0 / pot->xi;
@@ -1245,7 +1248,7 @@ static fire_status upload_tables(fire_handle* h) {
     const RglTables T32 = t32 ? build_rgl_tables(p.A, p.xi, p.p, p.q, p.r0, p.rs, p.rc) : RglTables{};
     h->potc.tab32 = T32.meta;
     std::vector<float> ffd, fff;
-    h->potc.ff = build_ff_tables(p.A, p.xi, p.p, p.q, p.r0, p.rs, p.rc, ffd, fff);
+    h->potc.ff = build_ff_tables(p.A, p.xi, p.p, p.q, p.r0, p.rs, p.rc, h->potc.lam, ffd, fff);
     const size_t nff = ffd.size();
     const size_t nd32 = T32.dens32.size(), nf32 = T32.force32.size();
     if (!h->tab_ffd) {
@@ -2227,15 +2230,15 @@ fire_status fire_diag_rgl_table(const fire_potential_t* pot, int64_t n, const do
         !(pot->rc > pot->rs && pot->rs > 0.0 && pot->r0 > 0.0 && pot->xi > 0.0))
         return FIRE_ERR_ARG;
     std::vector<float> ffd, fff;
-    const FFTab T = build_ff_tables(pot->A, pot->xi, pot->p, pot->q, pot->r0, pot->rs, pot->rc, ffd,
-                                    fff);
-    const float rc2_f = (float)(pot->rc * pot->rc);
+    const double lam = std::exp2(kFixedBits64 - fixed_bits(pot->rc));
+    const FFTab T = build_ff_tables(pot->A, pot->xi, pot->p, pot->q, pot->r0, pot->rs, pot->rc, lam,
+                                    ffd, fff);
     for (int64_t i = 0; i < n; ++i) {
         double* o = out + 4 * i;
         // the FP64 kernels' arithmetic from r^2 on (r^2 as a float pair)
-        const ffloat r2 = f64_to_ff(r[i] * r[i]);
+        const ffloat r2 = f64_to_ff(r[i] * r[i] / (lam * lam));
         const bool rows = ff_in_rows(T, r2.hi);
-        if (!rows && !(r2.hi < rc2_f)) {
+        if (!rows && !(r2.hi < T.rc2)) {
             o[0] = o[1] = o[2] = o[3] = 0.0;
         } else if (rows) {
             ffloat d[2], f[2];
@@ -2243,8 +2246,8 @@ fire_status fire_diag_rgl_table(const fire_potential_t* pot, int64_t n, const do
             ff_eval(fff, T, r2, f);
             o[0] = ff_to_f64(d[0]);                 // phi
             o[1] = ff_to_f64(d[1]);                 // g
-            o[2] = 0.5 * r[i] * ff_to_f64(f[0]);    // phi' = r (2 phi'/r) / 2
-            o[3] = r[i] * ff_to_f64(f[1]);          // g' = r (g'/r)
+            o[2] = 0.5 * r[i] / lam * ff_to_f64(f[0]);    // phi' = r (2 phi'/r) / 2
+            o[3] = r[i] / lam * ff_to_f64(f[1]);          // g' = r (g'/r)
         } else {
             double a[8];
             rgl_analytic(pot->A, pot->xi, pot->p, pot->q, pot->r0, pot->rs, pot->rc, r[i], a);

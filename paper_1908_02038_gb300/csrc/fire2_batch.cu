@@ -38,7 +38,7 @@ struct BInst {
     int nc[3];              // cells per axis; nc[0] == 0 -> all-pairs build
     int per[3];
     int Lq[3];              // box in fixed-point units (FP32-pair form)
-    long long Lq64[3];      // box in 2^-44 A units (FP64 table form)
+    long long Lq64[3];      // box in 2^-fbits A units (FP64 table form)
     double L[3], Linv[3];
     float Lf[3], Linvf[3];
     float rlist2f;
@@ -61,7 +61,7 @@ struct BArgs {
     dvec4 *x, *v, *f, *xref;
     int4* xq;
     float4* xf;
-    lvec4* xq64;            // FP64 table form: positions in 2^-44 A units
+    lvec4* xq64;            // FP64 table form: positions in 2^-fbits A units
     const float *tab_ffd, *tab_fff;   // FP64 table form: density / force rows
     int ff;                 // 1: FP64 table passes available (FP64 table form, or the
                             //    FP32-pair form confirming its stops)
@@ -273,7 +273,7 @@ __device__ __forceinline__ void b_shifts(const BInst& I, int* smem) {
 }
 
 // Separation x_j - x_i - shift of list entry e in the FP64 table form: exact
-// in 2^-44 A fixed point, split into float pairs.
+// in fixed point, split into float pairs.
 __device__ __forceinline__ ffvec b_sep_ff(const BShift& S, const lvec4& qi, const lvec4& qj,
                                           uint32_t e) {
     const int code = (int)(e >> kIdxBits);
@@ -339,13 +339,13 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
                 const lvec4 qj = a.xq64[I.off + (int)(e & kIdxMask)];
                 const ffloat r2 = ff_norm2(b_sep_ff(S, qi, qj, e));
                 const bool rows = ff_in_rows(P.ff, r2.hi);
-                if (!rows && !(r2.hi < P.rc2_f)) continue;
+                if (!rows && !(r2.hi < P.ff.rc2)) continue;
                 ffloat2 w;
                 if (rows) {
                     w = ff_eval2(a.tab_ffd, P.ff, r2);
                 } else {   // outside the rows: FP64 exponentials
                     double rinv, phi, dphi, g, dg;
-                    rgl_pair64(P, ff_to_f64(r2), etab, rinv, phi, dphi, g, dg);
+                    rgl_pair64(P, P.lam2 * ff_to_f64(r2), etab, rinv, phi, dphi, g, dg);
                     const ffloat p = f64_to_ff(phi), q = f64_to_ff(g);
                     w = {make_float2(p.hi, q.hi), make_float2(p.lo, q.lo)};
                 }
@@ -430,7 +430,7 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
                 const ffvec d = b_sep_ff(S, qi, qj, e);
                 const ffloat r2 = ff_norm2(d);
                 const bool rows = ff_in_rows(P.ff, r2.hi);
-                if (!rows && !(r2.hi < P.rc2_f)) continue;
+                if (!rows && !(r2.hi < P.ff.rc2)) continue;
                 ffloat c0, c1;
                 if (rows) {
                     const ffloat2 c = ff_eval2(a.tab_fff, P.ff, r2);
@@ -438,9 +438,9 @@ __device__ __forceinline__ double b_forces(const BArgs& a, const BInst& I, int l
                     c1 = ff_second(c);
                 } else {
                     double rinv, phi, dphi, g, dg;
-                    rgl_pair64(P, ff_to_f64(r2), etab, rinv, phi, dphi, g, dg);
-                    c0 = f64_to_ff(2.0 * dphi * rinv);
-                    c1 = f64_to_ff(dg * rinv);
+                    rgl_pair64(P, P.lam2 * ff_to_f64(r2), etab, rinv, phi, dphi, g, dg);
+                    c0 = f64_to_ff(2.0 * dphi * rinv * P.lam);
+                    c1 = f64_to_ff(dg * rinv * P.lam);
                 }
                 const ffloat fs = ff_madd(ff_add(fpi, fp_load(qj)), c1, c0);
                 const ffloat2 t = ff_mul2_neg(fs, d.xy);
@@ -551,8 +551,8 @@ __device__ __forceinline__ float b_update(const BArgs& a, const BInst& I, int lo
             a.xq[gi] = make_int4(to_fixed(x.x, a.qscale), to_fixed(x.y, a.qscale),
                                  to_fixed(x.z, a.qscale), 0);
         if (a.ff && (!F32 || fp64_phase))
-            a.xq64[gi] = {to_fixed64(x.x, kFixedBits64), to_fixed64(x.y, kFixedBits64),
-                          to_fixed64(x.z, kFixedBits64), 0ll};
+            a.xq64[gi] = {to_fixed64(x.x, a.P.fbits), to_fixed64(x.y, a.P.fbits),
+                          to_fixed64(x.z, a.P.fbits), 0ll};
         const float ddx = fx - f64_to_f32_trunc(r.x), ddy = fy - f64_to_f32_trunc(r.y),
                     ddz = fz - f64_to_f32_trunc(r.z);
         dmax = fmaxf(dmax, ddx * ddx + ddy * ddy + ddz * ddz);
@@ -728,8 +728,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_batch_relax(BArgs a) {
                 a.xq[gi] = make_int4(to_fixed(p[0], a.qscale), to_fixed(p[1], a.qscale),
                                      to_fixed(p[2], a.qscale), 0);
             else if (a.ff)
-                a.xq64[gi] = {to_fixed64(p[0], kFixedBits64), to_fixed64(p[1], kFixedBits64),
-                              to_fixed64(p[2], kFixedBits64), 0ll};
+                a.xq64[gi] = {to_fixed64(p[0], a.P.fbits), to_fixed64(p[1], a.P.fbits),
+                              to_fixed64(p[2], a.P.fbits), 0ll};
             a.v[gi] = make_dvec4(0.0, 0.0, 0.0, 0.0);
         }
         const double anybad = bmax((double)bad, red);
@@ -756,9 +756,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_batch_relax(BArgs a) {
                 // confirm the FP32-pair stop: FP64 forces at the same positions
                 for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
                     const dvec4 x = a.x[I.off + i];
-                    a.xq64[I.off + i] = {to_fixed64(x.x, kFixedBits64),
-                                         to_fixed64(x.y, kFixedBits64),
-                                         to_fixed64(x.z, kFixedBits64), 0ll};
+                    a.xq64[I.off + i] = {to_fixed64(x.x, a.P.fbits),
+                                         to_fixed64(x.y, a.P.fbits),
+                                         to_fixed64(x.z, a.P.fbits), 0ll};
                 }
                 if (CL) cg::this_cluster().sync();
                 else __syncthreads();
@@ -930,7 +930,7 @@ static fire_status batch_geometry(fire_handle_t* h, fire_batch_state* b, const d
             I.Linvf[k] = (float)(1.0 / L);
             I.per[k] = sys.periodic[k] ? 1 : 0;
             I.Lq[k] = (int)(unsigned)(unsigned long long)std::llrint(L * qscale);
-            I.Lq64[k] = std::llrint(std::ldexp(L, kFixedBits64));
+            I.Lq64[k] = std::llrint(std::ldexp(L, fire2_potc(h).fbits));
             // open axes take any cell count (clamped cells), periodic ones 3 or more
             I.nc[k] = std::max((int)std::floor(L / rl), I.per[k] ? 0 : 1);
             if (I.per[k] && I.nc[k] < 3) cells = false;

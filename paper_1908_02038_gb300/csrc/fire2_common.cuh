@@ -53,9 +53,10 @@ struct TabMeta {
 
 // Intervals of the FP64 form's pair tables (fire2_table.cuh): width h in r^2,
 // from row 0 = [j_lo h, (j_lo + 1) h); rs2 = rs^2.  The rows serve r2_lo = j_lo h
-// up to r2_hi: rc^2, or rs^2 where the taper is too narrow for them.
+// up to r2_hi: rc2 = rc^2, or rs^2 where the taper is too narrow for them.  All in
+// squares of the tables' unit of length (PotC::lam).
 struct FFTab {
-    float h, hinv, r2_lo, r2_hi, rs2;
+    float h, hinv, r2_lo, r2_hi, rs2, rc2;
     int j_lo, last;
 };
 
@@ -90,7 +91,9 @@ struct PotC {
     float qinv, qinv2;        // 1 / qscale, 1 / qscale^2
     double xi_inv;            // 1 / xi (theta-derivatives)
     double r0sq;              // r0^2 (table variable u = r^2 - r0^2)
-    float rc2_f;              // FP32 copy (cut-off test of the FP64 pass)
+    float rc2_f;              // FP32 copy (order of the batch's lists)
+    int fbits;                // fixed-point positions of the FP64 table form: 2^fbits per A
+    double lam, lam2;         // and the tables' unit of length, 2^(44 - fbits) A, its square
     FFTab ff;                 // intervals of the FP64 form's tables
     TabMeta tab32;            // knots of the FP32 tables
 };

@@ -42,7 +42,7 @@ struct GeoC {
     float rlist2f;         // (rc + skin + margin)^2, margin covers FP32 rounding
     int full;              // 1 = full list (both directions), 0 = half list
     int Lq[3];             // box lengths in fixed-point units, modulo 2^32
-    long long Lq64[3];     // box lengths in 2^-44 A units (FP64 form)
+    long long Lq64[3];     // box lengths in those of xq64 (FP64 form)
     // several images of one system in the same box (nudged elastic band):
     // atoms [k img_n, (k + 1) img_n) form image k and interact only among
     // themselves; one system: img_n = n
@@ -114,8 +114,9 @@ struct Bufs {
     const double* exp_table;  // 2^(j/256), j = 0..255
     // tabulated RGL pair functions (fire2_table.cuh); nullptr when analytic
     const float *tab_ffd, *tab_fff;   // FP64 form: density / force rows (kFFRow floats)
-    lvec4* xq64;               // FP64 form: positions in 2^-44 A units (x, y, z) and
+    lvec4* xq64;               // FP64 form: positions in 2^-fbits A units (x, y, z) and
                                //    F'(rho) as a float pair in w (fp_store / fp_load)
+    int fbits;                 // bits of that unit: 2^fbits per A (PotC)
     int pass_role;             // 0: always run; 1: FP32-pair pass that sits out the FP64
                                //    confirmation; 2: FP64 pass that runs only for it
     int nb_verify;             // blocks of the FP64 confirming passes
@@ -221,8 +222,8 @@ __global__ void k_prepare(Bufs b) {
         b.xq[i] = make_int4(to_fixed(p[0], b.qscale), to_fixed(p[1], b.qscale),
                             to_fixed(p[2], b.qscale), 0);
     if (b.xq64)
-        b.xq64[i] = {to_fixed64(p[0], kFixedBits64), to_fixed64(p[1], kFixedBits64),
-                     to_fixed64(p[2], kFixedBits64), 0ll};
+        b.xq64[i] = {to_fixed64(p[0], b.fbits), to_fixed64(p[1], b.fbits),
+                     to_fixed64(p[2], b.fbits), 0ll};
     b.v[i] = make_dvec4(0.0, 0.0, 0.0, 0.0);
     f_store(b, i, 0.0, 0.0, 0.0);
     if (b.rho) b.rho[i] = 0.0;
@@ -1416,14 +1417,14 @@ __device__ __forceinline__ void density_ff_body(const Bufs& b, const PotC& P, co
             if (k + TPA < m) e_nx = b.nbr[(size_t)(k + TPA) * b.n + i];
             const ffloat r2 = ff_norm2(pair_sep_ff(qt, qi, qj, e));
             const bool rows = ff_in_rows(P.ff, r2.hi);
-            if (!rows && !(r2.hi < P.rc2_f)) continue;
+            if (!rows && !(r2.hi < P.ff.rc2)) continue;
             ffloat2 v;   // phi (doubled at the end on the half list), g
             if (rows) {
                 v = ff_eval2(b.tab_ffd, P.ff, r2);
                 if (HALF) atomicAdd(&b.rho[j], ff_to_f64(ff_second(v)));
             } else {
                 double rinv, phi, dphi, gg, dg;
-                rgl_pair64(P, ff_to_f64(r2), etab, rinv, phi, dphi, gg, dg);
+                rgl_pair64(P, P.lam2 * ff_to_f64(r2), etab, rinv, phi, dphi, gg, dg);
                 const ffloat p = f64_to_ff(phi), q = f64_to_ff(gg);
                 v = {make_float2(p.hi, q.hi), make_float2(p.lo, q.lo)};
                 if (HALF) atomicAdd(&b.rho[j], gg);
@@ -1502,7 +1503,7 @@ __global__ void __launch_bounds__(BLK) k_force_ff(Bufs b, PotC P, GeoC g) {
         const ffvec d = pair_sep_ff(qt, qi, qj, e);
         const ffloat r2 = ff_norm2(d);
         const bool rows = ff_in_rows(P.ff, r2.hi);
-        if (!rows && !(r2.hi < P.rc2_f)) continue;
+        if (!rows && !(r2.hi < P.ff.rc2)) continue;
         ffloat c0, c1;
         if (rows) {
             const ffloat2 c = ff_eval2(b.tab_fff, P.ff, r2);
@@ -1510,9 +1511,9 @@ __global__ void __launch_bounds__(BLK) k_force_ff(Bufs b, PotC P, GeoC g) {
             c1 = ff_second(c);
         } else {
             double rinv, phi, dphi, gg, dg;
-            rgl_pair64(P, ff_to_f64(r2), etab, rinv, phi, dphi, gg, dg);
-            c0 = f64_to_ff(2.0 * dphi * rinv);
-            c1 = f64_to_ff(dg * rinv);
+            rgl_pair64(P, P.lam2 * ff_to_f64(r2), etab, rinv, phi, dphi, gg, dg);
+            c0 = f64_to_ff(2.0 * dphi * rinv * P.lam);
+            c1 = f64_to_ff(dg * rinv * P.lam);
         }
         const ffloat fs = ff_madd(ff_add(fpi, fp_load(qj)), c1, c0);
         // unnormalised products (x and y with the high part negated): the
@@ -1844,8 +1845,8 @@ __device__ __forceinline__ float update_range(const Bufs& b, const FireScal& s, 
             b.xq[i] = make_int4(to_fixed(x.x, b.qscale), to_fixed(x.y, b.qscale),
                                 to_fixed(x.z, b.qscale), 0);
         if (b.xq64)
-            b.xq64[i] = {to_fixed64(x.x, kFixedBits64), to_fixed64(x.y, kFixedBits64),
-                         to_fixed64(x.z, kFixedBits64), 0ll};
+            b.xq64[i] = {to_fixed64(x.x, b.fbits), to_fixed64(x.y, b.fbits),
+                         to_fixed64(x.z, b.fbits), 0ll};
         b.v[i] = v;
         if (b.accum) {
             f_store(b, i, 0.0, 0.0, 0.0);

@@ -133,13 +133,13 @@ __device__ __forceinline__ double loop_density(const Bufs& b, const PotC& P, con
             if (k + 2 * L < m) e_n2 = b.nbr[(size_t)(k + 2 * L) * b.n + i];
             const ffloat r2 = ff_norm2(pair_sep_ff(qt, qi, qj, en));
             const bool rows = ff_in_rows(P.ff, r2.hi);
-            if (!rows && !(r2.hi < P.rc2_f)) continue;
+            if (!rows && !(r2.hi < P.ff.rc2)) continue;
             ffloat2 v;
             if (rows) {
                 v = ff_eval2(b.tab_ffd, P.ff, r2);
             } else {
                 double rinv, phi, dphi, gg, dg;
-                rgl_pair64(P, ff_to_f64(r2), b.exp_table, rinv, phi, dphi, gg, dg);
+                rgl_pair64(P, P.lam2 * ff_to_f64(r2), b.exp_table, rinv, phi, dphi, gg, dg);
                 const ffloat p = f64_to_ff(phi), q = f64_to_ff(gg);
                 v = {make_float2(p.hi, q.hi), make_float2(p.lo, q.lo)};
             }
@@ -192,7 +192,7 @@ __device__ __forceinline__ void loop_force(const Bufs& b, const PotC& P, const l
             const ffvec d = pair_sep_ff(qt, qi, qj, en);
             const ffloat r2 = ff_norm2(d);
             const bool rows = ff_in_rows(P.ff, r2.hi);
-            if (!rows && !(r2.hi < P.rc2_f)) continue;
+            if (!rows && !(r2.hi < P.ff.rc2)) continue;
             ffloat c0, c1;
             if (rows) {
                 const ffloat2 c = ff_eval2(b.tab_fff, P.ff, r2);
@@ -200,9 +200,9 @@ __device__ __forceinline__ void loop_force(const Bufs& b, const PotC& P, const l
                 c1 = ff_second(c);
             } else {
                 double rinv, phi, dphi, gg, dg;
-                rgl_pair64(P, ff_to_f64(r2), b.exp_table, rinv, phi, dphi, gg, dg);
-                c0 = f64_to_ff(2.0 * dphi * rinv);
-                c1 = f64_to_ff(dg * rinv);
+                rgl_pair64(P, P.lam2 * ff_to_f64(r2), b.exp_table, rinv, phi, dphi, gg, dg);
+                c0 = f64_to_ff(2.0 * dphi * rinv * P.lam);
+                c1 = f64_to_ff(dg * rinv * P.lam);
             }
             const ffloat fs = ff_madd(ff_add(fpi, fp_load(qj)), c1, c0);
             const ffloat2 t = ff_mul2_neg(fs, d.xy);
@@ -360,8 +360,8 @@ __device__ __forceinline__ float loop_update(const Bufs& b, const FireScal& s, i
         v[share + a] = va.y;
         v[2 * share + a] = va.z;
         if (RGL)
-            b.xq64[i0 + a] = {to_fixed64(xa.x, kFixedBits64), to_fixed64(xa.y, kFixedBits64),
-                              to_fixed64(xa.z, kFixedBits64), 0ll};
+            b.xq64[i0 + a] = {to_fixed64(xa.x, b.fbits), to_fixed64(xa.y, b.fbits),
+                              to_fixed64(xa.z, b.fbits), 0ll};
         else
             b.x[i0 + a] = xa;
         const float dx = f64_to_f32_trunc(xa.x) - xr[a], dy = f64_to_f32_trunc(xa.y) - xr[share + a],

@@ -199,7 +199,7 @@ namespace fire2 {
 // FP64 instructions issue at 1/58 of the FP32 rate on this part, so the FP64
 // form's pair passes use no FP64 instruction per pair:
 //   * separations are exact: positions in 64-bit fixed point (2^44 units per
-//     A, i.e. a grid finer than the last bit of a double coordinate beyond
+//     A at cut-offs to 8 A, fixed_bits; i.e. a grid finer than the last bit of a double coordinate beyond
 //     ~2 A), differences in integers, then split exactly into two floats;
 //   * everything else is double-float arithmetic: each value is an
 //     unevaluated sum hi + lo of two floats (Dekker 1971; Knuth's TwoSum),
@@ -239,7 +239,17 @@ namespace fire2 {
 
 constexpr int kFFRow = 16;
 constexpr double kTaperRows = 8.0;   // intervals below which the taper is analytic
-constexpr int kFixedBits64 = 44;   // fixed-point positions of the FP64 form: 2^44 per A
+// Fixed-point positions of the FP64 form: 2^44 per A up to a cut-off of 8 A, and
+// half as many for every doubling beyond, so that a component of a pair in range
+// is below 2^47 units and splits exactly into two floats (fixed_to_ff).  The pair
+// passes take a unit for 2^-44 of a length and are none the wiser: the tables are
+// built for lengths in 8 A, 16 A, ... / 8, 2^44 units each.  (With 2^44 per A at any
+// cut-off, separations above 8 A were off by up to 2^-22 A: forces by 4e-8 at
+// r0 = 7.7, rc = 15, by 7e-7 at 25.6 and 50.)
+constexpr int kFixedBits64 = 44;
+inline int fixed_bits(double rc) {
+    return kFixedBits64 - std::max(0, (int)std::ceil(std::log2(rc / 8.0)));
+}
 
 
 __host__ __device__ __forceinline__ void dbl_words(double d, unsigned& hi, unsigned& lo) {
@@ -587,7 +597,7 @@ __device__ __forceinline__ ffloat ff_first(ffloat2 v) { return {v.hi.x, v.lo.x};
 __device__ __forceinline__ ffloat ff_second(ffloat2 v) { return {v.hi.y, v.lo.y}; }
 #endif  // __CUDACC__
 
-// Exact split of a 64-bit integer |n| < 2^47 times 2^-kFixedBits64 into a
+// Exact split of a 64-bit integer |n| <= 2^47 times 2^-kFixedBits64 into a
 // float pair (both parts exact: 24 + 23 bits).
 __host__ __device__ __forceinline__ ffloat fixed_to_ff(long long n) {
     const long long a = n >> 23;                          // floor(n / 2^23)
@@ -676,26 +686,29 @@ inline double ff_interval(double r0, double rs, double rc) {
 // middle, with its fifth-degree term replaced by the Chebyshev-economised
 // lower ones (x^5 -> (20 x^3 - 5 x) / 16 on [-1, 1]): relative error
 // (a h / 2)^5 / 1920 for a function of logarithmic slope a in r^2, 6e-15 for
-// the Cu phi near r0.
+// the Cu phi near r0.  lam: the unit of length of the rows (a power of two; exact).
 inline FFTab build_ff_tables(double A, double xi, double p, double q, double r0, double rs,
-                             double rc, std::vector<float>& dens, std::vector<float>& force) {
+                             double rc, double lam, std::vector<float>& dens,
+                             std::vector<float>& force) {
     const double h = ff_interval(r0, rs, rc);
     FFTab t;
-    t.h = (float)h;
-    t.hinv = (float)(1.0 / h);
+    const double u = 1.0 / (lam * lam);   // squares in the rows' unit
+    t.h = (float)(u * h);
+    t.hinv = (float)(1.0 / (u * h));
+    t.rc2 = (float)(u * rc * rc);
     const int j_rs = (int)std::floor(rs * rs / h), j_rc = (int)std::floor(rc * rc / h);
     // from r0 / 2 (beyond rc where that is); never below 81 h, which it is where
     // h is not limited by the number of rows: closer to 0 the functions, smooth in
     // r, are no polynomials in r^2
     t.j_lo = std::max(81, (int)std::min(std::floor(0.25 * r0 * r0 / h), j_rc + 1.0));
-    t.r2_lo = (float)(t.j_lo * h);
-    t.rs2 = (float)(rs * rs);
+    t.r2_lo = (float)(t.j_lo * u * h);
+    t.rs2 = (float)(u * rs * rs);
     // The taper is a quintic in (r - rs) / (rc - rs): economised over n intervals
     // it is off by about 6 / 512 n^-5 of the function, 4e-7 at 8; over fewer the
     // rows are soon useless (n = 1/2: off by more than the function), and such a
     // thin shell holds few pairs.  Pairs that round to rs^2 or just below go with the taper.
     const bool taper_rows = rc * rc - rs * rs >= kTaperRows * h;
-    t.r2_hi = taper_rows ? (float)(rc * rc) : std::nextafterf(t.rs2, 0.f);
+    t.r2_hi = taper_rows ? t.rc2 : std::nextafterf(t.rs2, 0.f);
     const int rows = std::max(j_rc - t.j_lo, 0) + 2;
     t.last = rows - 1;
     dens.assign((size_t)rows * kFFRow, 0.f);
@@ -703,7 +716,7 @@ inline FFTab build_ff_tables(double A, double xi, double p, double q, double r0,
     auto fill = [&](int row, const double fa[2][4], const double fb[2][4]) {
         for (int d = 0; d < 2; ++d)        // d = 0: f; d = 1: f_u, scaled for the force rows
             for (int k = 0; k < 2; ++k) {
-                const double scale = d == 0 ? 1.0 : (k == 0 ? 4.0 : 2.0);
+                const double scale = d == 0 ? 1.0 : (k == 0 ? 4.0 : 2.0) * lam;
                 const double* a = fa[k] + d;
                 const double* b = fb[k] + d;
                 double x[6];
@@ -713,7 +726,7 @@ inline FFTab build_ff_tables(double A, double xi, double p, double q, double r0,
                     for (int n = 4; n >= m; --n) x[n] += 0.5 * x[n + 1];
                 x[3] += 1.25 * 0.25 * x[5];          // 20/16 x^3 and -5/16 x of x^5
                 x[1] -= 0.3125 * 0.0625 * x[5];
-                const double s1 = 1.0 / h;           // powers of two: exact
+                const double s1 = 1.0 / (u * h);     // powers of two: exact
                 double sm = scale;
                 auto put = [&](int j, float v) {   // number j of polynomial k
                     const int e = 2 * j + k;

@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_density_tile(B
                 ffloat dx, dy, dz;
                 const ffloat r2 = tile_sep(qjx - qix, qjy - qiy, qjz - qiz, dx, dy, dz);
                 const bool rows = ff_in_rows(P.ff, r2.hi);
-                if (!rows && !(r2.hi < P.rc2_f)) continue;
+                if (!rows && !(r2.hi < P.ff.rc2)) continue;
                 ffloat v[2];
                 if (rows) {
                     const ffloat2 w = ff_eval2(b.tab_ffd, P.ff, r2);
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_density_tile(B
                     v[1] = ff_second(w);
                 } else {
                     double rinv, phi, dphi, gg, dg;
-                    rgl_pair64(P, ff_to_f64(r2), b.exp_table, rinv, phi, dphi, gg, dg);
+                    rgl_pair64(P, P.lam2 * ff_to_f64(r2), b.exp_table, rinv, phi, dphi, gg, dg);
                     v[0] = f64_to_ff(phi);
                     v[1] = f64_to_ff(gg);
                 }
@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_force_tile(Buf
                 ffloat dx, dy, dz;
                 const ffloat r2 = tile_sep(qjx - qix, qjy - qiy, qjz - qiz, dx, dy, dz);
                 const bool rows = ff_in_rows(P.ff, r2.hi);
-                if (!rows && !(r2.hi < P.rc2_f)) continue;
+                if (!rows && !(r2.hi < P.ff.rc2)) continue;
                 ffloat c[2];
                 if (rows) {
                     const ffloat2 w = ff_eval2(b.tab_fff, P.ff, r2);
@@ -470,9 +470,9 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_force_tile(Buf
                     c[1] = ff_second(w);
                 } else {
                     double rinv, phi, dphi, gg, dg;
-                    rgl_pair64(P, ff_to_f64(r2), b.exp_table, rinv, phi, dphi, gg, dg);
-                    c[0] = f64_to_ff(2.0 * dphi * rinv);
-                    c[1] = f64_to_ff(dg * rinv);
+                    rgl_pair64(P, P.lam2 * ff_to_f64(r2), b.exp_table, rinv, phi, dphi, gg, dg);
+                    c[0] = f64_to_ff(2.0 * dphi * rinv * P.lam);
+                    c[1] = f64_to_ff(dg * rinv * P.lam);
                 }
                 const ffloat fs = ff_madd(ff_add(fpi, {fpj2.x, fpj2.y}), c[1], c[0]);
                 // normalised products, as fx_split_pair assumes
