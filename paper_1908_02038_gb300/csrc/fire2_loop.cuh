@@ -76,11 +76,12 @@ __device__ __forceinline__ bool loop_barrier(DevState* st, unsigned& target, Loo
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u64 [%0], %1;"
                      :: "l"(&st->bar), "l"(1ull + (mine ? 1ull << 32 : 0ull)) : "memory");
+        const unsigned goal = target + (wait_ns == 0ull ? 1u : 0u);   // one more never comes
         unsigned long long t0 = 0ull, v;
         int ok = 1;
         for (int n = 0;; ++n) {
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&st->bar) : "memory");
-            if ((int)((unsigned)v - target) >= 0 && wait_ns != 0ull) break;
+            if ((int)((unsigned)v - goal) >= 0) break;
             if ((n & 255) != 255) continue;
             const unsigned long long t = globaltimer_ns();
             if (t0 == 0ull) t0 = t;
@@ -387,7 +388,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_loop(Bufs b, PotC P, GeoC g, LoopC 
         sh.fs = st->fs;
         sh.stop = 0;
         sh.status = st->status;
-        sh.ok = *(volatile unsigned*)&st->bar_abort == 0u;
+        sh.ok = st->bar_abort == 0u ? 1 : 0;
     }
     if (RGL)
         fill_qshift64_table(qt, g);
