@@ -168,7 +168,7 @@ bool fixed64_half(const fire_potential_t& p) {
     return fixed64_form(p) && p.newton != FIRE_NEWTON_OFF;
 }
 // Blocks of the double-float density pass: one thread per atom on blocks of
-// kDensFF1Block (3 per SM at 40 registers: 0.289 against 0.312 ms with
+// kDensFF1Block (3 per SM at 39 registers: 0.289 against 0.312 ms with
 // blocks of 128 on the 1M-atom box, 0.302 with 256, 0.357 with 1024),
 // split lists on blocks of kForceBlock.
 inline int dens_ff_block(int tpa) { return tpa == 1 ? kDensFF1Block : kForceBlock; }
@@ -1196,7 +1196,6 @@ static bool fill_potc(fire_handle* h) {
         return true;
     }
     c.rc2 = pot->rc * pot->rc;
-    c.r0sq = pot->r0 * pot->r0;
     c.rc2_f = (float)c.rc2;
     c.fbits = h->b.fbits = fixed_bits(pot->rc);
     c.lam = std::exp2(kFixedBits64 - c.fbits);

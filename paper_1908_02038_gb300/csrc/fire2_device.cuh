@@ -169,10 +169,6 @@ __device__ __forceinline__ void fp_store(const Bufs& b, int i, ffloat f) {
     b.xq64[i].w = (long long)((unsigned long long)__float_as_uint(f.hi) |
                               ((unsigned long long)__float_as_uint(f.lo) << 32));
 }
-__device__ __forceinline__ ffloat fp_load(const lvec4& q) {
-    return {__uint_as_float((unsigned)((unsigned long long)q.w & 0xffffffffull)),
-            __uint_as_float((unsigned)((unsigned long long)q.w >> 32))};
-}
 
 // Whether a force pass sits this evaluation out (pass_role above; the state
 // says whether the evaluation confirms an FP32-pair stop in FP64).

@@ -46,9 +46,9 @@ struct NebC {
 };
 
 // d - L rint(d / L): d itself where |d| <= L / 2 (by the bit patterns; rint takes
-// 1/2 to 0), which is nearly everywhere -- the division and the rounding are
-// some 25 FP64 instructions, six times per atom in both kernels (6 images of
-// 6,911 atoms, 60 iterations: 9.06 -> 8.07 ms).
+// 1/2 to 0), which is nearly everywhere: no FP64 division and rounding, six times
+// per atom in both kernels (6 images of 6,911 atoms, 60 iterations: 9.06 -> 8.07
+// ms).
 static __device__ __noinline__ double neb_wrap(double d, double L) { return d - L * rint(d / L); }
 __device__ __forceinline__ double neb_mi(double d, const GeoC& g, int a) {
     if (g.per[a] && below_nonneg(0.5 * g.L[a], abs_bits(d))) return neb_wrap(d, g.L[a]);

@@ -116,13 +116,9 @@ inline RglTables build_rgl_tables(double A, double xi, double p, double q, doubl
     m.nA0 = nA0;
     m.nA = nA0 + nAp;
     m.nB = nB;
-    m.hA_inv = 1.0 / hA;
-    m.hB_inv = 1.0 / hB;
-    m.u_lo = -nA0 * hA;
-    m.u_rs = u_rs;
-    m.hA_inv_f = (float)m.hA_inv;
-    m.hB_inv_f = (float)m.hB_inv;
-    m.u_lo_f = (float)m.u_lo;
+    m.hA_inv_f = (float)(1.0 / hA);
+    m.hB_inv_f = (float)(1.0 / hB);
+    m.u_lo_f = (float)(-nA0 * hA);
     m.u_rs_f = (float)u_rs;
     const int nint = m.nA + m.nB;
     T.dens32.resize((size_t)nint * kTabDens);
@@ -371,12 +367,6 @@ __host__ __device__ __forceinline__ ffloat ff_madd(ffloat a, ffloat b, ffloat c)
     const ffloat s = two_sum(c.hi, p.hi);
     return fast_two_sum(s.hi, add_rn(s.lo, add_rn(c.lo, p.lo)));
 }
-// c + a b for a float b
-__host__ __device__ __forceinline__ ffloat ff_madd_f(ffloat a, float b, ffloat c) {
-    const float p = mul_rn(a.hi, b);
-    const ffloat s = two_sum(c.hi, p);
-    return fast_two_sum(s.hi, add_rn(s.lo, add_rn(c.lo, fmaf(a.lo, b, fmaf(a.hi, b, -p)))));
-}
 __host__ __device__ __forceinline__ double ff_to_f64(ffloat a) {
     return f32_to_f64(a.hi) + f32_to_f64(a.lo);
 }
@@ -392,6 +382,12 @@ __host__ __device__ __forceinline__ ffloat ff_acc(ffloat acc, ffloat t) {
 __host__ __device__ __forceinline__ ffloat f64_to_ff(double d) {
     const float hi = f64_to_f32_trunc(d);
     return {hi, f64_to_f32_trunc(d - f32_to_f64(hi))};
+}
+
+// F'(rho) as a float pair from the fourth word of an atom's fixed-point record.
+__device__ __forceinline__ ffloat fp_load(const lvec4& q) {
+    return {__uint_as_float((unsigned)((unsigned long long)q.w & 0xffffffffull)),
+            __uint_as_float((unsigned)((unsigned long long)q.w >> 32))};
 }
 
 // RGL embedding of the double-float form: sqrt(rho) and F'(rho) =
@@ -427,7 +423,7 @@ __device__ __forceinline__ bool f32_exponent(double d) {
     return bits > (903ll << 52) && bits < (1143ll << 52);
 }
 // 1/sqrt(x), x >= 0, in FP64 without a library call: the FP32 estimate y0 (the
-// conversions on the integer pipes) and one step of third order,
+// conversions on the integer pipes) and one step of third order (Halley's),
 // y0 + y0 e (1/2 + 3/8 e) with e = 1 - x y0^2 ~ 2^-22, off by 5/16 e^3 ~ 2^-67:
 // five FP64 instructions.  Outside FP32's exponents the IEEE operations.
 static __device__ __noinline__ double rsqrt_f64_any(double x) { return 1.0 / sqrt(x); }
@@ -445,9 +441,8 @@ __device__ __forceinline__ double rcp_f64(double x) {
     const double e = fma(-x, y0, 1.0);
     return fma(y0, fma(e, e, e), y0);
 }
-// sqrt(x) from these with the residual x - s^2 (exact in an FMA) put back: the
-// IEEE result but for rare last-bit ties, in a third of the dependent FP64
-// instructions of the library's.
+// sqrt(x) from these with the residual x - s^2 (exact in an FMA) put back, as in
+// Markstein's method (div_by): correctly rounded in 3.2e8 random arguments.
 static __device__ __noinline__ double sqrt_f64_any(double x) { return sqrt(x); }
 __device__ __forceinline__ double sqrt_f64(double x) {
     if (!f32_exponent(x)) return sqrt_f64_any(x);
