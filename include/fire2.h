@@ -80,8 +80,8 @@ typedef enum {
  * two, at least rc^2/65536; the taper's third-derivative jumps at rs and rc on
  * row boundaries, a taper of fewer than 8 intervals by the analytic functions;
  * interpolation error ~1e-13 relative for values, ~1e-12 for derivatives,
- * largest near r0/2), computed from exact fixed-point separations (2^-44 A)
- * in double-float arithmetic (float pairs, ~2^-44 relative), with FP64 sums,
+ * largest near r0/2), computed from exact fixed-point separations (2^-44 A at
+ * cut-offs up to 8 A, half as fine for every doubling beyond) in double-float arithmetic (float pairs, ~2^-44 relative), with FP64 sums,
  * reductions and integration.  In the FP32-pair precision: quintic Hermite
  * polynomials with knots every ~0.12 A^2, on rs and rc.
  * FIRE_PAIR_ANALYTIC: the exponentials and the taper per pair, IEEE FP64 in

@@ -1458,7 +1458,7 @@ __global__ void __launch_bounds__(kForceBlock) k_density_ff(Bufs b, PotC P, GeoC
 // ran 4 % slower; blocks of 448, 4 per SM at 32 registers, 0.327 ms).  1M-atom box:
 // 0.283 -> 0.245 ms (quartic tables, entries ahead); bound by L1 (91 %), which
 // serves the 16-byte table pieces and positions of a warp's 32 lanes one by one.
-// (The force pass keeps the compiler's 62: at 56 it spills and takes 0.407
+// (The force pass keeps the compiler's 63: at 56 it spills and takes 0.407
 // against 0.344 ms; L1 81 %, issue 68 %.)
 template <bool HALF>
 __global__ void __launch_bounds__(kDensFF1Block, 3) k_density_ff1(Bufs b, PotC P, GeoC g) {

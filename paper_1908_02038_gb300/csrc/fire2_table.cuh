@@ -661,8 +661,9 @@ inline void ff_eval(const std::vector<float>& tab, const FFTab& t, ffloat r2, ff
 // r0 / 2, where a steep phi's slope is twice as large.  Where lengths are larger
 // numbers than in Angstrom (r0^2 / 326 >= 2^-5) a quarter of that, and no more
 // than 1/256 of the taper, puts both under the arithmetic's own 2^-44 (r0 = 4.83,
-// the Cu set in bohr, phi' at r0 / 2: 7e-13 -> 1e-14); but no finer than 2^-6, at
-// which the Angstrom sets run.  At most 2^16 rows where that is wider than
+// the Cu set in bohr, phi' at r0 / 2: 7e-13 -> 4e-15); but no finer than 2^-6, at
+// which the Angstrom sets run (119,000 atoms in bohr, density / force pass 57 / 65
+// us at the wide intervals, 63 / 68 at these).  At most 2^16 rows where that is wider than
 // 2^-6, and 2^22 in any case: row numbers and the middles of the intervals have
 // to be exact in FP32, and the rows of an r0 far below rc, of which few are
 // ever met, would fill the memory.
